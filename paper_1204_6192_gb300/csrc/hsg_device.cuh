@@ -355,6 +355,27 @@ __device__ __forceinline__ void store_chunks(unsigned char* p, long long plane_s
     *reinterpret_cast<C*>(p + pl * plane_stride) = c[pl];
 }
 
+// The chunks of one site at a 32-bit byte offset from its plane's and chunk group's
+// base, plane_stride bytes between planes.
+template <int F, int POLICY>
+__device__ __forceinline__ void load_chunks_at(const unsigned char* base, long long plane_stride,
+                                               uint32_t off, typename FmtInfo<F>::Chunk* c) {
+  using C = typename FmtInfo<F>::Chunk;
+#pragma unroll
+  for (int pl = 0; pl < FmtInfo<F>::PLANES; ++pl) {
+    const C* q = reinterpret_cast<const C*>(base + pl * plane_stride + off);
+    c[pl] = POLICY == LD_RO ? __ldg(q) : (POLICY == LD_CG ? __ldcg(q) : *q);
+  }
+}
+template <int F>
+__device__ __forceinline__ void store_chunks_at(unsigned char* base, long long plane_stride,
+                                                uint32_t off, const typename FmtInfo<F>::Chunk* c) {
+  using C = typename FmtInfo<F>::Chunk;
+#pragma unroll
+  for (int pl = 0; pl < FmtInfo<F>::PLANES; ++pl)
+    *reinterpret_cast<C*>(base + pl * plane_stride + off) = c[pl];
+}
+
 // Decode one system (lane w of the site's plane data) from raw storage.
 template <int F>
 __device__ __forceinline__ void decode_one(const unsigned char* plane0, long long plane_stride,

@@ -20,10 +20,11 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
   const int4 blk = p.blocks[bidx];
   if (!p.active[blk.x]) return;   // a frozen sample (the whole block belongs to it)
   const SampleDev& sd = p.samples[blk.x];
-  const uint32_t h = (uint32_t)blk.z + threadIdx.x;
   const uint32_t half_n = (uint32_t)sd.N >> 1;
+  uint32_t h = (uint32_t)blk.z + threadIdx.x;
   bool active = h < half_n;
   if (!EN && !active) return;
+  if (EN) h = min(h, half_n - 1);   // idle threads of an energy sweep repeat the last site, unstored
   const int g0 = blk.y * p.GPT;
   const int g1 = min(p.G, g0 + p.GPT);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -32,40 +33,37 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
   float j6[6], h3[3];
   uint32_t jh[6];                                  // FP16 couplings, broadcast pairs
   constexpr bool MIXED = (F == FMT_F16) && J16;
+  // Chunk addresses: a block-uniform 64-bit base per component plane and chunk
+  // group, plus a site's 32-bit byte offset within a group, which stays the same
+  // over the loop.
   const unsigned char* base = p.spins + sd.spin_off;
   const long long ps = sd.plane_stride;
   const long long gstride = (long long)sd.N * FmtInfo<F>::CHUNK;
-  // Chunk addresses: group g of every plane starts at base + g * gstride, and a
-  // site's chunk lies ss * CHUNK bytes further.  The plain sweeps keep the 32-bit
-  // site indices and form each address per chunk group (fewer live registers:
-  // OR half-sweep 0.179 -> 0.174 ms at L = 128, FP16); the sweeps that also sum
-  // energies keep 64-bit offsets from group g0, which spill less there.
-  long long nb_off[6], own_off = 0;
-  if (active) {
-    gm = site_geom(sd, h, p.parity);
-    {
-      // HSG_CHECK builds: the site in this parity's half, its neighbours in the
-      // other half, the chunk groups within the sample (else skip the site)
-      const uint32_t own0 = (uint32_t)p.parity * half_n, nb0 = (uint32_t)(1 - p.parity) * half_n;
-      bool bad = HSG_OUT_OF_BOUNDS(gm.own >= own0 && gm.own < own0 + half_n && g1 <= p.G, p.bounds_err);
+  const uint32_t ob = (uint32_t)(1 - p.parity) * half_n;
+  gm = site_geom(sd, h, p.parity);
+  {
+    // HSG_CHECK builds: the site in this parity's half, its neighbours in the
+    // other half, the chunk groups within the sample (else skip the site)
+    const uint32_t own0 = (uint32_t)p.parity * half_n, nb0 = (uint32_t)(1 - p.parity) * half_n;
+    bool bad = HSG_OUT_OF_BOUNDS(gm.own >= own0 && gm.own < own0 + half_n && g1 <= p.G, p.bounds_err);
 #pragma unroll
-      for (int n = 0; n < 6; ++n)
-        bad = bad || HSG_OUT_OF_BOUNDS(gm.nb[n] >= nb0 && gm.nb[n] < nb0 + half_n, p.bounds_err);
-      if (bad) {
-        active = false;
-        if (!EN) return;
-      }
+    for (int n = 0; n < 6; ++n)
+      bad = bad || HSG_OUT_OF_BOUNDS(gm.nb[n] >= nb0 && gm.nb[n] < nb0 + half_n, p.bounds_err);
+    if (bad) {
+      active = false;
+      if (!EN) return;
+      gm.own = own0;
+#pragma unroll
+      for (int n = 0; n < 6; ++n) gm.nb[n] = nb0;
     }
   }
-  if (active) {
-    load_record<J16>(p.rec, sd.rec_off + gm.own, j6, h3);
-    if (MIXED) load_record_j16(p.rec, sd.rec_off + gm.own, jh);
-    if constexpr (EN) {
+  load_record<J16>(p.rec, sd.rec_off + gm.own, j6, h3);
+  if (MIXED) load_record_j16(p.rec, sd.rec_off + gm.own, jh);
+  uint32_t nb_off[6];
 #pragma unroll
-      for (int n = 0; n < 6; ++n) nb_off[n] = chunk_offset<F>(sd, g0, gm.nb[n]);
-      own_off = chunk_offset<F>(sd, g0, gm.own);
-    }
-  }
+  for (int n = 0; n < 6; ++n)
+    nb_off[n] = DEC ? (gm.nb[n] - ob) * 16u : gm.nb[n] * (uint32_t)FmtInfo<F>::CHUNK;
+  const uint32_t own_off = gm.own * (uint32_t)FmtInfo<F>::CHUNK;
   const uint32_t sweep =
       HB ? (uint32_t)((CG ? __ldcg(p.counters + 2 * blk.x) : p.counters[2 * blk.x]) +
                       (unsigned long long)p.sweep_offset)
@@ -73,37 +71,25 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
 
   // DEC: the decoded opposite parity, chunk (g, h') at dec + (g N/2 + h') 16 bytes
   const unsigned char* decb = DEC ? p.dec + sd.dec_off : nullptr;
-  const uint32_t ob = (uint32_t)(1 - p.parity) * half_n;
+  const long long dps = DEC ? sd.dec_plane_stride : 0;
 
   for (int g = g0; g < g1; ++g) {
     float e[VEC];
-#pragma unroll
-    for (int v = 0; v < VEC; ++v) e[v] = 0.0f;
-    if (active) {
+    {
       Chunk nc[DEC ? 1 : 6][PL];
       uint4 ncd[DEC ? 6 : 1][3];
-      unsigned char* own_p;
       if constexpr (DEC) {
-        const unsigned char* dg = decb + (long long)g * half_n * 16;
+        const unsigned char* dg = decb + (long long)g * (gstride / FmtInfo<F>::CHUNK / 2 * 16);
 #pragma unroll
-        for (int n = 0; n < 6; ++n)
-          load_chunks<FMT_F32, CG ? LD_CG : LD_RO>(dg + (size_t)(gm.nb[n] - ob) * 16, sd.dec_plane_stride, ncd[n]);
-        own_p = p.spins + sd.spin_off + (long long)g * gstride + (size_t)gm.own * FmtInfo<F>::CHUNK;
-      } else if constexpr (EN) {
-        const long long dg = (long long)(g - g0) * gstride;
-#pragma unroll
-        for (int n = 0; n < 6; ++n) load_chunks<F, CG ? LD_CG : LD_RO>(base + nb_off[n] + dg, ps, nc[n]);
-        // (the address of the own chunk after the neighbour loads: fewer live registers)
-        own_p = p.spins + sd.spin_off + own_off + dg;
+        for (int n = 0; n < 6; ++n) load_chunks_at<FMT_F32, CG ? LD_CG : LD_RO>(dg, dps, nb_off[n], ncd[n]);
       } else {
-        const unsigned char* base_g = base + (long long)g * gstride;
 #pragma unroll
         for (int n = 0; n < 6; ++n)
-          load_chunks<F, CG ? LD_CG : LD_RO>(base_g + (size_t)gm.nb[n] * FmtInfo<F>::CHUNK, ps, nc[n]);
-        own_p = p.spins + sd.spin_off + (long long)g * gstride + (size_t)gm.own * FmtInfo<F>::CHUNK;
+          load_chunks_at<F, CG ? LD_CG : LD_RO>(base + (long long)g * gstride, ps, nb_off[n], nc[n]);
       }
+      unsigned char* own_b = const_cast<unsigned char*>(base) + (long long)g * gstride;
       Chunk c[PL];
-      load_chunks<F, CG ? LD_CG : LD_PLAIN>(own_p, ps, c);
+      load_chunks_at<F, CG ? LD_CG : LD_PLAIN>(own_b, ps, own_off, c);
 
       // local field h = sum_n J_n s_n + H, in the order +x, -x, +y, -y, +z, -z
       Spins<VEC> hf;
@@ -183,7 +169,7 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
         for (int k = 0; k < VEC / 2; ++k) or_move2(s.x[k], s.y[k], s.z[k], hf.x[k], hf.y[k], hf.z[k]);
       }
       encode<F>(s, c);
-      store_chunks<F>(own_p, ps, c);
+      if (!EN || active) store_chunks_at<F>(own_b, ps, own_off, c);
 
       if (EN) {
         // energy of the new state from the stored values: every bond joins one
@@ -198,8 +184,8 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
           } else {
             d = dot3_2(st.x[k], st.y[k], st.z[k], f2(h3[0]), f2(h3[1]), f2(h3[2]));
           }
-          e[2 * k] = -d.x;
-          e[2 * k + 1] = -d.y;
+          e[2 * k] = active ? -d.x : 0.0f;
+          e[2 * k + 1] = active ? -d.y : 0.0f;
         }
       }
     }
