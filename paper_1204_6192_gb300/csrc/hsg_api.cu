@@ -58,6 +58,7 @@ struct hsg_ctx {
   double* d_epart = nullptr;        // energy partials [2][n_sweep_blocks][Wp]
   double* d_epart2 = nullptr;       // second level [n_samples][e_splits][Wp]
   int e_splits = 1;
+  unsigned int* d_tickets = nullptr;  // [n_samples]: arrivals of the energy sums' blocks
   float* d_beta = nullptr;
   double* d_temps = nullptr;
   double* d_inv_temps = nullptr;
@@ -265,6 +266,7 @@ EnergyParams energy_params(hsg_ctx* c) {
   p.blocks = c->d_sweep_blocks;
   p.partials = c->d_epart;
   p.partials2 = c->d_epart2;
+  p.tickets = c->d_tickets;
   p.active = c->d_active;
   p.splits = c->e_splits;
   p.E = c->d_E;
@@ -276,7 +278,7 @@ EnergyParams energy_params(hsg_ctx* c) {
   return p;
 }
 
-PTParams pt_params(hsg_ctx* c, int sweeps_per_call, int bump_pt) {
+PTParams pt_params(hsg_ctx* c, int sweeps_per_call) {
   PTParams p;
   p.E = c->d_E;
   p.inv_temps = c->d_inv_temps;
@@ -295,7 +297,6 @@ PTParams pt_params(hsg_ctx* c, int sweeps_per_call, int bump_pt) {
   p.seed_lo = c->seed_lo;
   p.seed_hi = c->seed_hi;
   p.sweeps_per_call = sweeps_per_call;
-  p.bump_pt = bump_pt;
   return p;
 }
 
@@ -382,9 +383,13 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
   return HSG_OK;
 }
 
-hsg_status enqueue_energy(hsg_ctx* c) {
+// The energies of the current state, and (pt) a PT pass with them, after which
+// the sweep counters advance by `sweeps`.
+hsg_status enqueue_energy(hsg_ctx* c, bool pt = false, int sweeps = 0) {
   EnergyParams p = energy_params(c);
-  HSG_CUDA(c, launch_energy(c->fmt, c->j16, p, c->stream));
+  HSG_CUDA(c, launch_energy_partials(c->fmt, c->j16, p, c->stream));
+  HSG_CUDA(c, pt ? launch_energy_sums_pt(p, pt_params(c, sweeps), c->stream)
+                 : launch_energy_sums(p, c->stream));
   return HSG_OK;
 }
 
@@ -541,10 +546,9 @@ hsg_status enqueue_step(hsg_ctx* c) {
     for (; k < nor; ++k) HSG_TRY(half_sweeps(c, false, nhb + k, k == nor - 1, b0, b1));
   }
   if (nor > 0) {
-    HSG_CUDA(c, launch_energy_final_pt(energy_params(c), pt_params(c, nhb + nor, 1), c->stream));
+    HSG_CUDA(c, launch_energy_sums_pt(energy_params(c), pt_params(c, nhb + nor), c->stream));
   } else {
-    HSG_TRY(enqueue_energy(c));
-    HSG_CUDA(c, launch_pt(pt_params(c, nhb + nor, 1), c->stream));
+    HSG_TRY(enqueue_energy(c, true, nhb + nor));
   }
   return HSG_OK;
 }
@@ -566,7 +570,7 @@ PersistParams persist_params(hsg_ctx* c, int n_steps) {
   PersistParams P;
   P.sw = sweep_params(c, 0, 0);
   P.en = energy_params(c);
-  P.pt = pt_params(c, 0, 1);
+  P.pt = pt_params(c, 0);
   P.bar = c->d_bar;
   P.timeout_ns = (unsigned long long)std::max(1, c->opt.barrier_timeout_ms) * 1000000ull;
   P.n_steps = n_steps;
@@ -743,7 +747,7 @@ hsg_status configure_schedule(hsg_ctx* c, int variant, int gpt, long long pass_b
       for (int h0 = 0; h0 < d.N / 2; h0 += SWEEP_BS) blocks.push_back(make_int4(s, gg, h0, 0));
     }
     d.blk1 = (int)blocks.size();
-    max_rows = std::max(max_rows, d.blk1 - d.blk0);
+    max_rows = std::max(max_rows, (d.N / 2 + SWEEP_BS - 1) / SWEEP_BS);
   }
   bounds.push_back((int)blocks.size());
   if ((long long)blocks.size() > c->max_sweep_blocks) return fail(c, HSG_ESTATE, "sweep table overflow");
@@ -754,7 +758,7 @@ hsg_status configure_schedule(hsg_ctx* c, int variant, int gpt, long long pass_b
   c->pass_bytes = pass_bytes;
   HSG_CUDA(c, cudaMemcpyAsync(c->d_pass_bound, bounds.data(), sizeof(int) * bounds.size(),
                               cudaMemcpyHostToDevice, c->stream));
-  // energy sums: about 16 block rows per first-level unit, at most MAX_E_SPLITS
+  // energy sums: about 16 block rows (of one chunk group) per first-level unit, at most MAX_E_SPLITS
   c->e_splits = std::min(MAX_E_SPLITS, std::max(1, max_rows / 16));
   HSG_CUDA(c, cudaMemcpyAsync(c->d_sweep_blocks, blocks.data(), sizeof(int4) * blocks.size(),
                               cudaMemcpyHostToDevice, c->stream));
@@ -1187,6 +1191,7 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
   HSG_ALLOC(c->d_conv_blocks, sizeof(int4) * conv_blocks.size());
   HSG_ALLOC(c->d_epart, sizeof(double) * 2 * max_sweep_blocks * Wp);
   HSG_ALLOC(c->d_epart2, sizeof(double) * n_samples * MAX_E_SPLITS * Wp);
+  HSG_ALLOC(c->d_tickets, sizeof(unsigned int) * n_samples);
   HSG_ALLOC(c->d_beta, sizeof(float) * n_samples * Wp);
   HSG_ALLOC(c->d_temps, sizeof(double) * n_samples * n_temps);
   HSG_ALLOC(c->d_inv_temps, sizeof(double) * n_samples * n_temps);
@@ -1256,6 +1261,7 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
   if (e == cudaSuccess) e = cudaMemset(c->d_moved, 0, sizeof(unsigned long long) * perm.size());
   if (e == cudaSuccess) e = cudaMemset(c->d_tunnel, 0, sizeof(unsigned int) * perm.size());
   if (e == cudaSuccess) e = cudaMemset(c->d_E, 0, sizeof(double) * n_samples * Wp);
+  if (e == cudaSuccess) e = cudaMemset(c->d_tickets, 0, sizeof(unsigned int) * n_samples);
   if (e == cudaSuccess) e = cudaMemset(c->d_bar, 0, sizeof(unsigned int) * 8);
   if (e == cudaSuccess) e = cudaMemset(c->spins, 0, c->spin_bytes);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
@@ -1355,9 +1361,8 @@ hsg_status hsg_pt_exchange(hsg_ctx* c) {
   NvtxRange nvtx_("hsg_pt_exchange");
   HSG_CHECK_CTX(c);
   HSG_CUDA(c, cudaSetDevice(c->device));
-  HSG_TRY(enqueue_energy(c));
+  HSG_TRY(enqueue_energy(c, true));
   c->e_valid = true;
-  HSG_CUDA(c, launch_pt(pt_params(c, 0, 1), c->stream));
   return HSG_OK;
 }
 
@@ -1369,7 +1374,7 @@ hsg_status hsg_pt_exchange_energies(hsg_ctx* c, const double* E_sys) {
   HSG_CUDA(c, cudaMemcpy2DAsync(c->d_E, sizeof(double) * c->Wp, E_sys, sizeof(double) * c->W,
                                 sizeof(double) * c->W, c->ns, cudaMemcpyHostToDevice, c->stream));
   c->e_valid = false;   // the caller's energies need not be those of the state
-  HSG_CUDA(c, launch_pt(pt_params(c, 0, 1), c->stream));
+  HSG_CUDA(c, launch_pt(pt_params(c, 0), c->stream));
   // the host array may be released by the caller on return
   HSG_CUDA(c, cudaStreamSynchronize(c->stream));
   HSG_TRY(poll_device_error(c));
@@ -1433,8 +1438,7 @@ hsg_status hsg_step_multihit(hsg_ctx* c, int n_steps, int tile, int n_rounds, in
       p.blk_base = color == 0 ? 0 : c->mh_count[ti][0];
       HSG_CUDA(c, launch_multihit(c->fmt, c->j16, fast, tile, p, c->mh_count[ti][color], c->stream));
     }
-    HSG_TRY(enqueue_energy(c));
-    HSG_CUDA(c, launch_pt(pt_params(c, n_rounds * (n_or + n_hb), 1), c->stream));
+    HSG_TRY(enqueue_energy(c, true, n_rounds * (n_or + n_hb)));
   }
   c->e_valid = true;
   return HSG_OK;

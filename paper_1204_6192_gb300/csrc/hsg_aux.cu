@@ -103,40 +103,211 @@ __global__ void __launch_bounds__(RED_BS) k_energy(const EnergyParams p) {
     }
   }
   __syncthreads();
-  for (int j = threadIdx.x; j < p.Wp; j += RED_BS) {
+  for (int jj = threadIdx.x; jj < (g1 - g0) * VEC; jj += RED_BS) {
     double ae = 0.0, ao = 0.0;
-    const int jj = j - g0 * VEC;
-    if (jj >= 0 && jj < (g1 - g0) * VEC) {
-      for (int w = 0; w < RED_BS / 32; ++w) {
-        ae += (double)esum_even[w * stride + jj];
-        ao += (double)esum_odd[w * stride + jj];
-      }
+    for (int w = 0; w < RED_BS / 32; ++w) {
+      ae += (double)esum_even[w * stride + jj];
+      ao += (double)esum_odd[w * stride + jj];
     }
+    const int j = g0 * VEC + jj;
     p.partials[(long long)blockIdx.x * p.Wp + j] = ae;
     p.partials[((long long)p.n_blocks + blockIdx.x) * p.Wp + j] = ao;
   }
 }
 
-// E[s][w] = sum over the sample's blocks of the even-site and odd-site partials,
-// in two fixed-order levels: split k of the sample's rows is added by a block
-// of 32 systems x 8 row lanes (coalesced rows of Wp doubles), then the splits.
-__global__ void __launch_bounds__(256) k_energy_final1(const EnergyParams p) {
+// ---------------------------------------------------------------------------
+// The tail of a step in one launch: the FP64 energy sums (SUM; Eq. 1) and the
+// parallel-tempering pass (PT; Eq. 4).  Block (split, wg, s) adds split `split` of
+// the systems 32 wg .. 32 wg + 31 of sample s (energy_rows); the last block of a
+// sample to finish (a ticket per sample) adds the splits and runs the sample's
+// chains, and advances its counters.
+//
+// The PT pass visits the pairs (k, k+1) from the lowest temperature up and an
+// accepted pair swaps the two configurations, so pair k compares the
+// configuration that slot k+1 held before the pass with one carried up from some
+// slot j <= k: slot k's own when pair k-1 was rejected.  Whatever j will be, its
+// decision depends only on the energies and the pair's uniform, so all
+// (j <= k) decisions are taken at once, one warp per pair and 32 values of j, each
+// exactly as the sequential walk would take it.  What is left of the sequential
+// walk is one bit test per pair.  (R_T = 32: the walk with its FP64 arithmetic and
+// exponentials in the chain took 18 us, this launch with the sums takes 5; measured
+// on L32_fp32.)
+// ---------------------------------------------------------------------------
+constexpr int TAIL_BS = 256;
+constexpr int TAIL_MASKS = 4096;      // decision words in shared memory: the chains run in batches
+constexpr int MAX_W = 1024, MAX_R_T = 256;   // limits of a context
+
+template <bool SUM, bool PT>
+__global__ void __launch_bounds__(TAIL_BS) k_energy_tail(const EnergyParams e, const PTParams p) {
   __shared__ double red[8][32];
-  energy_final1_unit<false>(p, blockIdx.z, blockIdx.y, blockIdx.x, red);
+  __shared__ double sE[PT ? MAX_W : 1], sib[PT ? MAX_R_T : 1];   // energies by memory slot; inverse temperatures
+  __shared__ int sperm[PT ? MAX_W : 1];         // the permutations before the pass
+  __shared__ float su[PT ? MAX_W : 1];          // the pairs' uniforms
+  __shared__ uint32_t mask[PT ? TAIL_MASKS : 1];   // [chain of the batch][pair][j / 32]
+  __shared__ uint16_t walk[PT ? MAX_W : 1];     // [chain][slot]: carried j, bit 15: pair accepted
+  __shared__ unsigned char sts[PT ? MAX_W : 1]; // tunnelling states
+  __shared__ bool s_last;
+  const int s = blockIdx.y, tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+  const unsigned char* active = SUM ? e.active : p.active;
+  const bool frozen = !active[s];
+  const int R = PT ? p.R_T : 1, R1 = R - 1, nw = (R + 31) / 32, W = PT ? p.R_O * R : 0;
+  const int c0 = PT ? s * p.R_O : 0;
+  if (PT)
+    for (int i = tid; i < R; i += TAIL_BS) sib[i] = p.inv_temps[(long long)s * R + i];
+  if (frozen) return;   // frozen sample (every block of it): energies, chains and counters stand
+  // the chains' state, on its way while the sums run
+  constexpr int PER = MAX_W / TAIL_BS;
+  int conf[PT ? PER : 1];
+  unsigned char ts[PT ? PER : 1];
+  uint32_t step = 0;
+  if constexpr (PT) {
+    step = (uint32_t)p.counters[2 * s + 1];     // the sample's PT passes key its uniforms
+#pragma unroll
+    for (int m = 0; m < PER; ++m) {
+      const int i = tid + m * TAIL_BS;
+      if (i < W) {
+        conf[m] = p.perm[(long long)c0 * R + i];
+        ts[m] = p.tstate[(long long)c0 * R + i];
+      }
+    }
+  }
+  if constexpr (SUM) {
+    const int wgs = (e.Wp + 31) / 32;
+    const int wg = blockIdx.x % wgs, split = blockIdx.x / wgs;
+    double* dst = e.splits == 1 ? e.E + (long long)s * e.Wp
+                                : e.partials2 + ((long long)s * e.splits + split) * e.Wp;
+    const int w = wg * 32 + tx;
+    const double t = energy_lanes(w < e.Wp ? energy_rows<false>(e, s, w, split, ty) : 0.0, tx, ty, red);
+    if (ty == 0 && w < e.Wp) {
+      dst[w] = t;
+      if (PT && gridDim.x == 1) sE[w] = t;
+    }
+    if (gridDim.x > 1) {
+      __threadfence();
+      __syncthreads();
+      if (tid == 0) s_last = atomicAdd(e.tickets + s, 1u) == gridDim.x - 1;
+      __syncthreads();
+      if (!s_last) return;
+      if (tid == 0) e.tickets[s] = 0u;
+      __threadfence();
+      for (int g = 0; g < wgs; ++g) {
+        const int v = g * 32 + tx;
+        double acc = 0.0;
+        if (v < e.Wp) {
+          const double* src = e.splits == 1 ? e.E + (long long)s * e.Wp : e.partials2 + (long long)s * e.splits * e.Wp;
+#pragma unroll 4
+          for (int k = ty; k < e.splits; k += 8) acc += __ldcg(src + (long long)k * e.Wp + v);
+        }
+        acc = energy_lanes(acc, tx, ty, red);
+        if (ty == 0 && v < e.Wp) {
+          if (e.splits > 1) e.E[(long long)s * e.Wp + v] = acc;
+          if (PT) sE[v] = acc;
+        }
+      }
+    }
+  } else if constexpr (PT) {
+    for (int i = tid; i < W; i += TAIL_BS) sE[i] = p.E[(long long)s * p.Wp + i];
+  }
+  if constexpr (PT) {
+#pragma unroll
+    for (int m = 0; m < PER; ++m) {
+      const int i = tid + m * TAIL_BS;
+      if (i < W) {
+        sperm[i] = conf[m];
+        sts[i] = ts[m];
+        if (R1 > 0)
+          su[i] = u01(philox4x32_10(make_uint4((uint32_t)(i % R), (uint32_t)(c0 + i / R), step, TAG_PT),
+                                    p.seed_lo, p.seed_hi).x);
+      }
+    }
+    __syncthreads();
+    const int batch = R1 > 0 ? TAIL_MASKS / (R1 * nw) : p.R_O;
+    for (int b0 = 0; b0 < p.R_O; b0 += batch) {
+      const int nb = min(batch, p.R_O - b0);
+      for (int i = ty; i < nb * R1 * nw; i += TAIL_BS / 32) {
+        const int jw = i % nw, ck = i / nw, k = ck % R1, at = (b0 + ck / R1) * R;
+        const int j = jw * 32 + tx;
+        bool acc = false;
+        if (j <= k) {
+          const double dbeta = sib[k + 1] - sib[k];
+          const double dE = sE[at + sperm[at + k + 1]] - sE[at + sperm[at + j]];
+          acc = pt_accept(dbeta * dE, su[at + k]);
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, acc);
+        if (tx == 0) mask[i] = m;
+      }
+      __syncthreads();
+      for (int c = tid; c < nb; c += TAIL_BS) {
+        uint16_t* wk = walk + (b0 + c) * R;
+        int j = 0;
+        if (nw == 1) {
+          const uint32_t* m = mask + c * R1;
+#pragma unroll 8
+          for (int k = 0; k < R1; ++k) {
+            const uint32_t acc = (m[k] >> j) & 1u;
+            wk[k] = (uint16_t)(j | (acc << 15));
+            j = acc ? j : k + 1;
+          }
+        } else {
+          for (int k = 0; k < R1; ++k) {
+            const uint32_t acc = (mask[(c * R1 + k) * nw + (j >> 5)] >> (j & 31)) & 1u;
+            wk[k] = (uint16_t)(j | (acc << 15));
+            j = acc ? j : k + 1;
+          }
+        }
+        wk[R1] = (uint16_t)j;
+      }
+      __syncthreads();
+    }
+    // the new permutations, inverse temperatures and diagnostics: the
+    // configuration that held slot k before the pass moved iff pair (k-1, k) moved
+    // it down or, failing that, pair (k, k+1) moved it up
+    auto holder = [&](int i) {   // configuration that holds slot i % R of chain i / R after the pass
+      const int v = walk[i];
+      return (v & 0x8000) ? sperm[i + 1] : sperm[i / R * R + v];
+    };
+    for (int i = tid; i < W; i += TAIL_BS) {
+      const int c = i / R, k = i - c * R;
+      const int cf = holder(i);
+      const bool acc = walk[i] & 0x8000, prev = k > 0 && (walk[i - 1] & 0x8000);
+      p.perm[(long long)c0 * R + i] = cf;
+      p.beta[(long long)s * p.Wp + c * R + cf] = (float)sib[k];
+      if (acc || prev) atomicAdd(p.moved + (long long)c0 * R + i, 1ull);
+      if (acc) atomicAdd(p.accepted + (long long)(c0 + c) * R1 + k, 1ull);
+    }
+    if (R > 1) {
+      // tunnelling: a configuration that reaches T_1 after T_R after T_1 closes a loop
+      for (int c = tid; c < p.R_O; c += TAIL_BS) {
+        const int bottom = holder(c * R), top = holder(c * R + R1);
+        unsigned char* out = p.tstate + (long long)(c0 + c) * R;
+        if (sts[c * R + bottom] == 2) atomicAdd(p.tunnel + (long long)(c0 + c) * R + bottom, 1u);
+        out[bottom] = 1;
+        if (sts[c * R + top] == 1) out[top] = 2;
+      }
+    }
+    if (tid == 0) {
+      atomicAdd(p.counters + 2 * s, (unsigned long long)p.sweeps_per_call);
+      atomicAdd(p.counters + 2 * s + 1, 1ull);
+    }
+  }
 }
 
-// one warp per system (8 per block)
-__global__ void k_energy_final2(const EnergyParams p) {
-  const int gw = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (gw >= p.n_samples * p.Wp) return;
-  energy_final2_warp<false>(p, gw / p.Wp, gw % p.Wp, threadIdx.x & 31);
+static dim3 tail_grid(const EnergyParams& e) {
+  return dim3(e.splits * ((e.Wp + 31) / 32), e.n_samples);
 }
 
-cudaError_t launch_energy_final(const EnergyParams& p, cudaStream_t st) {
-  k_energy_final1<<<dim3(p.splits, (p.Wp + 31) / 32, p.n_samples), 256, 0, st>>>(p);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_energy_final2<<<(p.n_samples * p.Wp + 7) / 8, 256, 0, st>>>(p);
+cudaError_t launch_energy_sums(const EnergyParams& e, cudaStream_t st) {
+  k_energy_tail<true, false><<<tail_grid(e), TAIL_BS, 0, st>>>(e, PTParams{});
+  return cudaGetLastError();
+}
+
+cudaError_t launch_energy_sums_pt(const EnergyParams& e, const PTParams& p, cudaStream_t st) {
+  k_energy_tail<true, true><<<tail_grid(e), TAIL_BS, 0, st>>>(e, p);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pt(const PTParams& p, cudaStream_t st) {
+  k_energy_tail<false, true><<<dim3(1, p.n_samples), TAIL_BS, 0, st>>>(EnergyParams{}, p);
   return cudaGetLastError();
 }
 
@@ -144,12 +315,10 @@ template <int F, bool J16>
 static cudaError_t energy_fmt(const EnergyParams& p, cudaStream_t st) {
   const size_t smem = sizeof(float) * 2 * (RED_BS / 32) * p.GPT * FmtInfo<F>::VEC;
   k_energy<F, J16><<<p.n_blocks, RED_BS, smem, st>>>(p);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_energy_final(p, st);
+  return cudaGetLastError();
 }
 
-cudaError_t launch_energy(int fmt, bool j16, const EnergyParams& p, cudaStream_t st) {
+cudaError_t launch_energy_partials(int fmt, bool j16, const EnergyParams& p, cudaStream_t st) {
   switch (fmt) {
     case FMT_F32: return j16 ? energy_fmt<FMT_F32, true>(p, st) : energy_fmt<FMT_F32, false>(p, st);
     case FMT_F16: return j16 ? energy_fmt<FMT_F16, true>(p, st) : energy_fmt<FMT_F16, false>(p, st);
@@ -159,100 +328,6 @@ cudaError_t launch_energy(int fmt, bool j16, const EnergyParams& p, cudaStream_t
     case FMT_YX4: return j16 ? energy_fmt<FMT_YX4, true>(p, st) : energy_fmt<FMT_YX4, false>(p, st);
   }
   return cudaErrorInvalidValue;
-}
-
-// ---------------------------------------------------------------------------
-// Parallel tempering, Eq. (4): one thread per (sample, replica) chain walks the
-// pairs (k, k+1) upwards from the lowest temperature; an accepted exchange
-// swaps the temperatures of the two configurations.  Runs as one block so that
-// the counters can be advanced after every chain is done.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_pt(const PTParams p) {
-  const int n_chains = p.n_samples * p.R_O;
-  for (int c = threadIdx.x; c < n_chains; c += blockDim.x) pt_chain<false>(p, c);
-  __syncthreads();
-  for (int s = threadIdx.x; s < p.n_samples; s += blockDim.x) {
-    if (!p.active[s]) continue;
-    p.counters[2 * s] += (unsigned long long)p.sweeps_per_call;
-    p.counters[2 * s + 1] += (unsigned long long)p.bump_pt;
-  }
-}
-
-cudaError_t launch_pt(const PTParams& p, cudaStream_t st) {
-  int n = p.n_samples * p.R_O;
-  int bs = n >= 1024 ? 1024 : ((n + 31) / 32) * 32;
-  k_pt<<<1, bs, 0, st>>>(p);
-  return cudaGetLastError();
-}
-
-// The last level of the FP64 energy sums (Eq. 1) and the PT pass (Eq. 4) in one
-// block, for steps with few systems: each warp sums the level-1 partials of its
-// systems (the same code and order as k_energy_final2), then, after a block
-// barrier, one thread per chain walks its pairs as k_pt does.  One launch
-// instead of two.  With `staged`, the permutations, energies and inverse
-// temperatures are first copied into shared memory (dynamic, laid out as
-// [samples][Wp] and [samples][R_T] doubles, then [chains][R_T] ints and the
-// chains' uniforms [chains][R_T - 1]): each pair of a chain reads its slot's
-// configuration and then that configuration's energy, two dependent loads that
-// now hit shared memory instead of L2, and the uniforms are drawn by all threads
-// at once instead of by each chain's thread.  The same arithmetic on the same
-// values, so the same decisions.
-__global__ void __launch_bounds__(1024) k_energy2_pt(const EnergyParams e, const PTParams p, int staged) {
-  extern __shared__ double pt_smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int gw = warp; gw < e.n_samples * e.Wp; gw += nw)
-    energy_final2_warp<false>(e, gw / e.Wp, gw % e.Wp, lane);
-  __syncthreads();
-  const int n_chains = p.n_samples * p.R_O;
-  if (staged) {
-    const int np = n_chains * p.R_T, ne = p.n_samples * p.Wp, nb = p.n_samples * p.R_T;
-    const int R1 = p.R_T > 1 ? p.R_T - 1 : 1, nu = n_chains * R1;
-    double* sE = pt_smem;
-    double* sib = sE + ne;
-    int* sperm = reinterpret_cast<int*>(sib + nb);
-    float* su = reinterpret_cast<float*>(sperm + np);
-    for (int i = threadIdx.x; i < ne; i += blockDim.x) sE[i] = p.E[i];
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) sib[i] = p.inv_temps[i];
-    for (int i = threadIdx.x; i < np; i += blockDim.x) sperm[i] = p.perm[i];
-    if (p.bump_pt)
-      for (int i = threadIdx.x; i < nu; i += blockDim.x) su[i] = pt_uniform(p, i / R1, i % R1);
-    __syncthreads();
-    for (int c = threadIdx.x; c < n_chains; c += blockDim.x) {
-      const int s = c / p.R_O, r = c - s * p.R_O;
-      pt_chain_on<false>(p, c, sperm + c * p.R_T, sE + s * p.Wp + r * p.R_T, sib + s * p.R_T,
-                         su + c * R1);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < np; i += blockDim.x) p.perm[i] = sperm[i];
-  } else {
-    for (int c = threadIdx.x; c < n_chains; c += blockDim.x) pt_chain<false>(p, c);
-  }
-  __syncthreads();
-  for (int s = threadIdx.x; s < p.n_samples; s += blockDim.x) {
-    if (!p.active[s]) continue;
-    p.counters[2 * s] += (unsigned long long)p.sweeps_per_call;
-    p.counters[2 * s + 1] += (unsigned long long)p.bump_pt;
-  }
-}
-
-bool energy_pt_folded(int n_samples, int Wp) { return (long long)n_samples * Wp <= ENERGY_PT_FOLD_SYSTEMS; }
-
-cudaError_t launch_energy_final_pt(const EnergyParams& e, const PTParams& p, cudaStream_t st) {
-  if (!energy_pt_folded(e.n_samples, e.Wp)) {
-    cudaError_t err = launch_energy_final(e, st);
-    if (err != cudaSuccess) return err;
-    return launch_pt(p, st);
-  }
-  k_energy_final1<<<dim3(e.splits, (e.Wp + 31) / 32, e.n_samples), 256, 0, st>>>(e);
-  cudaError_t err = cudaGetLastError();
-  if (err != cudaSuccess) return err;
-  // shared-memory copies of the chains (48 kB at most without an opt-in)
-  const size_t n_chains = (size_t)p.n_samples * p.R_O;
-  const size_t smem = sizeof(double) * ((size_t)p.n_samples * p.Wp + (size_t)p.n_samples * p.R_T) +
-                      sizeof(int) * n_chains * p.R_T + sizeof(float) * n_chains * std::max(1, p.R_T - 1);
-  const bool staged = smem <= 48 * 1024;
-  k_energy2_pt<<<1, 1024, staged ? smem : 0, st>>>(e, p, staged ? 1 : 0);
-  return cudaGetLastError();
 }
 
 __global__ void k_bump(unsigned long long* counters, const unsigned char* active, int n_samples,

@@ -27,8 +27,8 @@ namespace hsg {
 // spin storage formats (values of hsg_precision)
 enum Fmt { FMT_F32 = 0, FMT_F16 = 1, FMT_BF16 = 2, FMT_ANG16 = 3, FMT_OCT16 = 4, FMT_YX4 = 5 };
 
-constexpr int SWEEP_BS = 256;
-constexpr int MAX_E_SPLITS = 256;   // first-level units per sample of the energy sums     // threads per block, streaming sweep kernels
+constexpr int SWEEP_BS = 256;       // threads per block, streaming sweep kernels
+constexpr int MAX_E_SPLITS = 256;   // first-level units per sample of the energy sums
 constexpr int RED_BS = SWEEP_BS;  // energy kernel: same blocks as the sweep
 
 struct FastDivH {
@@ -60,7 +60,7 @@ struct SweepParams {
   uint32_t seed_lo, seed_hi;
   int parity;
   int sweep_offset;
-  double* epart;            // energy partials [2][n_blocks][Wp] (energy variant only)
+  double* epart;            // energy partials [2][n_blocks][Wp] (energy variant only; a block writes its own chunk groups' columns)
   int n_blocks;
   int blk_base;             // block table entry of launch block 0 (a pass's first block)
   int n_launch;             // blocks of this launch
@@ -94,6 +94,7 @@ struct EnergyParams {
   double* partials;         // [2][n_blocks][Wp]: even-site and odd-site terms per block
   double* partials2;        // [n_samples][splits][Wp]: second reduction level
   double* E;                // [n_samples][Wp]
+  unsigned int* tickets;    // [n_samples]: blocks of a sample that have added their split (0 between launches)
   const unsigned char* active;   // [n_samples]: frozen samples keep their energies
   int G, Wp, GPT, n_samples, n_blocks, splits;
 };
@@ -112,7 +113,6 @@ struct PTParams {
   int n_samples, R_O, R_T, Wp;
   uint32_t seed_lo, seed_hi;
   int sweeps_per_call;      // added to each active sample's sweep counter after the pass
-  int bump_pt;              // 1: this is a PT pass (each active sample's PT counter += 1)
 };
 
 
@@ -273,14 +273,11 @@ cudaError_t launch_half_sweep(int fmt, bool hb, bool j16, bool fast, bool energy
                               const SweepParams& p, int n_blocks, cudaStream_t st);
 cudaError_t launch_decode_parity(int fmt, const SweepParams& p, int parity, int n_blocks,
                                  cudaStream_t st);
-cudaError_t launch_energy(int fmt, bool j16, const EnergyParams& p, cudaStream_t st);
-cudaError_t launch_energy_final(const EnergyParams& p, cudaStream_t st);
+cudaError_t launch_energy_partials(int fmt, bool j16, const EnergyParams& p, cudaStream_t st);
+// the sums of the partials; the same and a PT pass; a PT pass with the energies in p.E
+cudaError_t launch_energy_sums(const EnergyParams& p, cudaStream_t st);
+cudaError_t launch_energy_sums_pt(const EnergyParams& e, const PTParams& p, cudaStream_t st);
 cudaError_t launch_pt(const PTParams& p, cudaStream_t st);
-// The energy sums' last level and the PT pass of a step: one launch after the
-// level-1 sums when samples x systems <= ENERGY_PT_FOLD_SYSTEMS, else two.
-constexpr long long ENERGY_PT_FOLD_SYSTEMS = 4096;
-bool energy_pt_folded(int n_samples, int Wp);
-cudaError_t launch_energy_final_pt(const EnergyParams& e, const PTParams& p, cudaStream_t st);
 // counters of the active samples += (sweeps, pts)
 cudaError_t launch_bump(unsigned long long* counters, const unsigned char* active, int n_samples,
                         int sweeps, int pts, cudaStream_t st);

@@ -198,51 +198,59 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
   if (EN) {
     __syncthreads();
     double* out = p.epart + ((long long)p.parity * p.n_blocks + bidx) * p.Wp;
-    for (int j = threadIdx.x; j < p.Wp; j += SWEEP_BS) {
+    for (int jj = threadIdx.x; jj < (g1 - g0) * VEC; jj += SWEEP_BS) {
       double acc = 0.0;
-      const int jj = j - g0 * VEC;
-      if (jj >= 0 && jj < (g1 - g0) * VEC) {
-        for (int w = 0; w < SWEEP_BS / 32; ++w) acc += (double)esum[w * p.GPT * VEC + jj];
-      }
-      out[j] = acc;
+      for (int w = 0; w < SWEEP_BS / 32; ++w) acc += (double)esum[w * p.GPT * VEC + jj];
+      out[g0 * VEC + jj] = acc;
     }
     __syncthreads();   // esum is reused by the next virtual block of this block
   }
 }
 
 // ---------------------------------------------------------------------------
-// FP64 energy sums.  Level 1: split `split` of the sample's block rows, systems
-// 32*wg .. 32*wg+31, on 256 threads = 32 systems x 8 row lanes.  Level 2: the
-// splits of one system.  Fixed order throughout.
+// FP64 energy sums.  Level 1: split `split` of the block rows that hold a
+// system's chunk group, systems 32*wg .. 32*wg+31, on 256 threads = 32 systems x
+// 8 row lanes.  Level 2: the splits of one system.  Fixed order throughout.  A
+// block of the sweep block table leaves partials only for the systems of its own
+// chunk groups, so a system's rows are those of its group.
 // ---------------------------------------------------------------------------
+template <bool CG>
+__device__ __forceinline__ double energy_rows(const EnergyParams& p, int s, int w, int split, int ty) {
+  const SampleDev& sd = p.samples[s];
+  const int rows = ((sd.N >> 1) + SWEEP_BS - 1) / SWEEP_BS;          // block rows of one chunk group
+  const int base = sd.blk0 + (w >> 2) / p.GPT * rows;
+  const int per = (rows + p.splits - 1) / p.splits;
+  const int r0 = base + split * per, r1 = base + min(split * per + per, rows);
+  double acc = 0.0;
+#pragma unroll 2
+  for (int r = r0 + ty; r < r1; r += 8) {
+    const double* a = p.partials + (long long)r * p.Wp + w;
+    const double* b = p.partials + ((long long)p.n_blocks + r) * p.Wp + w;
+    acc += CG ? __ldcg(a) : *a;
+    acc += CG ? __ldcg(b) : *b;
+  }
+  return acc;
+}
+
+// the eight row lanes of each system, in order (result in ty == 0)
+__device__ __forceinline__ double energy_lanes(double acc, int tx, int ty, double (*red)[32]) {
+  red[ty][tx] = acc;
+  __syncthreads();
+  double t = 0.0;
+  if (ty == 0)
+    for (int k = 0; k < 8; ++k) t += red[k][tx];
+  __syncthreads();
+  return t;
+}
+
 template <bool CG>
 __device__ __forceinline__ void energy_final1_unit(const EnergyParams& p, int s, int wg, int split,
                                                    double (*red)[32]) {
   if (!p.active[s]) return;   // frozen sample: its energies stand (block-uniform)
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int w = wg * 32 + tx;
-  const SampleDev& sd = p.samples[s];
-  const int nrows = sd.blk1 - sd.blk0;
-  const int per = (nrows + p.splits - 1) / p.splits;
-  const int r0 = sd.blk0 + split * per;
-  const int r1 = min(r0 + per, sd.blk1);
-  double acc = 0.0;
-  if (w < p.Wp) {
-    for (int r = r0 + ty; r < r1; r += 8) {
-      const double* a = p.partials + (long long)r * p.Wp + w;
-      const double* b = p.partials + ((long long)p.n_blocks + r) * p.Wp + w;
-      acc += CG ? __ldcg(a) : *a;
-      acc += CG ? __ldcg(b) : *b;
-    }
-  }
-  red[ty][tx] = acc;
-  __syncthreads();
-  if (ty == 0 && w < p.Wp) {
-    double t = 0.0;
-    for (int k = 0; k < 8; ++k) t += red[k][tx];
-    p.partials2[((long long)s * p.splits + split) * p.Wp + w] = t;
-  }
-  __syncthreads();
+  const double t = energy_lanes(w < p.Wp ? energy_rows<CG>(p, s, w, split, ty) : 0.0, tx, ty, red);
+  if (ty == 0 && w < p.Wp) p.partials2[((long long)s * p.splits + split) * p.Wp + w] = t;
 }
 
 // Level 2 for system w of sample s, one warp: lane j adds splits j, j + 32, ...
@@ -261,15 +269,17 @@ __device__ __forceinline__ void energy_final2_warp(const EnergyParams& p, int s,
 }
 
 // Metropolis decision of a PT pair (Eq. 4): accept iff x >= 0 or u < exp(x),
-// decided exactly as in binary64.  u >= 2^-24 > exp(-17), so x < -17 always
-// rejects.  Otherwise exp is evaluated in FP32 (expf: within 2 ulp; rounding
-// x to FP32 adds at most 17 * 2^-24 relative), and only a u within 4e-6
-// relative of it goes to the FP64 exp.  (GB300's FP64 rate is a small fraction
-// of its FP32 rate and this chain is sequential.)
+// decided exactly as in binary64.  xf is x rounded to FP32: where x < 0 rounds to
+// -0 its exp is above every uniform (u <= 1 - 2^-24), so xf >= 0 accepts as x does;
+// u >= 2^-24 > exp(-17), so xf < -17 always rejects.  Otherwise exp is evaluated
+// in FP32 (expf: within 2 ulp; rounding x to FP32 adds at most 17 * 2^-24
+// relative), and only a u within 4e-6 relative of it goes to the FP64 exp.
+// (GB300's FP64 rate is a small fraction of its FP32 rate.)
 __device__ __forceinline__ bool pt_accept(double x, float u) {
-  if (x >= 0.0) return true;
-  if (x < -17.0) return false;
-  const float e = expf((float)x);
+  const float xf = (float)x;
+  if (xf >= 0.0f) return true;
+  if (xf < -17.0f) return false;
+  const float e = expf(xf);
   if (u < e * (1.0f - 4e-6f)) return true;
   if (u > e * (1.0f + 4e-6f)) return false;
   return (double)u < exp(x);
@@ -282,25 +292,25 @@ __device__ __forceinline__ bool pt_accept(double x, float u) {
 // temperature random walk (Sec. 4): per slot, the passes after which the
 // configuration that held it has moved (p_diff = moved / passes), and per
 // configuration the closed loops T_1 -> T_R -> T_1 (tunnelling events).
-// The chain's permutation row, energies and inverse temperatures are read (and
-// the permutation written) through perm, E and ib: the global arrays, or copies
-// in shared memory (then CG is false and the caller writes perm back).  uf: the
-// chain's R_T - 1 uniforms, drawn beforehand (same counters), or null.
+// One thread walks the chain (the persistent step kernel; other passes run
+// k_energy_tail, which takes the same decisions in parallel).
 template <bool CG>
-__device__ __forceinline__ void pt_chain_on(const PTParams& p, int c, int* perm, const double* E,
-                                            const double* ib, const float* uf = nullptr) {
+__device__ __forceinline__ void pt_chain(const PTParams& p, int c) {
   const int s = c / p.R_O, r = c - s * p.R_O;
   if (!p.active[s]) return;
+  int* perm = p.perm + (long long)c * p.R_T;
+  const double* E = p.E + (long long)s * p.Wp + r * p.R_T;
+  const double* ib = p.inv_temps + (long long)s * p.R_T;
   // the sample's own PT pass counter keys its random numbers
   const uint32_t step = (uint32_t)(CG ? __ldcg(p.counters + 2 * s + 1) : p.counters[2 * s + 1]);
-  if (p.bump_pt) {
+  {
     unsigned long long* moved = p.moved + (long long)c * p.R_T;
     bool prev_acc = false;
     // the uniforms do not depend on the decisions: they are drawn 32 pairs at a
     // time ahead of the sequential chain, so the Philox evaluations overlap
     float uk[32];
     for (int k = 0; k + 1 < p.R_T; ++k) {
-      if (!uf && (k & 31) == 0) {
+      if ((k & 31) == 0) {
 #pragma unroll 4
         for (int j = 0; j < 32; ++j)
           uk[j] = (k + j + 1 < p.R_T)
@@ -312,7 +322,7 @@ __device__ __forceinline__ void pt_chain_on(const PTParams& p, int c, int* perm,
       const double dbeta = ib[k + 1] - ib[k];
       const double dE = (CG ? __ldcg(E + b) : E[b]) - (CG ? __ldcg(E + a) : E[a]);
       const double x = dbeta * dE;
-      const bool acc = pt_accept(x, uf ? uf[k] : uk[k & 31]);
+      const bool acc = pt_accept(x, uk[k & 31]);
       // the configuration that held slot k before the pass moved iff pair (k-1, k)
       // moved it down or, failing that, pair (k, k+1) moved it up
       if (acc || prev_acc) moved[k] += 1ull;
@@ -336,20 +346,6 @@ __device__ __forceinline__ void pt_chain_on(const PTParams& p, int c, int* perm,
   }
   float* beta = p.beta + (long long)s * p.Wp + r * p.R_T;
   for (int t = 0; t < p.R_T; ++t) beta[perm[t]] = (float)ib[t];
-}
-
-// The uniform of pair k of chain c in the current PT pass (as pt_chain_on draws it).
-__device__ __forceinline__ float pt_uniform(const PTParams& p, int c, int k) {
-  const int s = c / p.R_O;
-  const uint32_t step = (uint32_t)p.counters[2 * s + 1];
-  return u01(philox4x32_10(make_uint4((uint32_t)k, (uint32_t)c, step, TAG_PT), p.seed_lo, p.seed_hi).x);
-}
-
-template <bool CG>
-__device__ __forceinline__ void pt_chain(const PTParams& p, int c) {
-  const int s = c / p.R_O, r = c - s * p.R_O;
-  pt_chain_on<CG>(p, c, p.perm + (long long)c * p.R_T, p.E + (long long)s * p.Wp + r * p.R_T,
-                  p.inv_temps + (long long)s * p.R_T);
 }
 
 }  // namespace hsg

@@ -307,13 +307,10 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
   if constexpr (EN) {
     __syncthreads();
     double* out = p.epart + ((long long)par * p.n_blocks + bidx) * p.Wp;
-    for (int j = tid; j < p.Wp; j += SWEEP_BS) {
+    for (int jj = tid; jj < ng * VEC; jj += SWEEP_BS) {
       double acc = 0.0;
-      const int jj = j - g0 * VEC;
-      if (jj >= 0 && jj < ng * VEC) {
-        for (int w = 0; w < NW; ++w) acc += (double)esum[w * p.GPT * VEC + jj];
-      }
-      out[j] = acc;
+      for (int w = 0; w < NW; ++w) acc += (double)esum[w * p.GPT * VEC + jj];
+      out[g0 * VEC + jj] = acc;
     }
   }
   __syncthreads();   // the ring and its barriers are reused by nothing after this
