@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(RED_BS) k_energy(const EnergyParams p) {
   constexpr int VEC = FmtInfo<F>::VEC, PL = FmtInfo<F>::PLANES;
   using Chunk = typename FmtInfo<F>::Chunk;
   extern __shared__ float esum[];                 // [2][RED_BS / 32][GPT * VEC]
+  chain_trigger();
   const int4 blk = p.blocks[blockIdx.x];
   const SampleDev& sd = p.samples[blk.x];
   const uint32_t h = (uint32_t)blk.z + threadIdx.x;
@@ -47,6 +48,7 @@ __global__ void __launch_bounds__(RED_BS) k_energy(const EnergyParams p) {
     odd_off = chunk_offset<F>(sd, g0, gm.own);
     even_off = chunk_offset<F>(sd, g0, h);
   }
+  chain_wait();
   for (int g = g0; g < g1; ++g) {
     float eo[VEC], ee[VEC];
 #pragma unroll
@@ -55,9 +57,9 @@ __global__ void __launch_bounds__(RED_BS) k_energy(const EnergyParams p) {
       const long long dg = (long long)(g - g0) * gstride;
       Chunk nc[6][PL], co[PL], ce[PL];
 #pragma unroll
-      for (int n = 0; n < 6; ++n) load_chunks<F, LD_RO>(base + nb_off[n] + dg, ps, nc[n]);
-      load_chunks<F, LD_RO>(base + odd_off + dg, ps, co);
-      load_chunks<F, LD_RO>(base + even_off + dg, ps, ce);
+      for (int n = 0; n < 6; ++n) load_chunks<F, LD_PLAIN>(base + nb_off[n] + dg, ps, nc[n]);
+      load_chunks<F, LD_PLAIN>(base + odd_off + dg, ps, co);
+      load_chunks<F, LD_PLAIN>(base + even_off + dg, ps, ce);
       Spins<VEC> hf, t;
       decode<F>(nc[0], t);
 #pragma unroll
@@ -147,6 +149,7 @@ __global__ void __launch_bounds__(TAIL_BS) k_energy_tail(const EnergyParams e, c
   __shared__ uint16_t walk[PT ? MAX_W : 1];     // [chain][slot]: carried j, bit 15: pair accepted
   __shared__ unsigned char sts[PT ? MAX_W : 1]; // tunnelling states
   __shared__ bool s_last;
+  chain_trigger();
   const int s = blockIdx.y, tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   const unsigned char* active = SUM ? e.active : p.active;
   const bool frozen = !active[s];
@@ -154,6 +157,7 @@ __global__ void __launch_bounds__(TAIL_BS) k_energy_tail(const EnergyParams e, c
   const int c0 = PT ? s * p.R_O : 0;
   if (PT)
     for (int i = tid; i < R; i += TAIL_BS) sib[i] = p.inv_temps[(long long)s * R + i];
+  chain_wait();
   if (frozen) return;   // frozen sample (every block of it): energies, chains and counters stand
   // the chains' state, on its way while the sums run
   constexpr int PER = MAX_W / TAIL_BS;
@@ -297,25 +301,21 @@ static dim3 tail_grid(const EnergyParams& e) {
 }
 
 cudaError_t launch_energy_sums(const EnergyParams& e, cudaStream_t st) {
-  k_energy_tail<true, false><<<tail_grid(e), TAIL_BS, 0, st>>>(e, PTParams{});
-  return cudaGetLastError();
+  return launch_chained(k_energy_tail<true, false>, tail_grid(e), TAIL_BS, 0, st, e, PTParams{});
 }
 
 cudaError_t launch_energy_sums_pt(const EnergyParams& e, const PTParams& p, cudaStream_t st) {
-  k_energy_tail<true, true><<<tail_grid(e), TAIL_BS, 0, st>>>(e, p);
-  return cudaGetLastError();
+  return launch_chained(k_energy_tail<true, true>, tail_grid(e), TAIL_BS, 0, st, e, p);
 }
 
 cudaError_t launch_pt(const PTParams& p, cudaStream_t st) {
-  k_energy_tail<false, true><<<dim3(1, p.n_samples), TAIL_BS, 0, st>>>(EnergyParams{}, p);
-  return cudaGetLastError();
+  return launch_chained(k_energy_tail<false, true>, dim3(1, p.n_samples), TAIL_BS, 0, st, EnergyParams{}, p);
 }
 
 template <int F, bool J16>
 static cudaError_t energy_fmt(const EnergyParams& p, cudaStream_t st) {
   const size_t smem = sizeof(float) * 2 * (RED_BS / 32) * p.GPT * FmtInfo<F>::VEC;
-  k_energy<F, J16><<<p.n_blocks, RED_BS, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_chained(k_energy<F, J16>, p.n_blocks, RED_BS, smem, st, p);
 }
 
 cudaError_t launch_energy_partials(int fmt, bool j16, const EnergyParams& p, cudaStream_t st) {
@@ -332,6 +332,8 @@ cudaError_t launch_energy_partials(int fmt, bool j16, const EnergyParams& p, cud
 
 __global__ void k_bump(unsigned long long* counters, const unsigned char* active, int n_samples,
                        int sweeps, int pts) {
+  chain_trigger();
+  chain_wait();
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n_samples; s += gridDim.x * blockDim.x) {
     if (!active[s]) continue;
     counters[2 * s] += (unsigned long long)sweeps;
@@ -341,8 +343,7 @@ __global__ void k_bump(unsigned long long* counters, const unsigned char* active
 
 cudaError_t launch_bump(unsigned long long* counters, const unsigned char* active, int n_samples,
                         int sweeps, int pts, cudaStream_t st) {
-  k_bump<<<(n_samples + 255) / 256, 256, 0, st>>>(counters, active, n_samples, sweeps, pts);
-  return cudaGetLastError();
+  return launch_chained(k_bump, (n_samples + 255) / 256, 256, 0, st, counters, active, n_samples, sweeps, pts);
 }
 
 
@@ -411,9 +412,11 @@ __global__ void k_init(const ConvParams p) {
 template <int F>
 __global__ void k_get(const ConvParams p) {
   constexpr int VEC = FmtInfo<F>::VEC, PL = FmtInfo<F>::PLANES;
+  chain_trigger();
   const ConvItem it = conv_item(p);
-  if (!it.ok) return;
   const int sidx = p.blocks[blockIdx.x].x;
+  chain_wait();
+  if (!it.ok) return;
   const unsigned char* o = p.spins + it.sd->spin_off + chunk_offset<F>(*it.sd, it.g, it.ss);
   typename FmtInfo<F>::Chunk c[PL];
   load_chunks<F, LD_PLAIN>(o, it.sd->plane_stride, c);
@@ -501,7 +504,15 @@ cudaError_t launch_init(int fmt, const ConvParams& p, int nb, cudaStream_t st) {
   HSG_CONV_SWITCH(k_init)
 }
 cudaError_t launch_get(int fmt, const ConvParams& p, int nb, cudaStream_t st) {
-  HSG_CONV_SWITCH(k_get)
+  switch (fmt) {
+    case FMT_F32: return launch_chained(k_get<FMT_F32>, nb, 256, 0, st, p);
+    case FMT_F16: return launch_chained(k_get<FMT_F16>, nb, 256, 0, st, p);
+    case FMT_BF16: return launch_chained(k_get<FMT_BF16>, nb, 256, 0, st, p);
+    case FMT_ANG16: return launch_chained(k_get<FMT_ANG16>, nb, 256, 0, st, p);
+    case FMT_OCT16: return launch_chained(k_get<FMT_OCT16>, nb, 256, 0, st, p);
+    case FMT_YX4: return launch_chained(k_get<FMT_YX4>, nb, 256, 0, st, p);
+  }
+  return cudaErrorInvalidValue;
 }
 cudaError_t launch_set(int fmt, const ConvParams& p, int nb, cudaStream_t st) {
   HSG_CONV_SWITCH(k_set)

@@ -355,6 +355,16 @@ __device__ __forceinline__ void store_chunks(unsigned char* p, long long plane_s
     *reinterpret_cast<C*>(p + pl * plane_stride) = c[pl];
 }
 
+// Programmatic dependent launch.  A kernel launched by launch_chained
+// (hsg_internal.h) may start while the kernel before it in the stream still runs:
+// it reads only what no kernel writes (block table, geometry, couplings) before
+// chain_wait(), which returns when every kernel before it has completed and its
+// writes are visible.  Every block calls chain_wait() before it exits, so that a
+// kernel's completion implies that of all before it.  Data of earlier kernels are
+// read by plain loads after the wait, never by the read-only path.
+__device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // The chunks of one site at a 32-bit byte offset from its plane's and chunk group's
 // base, plane_stride bytes between planes.
 template <int F, int POLICY>

@@ -17,8 +17,14 @@ template <int F, bool HB, bool J16, bool FAST, bool EN, bool CG, bool DEC = fals
 __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, float* esum) {
   constexpr int VEC = FmtInfo<F>::VEC, PL = FmtInfo<F>::PLANES;
   using Chunk = typename FmtInfo<F>::Chunk;
+  // (CHAINED: a kernel of its own; the block's constants are read before the wait
+  // for the kernels before it)
+  constexpr bool CHAINED = !CG;
   const int4 blk = p.blocks[bidx];
-  if (!p.active[blk.x]) return;   // a frozen sample (the whole block belongs to it)
+  if (!p.active[blk.x]) {         // a frozen sample (the whole block belongs to it)
+    if (CHAINED) chain_wait();
+    return;
+  }
   const SampleDev& sd = p.samples[blk.x];
   const uint32_t half_n = (uint32_t)sd.N >> 1;
   uint32_t h = (uint32_t)blk.z + threadIdx.x;
@@ -64,6 +70,7 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
   for (int n = 0; n < 6; ++n)
     nb_off[n] = DEC ? (gm.nb[n] - ob) * 16u : gm.nb[n] * (uint32_t)FmtInfo<F>::CHUNK;
   const uint32_t own_off = gm.own * (uint32_t)FmtInfo<F>::CHUNK;
+  if (CHAINED) chain_wait();
   const uint32_t sweep =
       HB ? (uint32_t)((CG ? __ldcg(p.counters + 2 * blk.x) : p.counters[2 * blk.x]) +
                       (unsigned long long)p.sweep_offset)
@@ -81,11 +88,11 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
       if constexpr (DEC) {
         const unsigned char* dg = decb + (long long)g * (gstride / FmtInfo<F>::CHUNK / 2 * 16);
 #pragma unroll
-        for (int n = 0; n < 6; ++n) load_chunks_at<FMT_F32, CG ? LD_CG : LD_RO>(dg, dps, nb_off[n], ncd[n]);
+        for (int n = 0; n < 6; ++n) load_chunks_at<FMT_F32, CG ? LD_CG : LD_PLAIN>(dg, dps, nb_off[n], ncd[n]);
       } else {
 #pragma unroll
         for (int n = 0; n < 6; ++n)
-          load_chunks_at<F, CG ? LD_CG : LD_RO>(base + (long long)g * gstride, ps, nb_off[n], nc[n]);
+          load_chunks_at<F, CG ? LD_CG : LD_PLAIN>(base + (long long)g * gstride, ps, nb_off[n], nc[n]);
       }
       unsigned char* own_b = const_cast<unsigned char*>(base) + (long long)g * gstride;
       Chunk c[PL];

@@ -267,13 +267,17 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
   __shared__ uint64_t empty[MS_STAGES];  // every warp is done with a stage's buffer
   __shared__ float2 tw[512];             // (cos, sin)(2 pi x / L)
   __shared__ float red[NV][32];          // the block's sums per (value, slot of the round)
+  chain_trigger();
   const int s = blockIdx.z, round = blockIdx.y;
   // the sample's geometry in registers: the loop's barrier operations are
   // memory clobbers, which would otherwise reload it every site
   const SampleDev sd = p.samples[s];
   const uint32_t N = (uint32_t)sd.N, Nh = N >> 1;
   const uint32_t b0 = blockIdx.x * (uint32_t)p.tile_ss;
-  if (b0 >= N) return;
+  if (b0 >= N) {
+    chain_wait();
+    return;
+  }
   const uint32_t b1 = min(N, b0 + (uint32_t)p.tile_ss);
   const int sub = p.sub;
   const int n_sub = (int)((b1 - b0 + (uint32_t)sub - 1) / (uint32_t)sub);
@@ -294,6 +298,7 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
     sincospif(2.0f * (float)x / (float)L, &sn, &cs);
     tw[x] = make_float2(cs, sn);
   }
+  chain_wait();      // spins and permutations of the kernels before it from here on
   __syncthreads();
 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -462,6 +467,8 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
 // the total times 1/N.  Eight values per block of 256 threads.
 template <int MODE>
 __global__ void __launch_bounds__(256) k_meas_final_staged(const OverlapParams p, int NV) {
+  chain_trigger();
+  chain_wait();
   const int t = blockIdx.x % p.R_T, s = blockIdx.x / p.R_T;
   const int v = blockIdx.y * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (v >= NV) return;
@@ -506,11 +513,9 @@ static cudaError_t staged_launch(const OverlapParams& p, cudaStream_t st) {
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const dim3 grid(p.n_tiles, (p.R_T + 31) / 32, p.n_samples);
-  k_meas_staged<F, MODE, NR><<<grid, MEAS_BS, smem, st>>>(p);
-  e = cudaGetLastError();
+  e = launch_chained(k_meas_staged<F, MODE, NR>, grid, MEAS_BS, smem, st, p);
   if (e != cudaSuccess) return e;
-  k_meas_final_staged<MODE><<<dim3(p.n_samples * p.R_T, (NV + 7) / 8), 256, 0, st>>>(p, NV);
-  return cudaGetLastError();
+  return launch_chained(k_meas_final_staged<MODE>, dim3(p.n_samples * p.R_T, (NV + 7) / 8), 256, 0, st, p, NV);
 }
 
 template <int F, int MODE>
@@ -565,9 +570,11 @@ template <int F>
 __global__ void __launch_bounds__(SWEEP_BS) k_chirality(const ChiralityParams p) {
   constexpr int VEC = 4, PL = FmtInfo<F>::PLANES;
   using Chunk = typename FmtInfo<F>::Chunk;
+  chain_trigger();
   const int4 blk = p.blocks[blockIdx.x];
   const SampleDev& sd = p.samples[blk.x];
   const uint32_t h = (uint32_t)blk.z + threadIdx.x;
+  chain_wait();
   if (h >= ((uint32_t)sd.N >> 1)) return;
   const int g0 = blk.y * p.GPT, g1 = min(p.Gu, min(p.G, g0 + p.GPT));
   if (g0 >= g1) return;
@@ -579,14 +586,14 @@ __global__ void __launch_bounds__(SWEEP_BS) k_chirality(const ChiralityParams p)
   const long long kps = kd.plane_stride;
   for (int g = g0; g < g1; ++g) {
     Chunk c[PL];
-    load_chunks<F, LD_RO>(base + chunk_offset<F>(sd, g, gm.own), ps, c);
+    load_chunks<F, LD_PLAIN>(base + chunk_offset<F>(sd, g, gm.own), ps, c);
     Spins<VEC> s0;
     decode<F>(c, s0);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       Chunk cp[PL], cm[PL];
-      load_chunks<F, LD_RO>(base + chunk_offset<F>(sd, g, gm.nb[2 * a]), ps, cp);
-      load_chunks<F, LD_RO>(base + chunk_offset<F>(sd, g, gm.nb[2 * a + 1]), ps, cm);
+      load_chunks<F, LD_PLAIN>(base + chunk_offset<F>(sd, g, gm.nb[2 * a]), ps, cp);
+      load_chunks<F, LD_PLAIN>(base + chunk_offset<F>(sd, g, gm.nb[2 * a + 1]), ps, cm);
       Spins<VEC> sp, sm;
       decode<F>(cp, sp);
       decode<F>(cm, sm);
@@ -608,15 +615,14 @@ __global__ void __launch_bounds__(SWEEP_BS) k_chirality(const ChiralityParams p)
 
 cudaError_t launch_chirality(int fmt, const ChiralityParams& p, int n_blocks, cudaStream_t st) {
   switch (fmt) {
-    case FMT_F32: k_chirality<FMT_F32><<<n_blocks, SWEEP_BS, 0, st>>>(p); break;
-    case FMT_F16: k_chirality<FMT_F16><<<n_blocks, SWEEP_BS, 0, st>>>(p); break;
-    case FMT_BF16: k_chirality<FMT_BF16><<<n_blocks, SWEEP_BS, 0, st>>>(p); break;
-    case FMT_ANG16: k_chirality<FMT_ANG16><<<n_blocks, SWEEP_BS, 0, st>>>(p); break;
-    case FMT_OCT16: k_chirality<FMT_OCT16><<<n_blocks, SWEEP_BS, 0, st>>>(p); break;
-    case FMT_YX4: k_chirality<FMT_YX4><<<n_blocks, SWEEP_BS, 0, st>>>(p); break;
+    case FMT_F32: return launch_chained(k_chirality<FMT_F32>, n_blocks, SWEEP_BS, 0, st, p);
+    case FMT_F16: return launch_chained(k_chirality<FMT_F16>, n_blocks, SWEEP_BS, 0, st, p);
+    case FMT_BF16: return launch_chained(k_chirality<FMT_BF16>, n_blocks, SWEEP_BS, 0, st, p);
+    case FMT_ANG16: return launch_chained(k_chirality<FMT_ANG16>, n_blocks, SWEEP_BS, 0, st, p);
+    case FMT_OCT16: return launch_chained(k_chirality<FMT_OCT16>, n_blocks, SWEEP_BS, 0, st, p);
+    case FMT_YX4: return launch_chained(k_chirality<FMT_YX4>, n_blocks, SWEEP_BS, 0, st, p);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 // chiral pair overlaps from the binary32 chirality buffer (staged kernel)

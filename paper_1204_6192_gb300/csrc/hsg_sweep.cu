@@ -28,6 +28,7 @@ constexpr int sweep_min_blocks() {
 template <int F, bool HB, bool J16, bool FAST, bool EN, bool DEC>
 __global__ void __launch_bounds__(SWEEP_BS, sweep_min_blocks<F, HB, J16, EN>()) k_half_sweep(const SweepParams p) {
   extern __shared__ float esum[];
+  chain_trigger();
   const int k = p.reverse ? p.n_launch - 1 - (int)blockIdx.x : (int)blockIdx.x;
   sweep_block<F, HB, J16, FAST, EN, false, DEC>(p, p.blk_base + k, esum);
 }
@@ -39,19 +40,21 @@ template <int F>
 __global__ void __launch_bounds__(SWEEP_BS) k_decode_parity(const SweepParams p, int parity) {
   constexpr int PL = FmtInfo<F>::PLANES;
   using Chunk = typename FmtInfo<F>::Chunk;
+  chain_trigger();
   const int4 blk = p.blocks[p.blk_base + (int)blockIdx.x];
-  if (!p.active[blk.x]) return;
+  const bool frozen = !p.active[blk.x];
   const SampleDev& sd = p.samples[blk.x];
   const uint32_t half_n = (uint32_t)sd.N >> 1;
   const uint32_t h = (uint32_t)blk.z + threadIdx.x;
-  if (h >= half_n) return;
+  chain_wait();
+  if (frozen || h >= half_n) return;
   const int g0 = blk.y * p.GPT, g1 = min(p.G, g0 + p.GPT);
   const long long gstride = (long long)sd.N * FmtInfo<F>::CHUNK;
   const unsigned char* src = p.spins + sd.spin_off + ((size_t)parity * half_n + h) * FmtInfo<F>::CHUNK;
   unsigned char* dst = const_cast<unsigned char*>(p.dec) + sd.dec_off + (size_t)h * 16;
   for (int g = g0; g < g1; ++g) {
     Chunk c[PL];
-    load_chunks<F, LD_RO>(src + (long long)g * gstride, sd.plane_stride, c);
+    load_chunks<F, LD_PLAIN>(src + (long long)g * gstride, sd.plane_stride, c);
     Spins<4> s;
     decode<F>(c, s);
     uint4* d = reinterpret_cast<uint4*>(dst + (long long)g * half_n * 16);
@@ -75,20 +78,19 @@ static cudaError_t launch_fmt_dec(bool hb, bool j16, bool fast, bool en, const S
   const size_t smem = en ? sizeof(float) * (SWEEP_BS / 32) * p.GPT * FmtInfo<F>::VEC : 0;
   if (hb) {
     if (j16) {
-      if (fast) k_half_sweep<F, true, true, true, false, DEC><<<grid, block, 0, st>>>(p);
-      else k_half_sweep<F, true, true, false, false, DEC><<<grid, block, 0, st>>>(p);
+      if (fast) return launch_chained(k_half_sweep<F, true, true, true, false, DEC>, grid, block, 0, st, p);
+      else return launch_chained(k_half_sweep<F, true, true, false, false, DEC>, grid, block, 0, st, p);
     } else {
-      if (fast) k_half_sweep<F, true, false, true, false, DEC><<<grid, block, 0, st>>>(p);
-      else k_half_sweep<F, true, false, false, false, DEC><<<grid, block, 0, st>>>(p);
+      if (fast) return launch_chained(k_half_sweep<F, true, false, true, false, DEC>, grid, block, 0, st, p);
+      else return launch_chained(k_half_sweep<F, true, false, false, false, DEC>, grid, block, 0, st, p);
     }
   } else if (en) {
-    if (j16) k_half_sweep<F, false, true, false, true, DEC><<<grid, block, smem, st>>>(p);
-    else k_half_sweep<F, false, false, false, true, DEC><<<grid, block, smem, st>>>(p);
+    if (j16) return launch_chained(k_half_sweep<F, false, true, false, true, DEC>, grid, block, smem, st, p);
+    else return launch_chained(k_half_sweep<F, false, false, false, true, DEC>, grid, block, smem, st, p);
   } else {
-    if (j16) k_half_sweep<F, false, true, false, false, DEC><<<grid, block, 0, st>>>(p);
-    else k_half_sweep<F, false, false, false, false, DEC><<<grid, block, 0, st>>>(p);
+    if (j16) return launch_chained(k_half_sweep<F, false, true, false, false, DEC>, grid, block, 0, st, p);
+    else return launch_chained(k_half_sweep<F, false, false, false, false, DEC>, grid, block, 0, st, p);
   }
-  return cudaGetLastError();
 }
 
 template <int F>
@@ -118,12 +120,11 @@ cudaError_t launch_decode_parity(int fmt, const SweepParams& p, int parity, int 
                                  cudaStream_t st) {
   if (n_blocks <= 0) return cudaSuccess;
   switch (fmt) {
-    case FMT_ANG16: k_decode_parity<FMT_ANG16><<<n_blocks, SWEEP_BS, 0, st>>>(p, parity); break;
-    case FMT_OCT16: k_decode_parity<FMT_OCT16><<<n_blocks, SWEEP_BS, 0, st>>>(p, parity); break;
-    case FMT_YX4: k_decode_parity<FMT_YX4><<<n_blocks, SWEEP_BS, 0, st>>>(p, parity); break;
+    case FMT_ANG16: return launch_chained(k_decode_parity<FMT_ANG16>, n_blocks, SWEEP_BS, 0, st, p, parity);
+    case FMT_OCT16: return launch_chained(k_decode_parity<FMT_OCT16>, n_blocks, SWEEP_BS, 0, st, p, parity);
+    case FMT_YX4: return launch_chained(k_decode_parity<FMT_YX4>, n_blocks, SWEEP_BS, 0, st, p, parity);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 }  // namespace hsg

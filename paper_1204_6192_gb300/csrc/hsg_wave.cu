@@ -81,7 +81,10 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
   unsigned char* stages = smem + p.stage_off;
 
   const int4 blk = p.blocks[bidx];
-  if (!p.active[blk.x]) return;   // a frozen sample (block-uniform)
+  if (!p.active[blk.x]) {         // a frozen sample (block-uniform)
+    chain_wait();
+    return;
+  }
   const SampleDev& sd = p.samples[blk.x];
   const int L = sd.L, Lh = sd.Lh, R = SWEEP_BS / Lh;
   const int par = p.parity;
@@ -140,11 +143,6 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
-  if (warp == 0) {
-    for (int i = 0; i < S && i < ng; ++i) issue(i);
-  }
-
   // this thread's site, its neighbours' chunk offsets in a stage plane (+x, -x,
   // +y, -y, +z, -z) and its couplings
   const int lr = tid / Lh, hx = tid - lr * Lh;
@@ -177,6 +175,11 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
   uint32_t jh[6];
   load_record<J16>(p.rec, sd.rec_off + own, j6, h3);
   if (MIXED) load_record_j16(p.rec, sd.rec_off + own, jh);
+  chain_wait();      // spins of the kernels before it from here on
+  __syncthreads();
+  if (warp == 0) {
+    for (int i = 0; i < S && i < ng; ++i) issue(i);
+  }
   unsigned char* own_base = p.spins + sd.spin_off + (long long)own * CH;
   const long long ps = sd.plane_stride;
 
@@ -319,6 +322,7 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
 template <int F, bool J16, bool EN>
 __global__ void __launch_bounds__(SWEEP_BS, 4) k_staged_half(const SweepParams p) {
   extern __shared__ __align__(128) unsigned char smem[];
+  chain_trigger();
   const int k = p.reverse ? p.n_launch - 1 - (int)blockIdx.x : (int)blockIdx.x;
   staged_block<F, J16, EN>(p, p.blk_base + k, smem);
 }
@@ -404,8 +408,7 @@ template <int F, bool J16, bool EN>
 cudaError_t launch_h(const SweepParams& p, int n_blocks, size_t smem, cudaStream_t st) {
   cudaError_t e = allow_smem(k_staged_half<F, J16, EN>, smem);
   if (e != cudaSuccess) return e;
-  k_staged_half<F, J16, EN><<<n_blocks, SWEEP_BS, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_chained(k_staged_half<F, J16, EN>, n_blocks, SWEEP_BS, smem, st, p);
 }
 
 template <int F>
