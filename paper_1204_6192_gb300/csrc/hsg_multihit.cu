@@ -46,6 +46,13 @@ __device__ __forceinline__ int tentry(int x, int y, int z) {
   return (x < 0 || x >= T) ? TileShape<T>::NM + row_of<T>(y, z) : row_of<T>(y, z) * (T / 2) + (x >> 1);
 }
 
+// What bounds it: with binary32 tiles the shared-memory reads.  A half tile sweep
+// read six neighbours and the own spin (7 x 3 x 16 bytes a thread) and wrote one, 96
+// cycles of the SM's 128-byte path per warp against ~65 issue cycles; a thread's two
+// sites are each other's neighbours and its own spins are in registers, so it reads
+// five neighbours now (72 cycles).  Table 1's systems (256 of L = 32, FP32, 10 x (10 OR
+// + 1 HB)): 1653 -> 1387 us per colour.
+
 // What shared memory holds per (site, component): the four systems' binary16
 // or bfloat16 values as stored, or the decoded binary32 values (formats whose
 // decode is not a conversion).
@@ -99,11 +106,13 @@ __device__ __forceinline__ void sh_write(typename Sh<F>::E* A, int cs, int q,
 
 }  // namespace
 
-// Binary32 tiles: at most 80 registers per thread, i.e. 3 blocks of 256 threads
-// (T = 8) or 24 of 32 (T = 4) per SM; unbounded they take 92-99 registers and
-// run 2 blocks per SM.  The 16-bit formats compile to 80 registers unbounded.
+// Component formats: at most 80 registers per thread, i.e. 3 blocks of 256 threads
+// (T = 8) or 24 of 32 (T = 4) per SM; unbounded the binary32 tiles take 92-99
+// registers and run 2 blocks per SM.
 template <int F, int T>
-constexpr int multihit_min_blocks() { return F == FMT_F32 ? (T == 8 ? 3 : 24) : 0; }
+constexpr int multihit_min_blocks() {
+  return F == FMT_F32 || F == FMT_F16 || F == FMT_BF16 ? (T == 8 ? 3 : 24) : 0;
+}
 
 template <int F, bool J16, bool FAST, int T>
 __global__ void __launch_bounds__(TileShape<T>::NT, multihit_min_blocks<F, T>()) k_multihit(const MultihitParams p) {
@@ -153,23 +162,34 @@ __global__ void __launch_bounds__(TileShape<T>::NT, multihit_min_blocks<F, T>())
     fetch(((y + z + 1) & 1) == par ? -1 : T, y, z);
   }
 
-  // this thread's two sites, one of each parity
+  // This thread's two sites, x = 2 xh and 2 xh + 1 of one row: one of each parity, at
+  // the same entry e0 of their arrays, and each the other's neighbour along x.  Their
+  // other five neighbours lie at fixed distances from e0 but for the one along x,
+  // which may be a halo site.  For T = 8 the 32 lanes of a warp take rows of one
+  // parity of y + z, so that every lane's own pair lies on the same side (two rows
+  // adjacent in y and z per 8 lanes, which fall 16 banks apart: no bank conflict).
   const int t = threadIdx.x;
-  const int xh = t % (T / 2), y = (t / (T / 2)) % T, z = t / ((T / 2) * T);
-  int own[2], nb[2][6];
+  constexpr int HX = T / 2;
+  const int xh = t % HX;
+  int y, z;
+  if constexpr (T == 8) {
+    const int w = t >> 5, b = (t >> 2) & 1;
+    z = 2 * (w >> 1) + b;
+    y = (2 * ((t >> 3) & 3) + b + (w & 1)) & 7;
+  } else {
+    y = (t / HX) % T;
+    z = t / (HX * T);
+  }
+  const int row = row_of<T>(y, z), e0 = row * HX + xh;
+  int side[2];
   uint32_t gsite[2], gss[2];
   float j6[2][6], h3[2][3];
   uint32_t jh[2][6];
 #pragma unroll
   for (int par = 0; par < 2; ++par) {
-    const int x = 2 * xh + ((par + y + z) & 1);
-    own[par] = tentry<T>(x, y, z);
-    nb[par][0] = tentry<T>(x + 1, y, z);
-    nb[par][1] = tentry<T>(x - 1, y, z);
-    nb[par][2] = tentry<T>(x, y + 1, z);
-    nb[par][3] = tentry<T>(x, y - 1, z);
-    nb[par][4] = tentry<T>(x, y, z + 1);
-    nb[par][5] = tentry<T>(x, y, z - 1);
+    const int f = (par + y + z) & 1;
+    const int x = 2 * xh + f;
+    side[par] = f ? (xh == HX - 1 ? TS::NM + row : e0 + 1) : (xh == 0 ? TS::NM + row : e0 - 1);
     gss[par] = locate(x, y, z, gsite[par]);
     load_record<J16>(p.rec, sd.rec_off + gss[par], j6[par], h3[par]);
     if (MIXED) load_record_j16(p.rec, sd.rec_off + gss[par], jh[par]);
@@ -181,7 +201,17 @@ __global__ void __launch_bounds__(TileShape<T>::NT, multihit_min_blocks<F, T>())
   const uint32_t sweep0 = (uint32_t)p.counters[2 * blk.x];
   __syncthreads();
 
-  Chunk keep[2][PL];            // the last encoded state of the thread's two sites
+  // The last encoded state of the thread's two sites.  Component formats read their
+  // own spin and their neighbour's in the same thread from here instead of from
+  // shared memory.
+  Chunk keep[2][PL];
+  constexpr bool KEPT = F == FMT_F32 || F == FMT_F16 || F == FMT_BF16;
+  if constexpr (KEPT) {
+#pragma unroll
+    for (int par = 0; par < 2; ++par)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) keep[par][c] = *reinterpret_cast<const Chunk*>(&A[par][c * TS::CS + e0]);
+  }
   const int per = p.n_or + p.n_hb;
   for (int r = 0; r < p.n_rounds; ++r) {
     for (int k = 0; k < per; ++k) {
@@ -192,48 +222,64 @@ __global__ void __launch_bounds__(TileShape<T>::NT, multihit_min_blocks<F, T>())
         const E* O = A[par ^ 1];
         // local field h = sum_n J_n s_n + H, in the order +x, -x, +y, -y, +z, -z
         Spins<VEC> hf;
-        if constexpr (MIXED) {
+        auto add_spins = [&](int n, const Spins<VEC>& v) {
+          const float2 jj = f2(j6[par][n]);
 #pragma unroll
           for (int q = 0; q < VEC / 2; ++q) {
-            hf.x[q] = make_float2(0.0f, 0.0f);
-            hf.y[q] = make_float2(0.0f, 0.0f);
-            hf.z[q] = make_float2(0.0f, 0.0f);
+            hf.x[q] = n == 0 ? mul2(jj, v.x[q]) : fma2(jj, v.x[q], hf.x[q]);
+            hf.y[q] = n == 0 ? mul2(jj, v.y[q]) : fma2(jj, v.y[q], hf.y[q]);
+            hf.z[q] = n == 0 ? mul2(jj, v.z[q]) : fma2(jj, v.z[q], hf.z[q]);
           }
+        };
+        auto add_raw = [&](int n, uint2 a, uint2 b, uint2 c) {   // FP16 spins and couplings: exact products
+          if (n == 0) {
 #pragma unroll
-          for (int n = 0; n < 6; ++n) {
-            const uint2 a = O[nb[par][n]], b = O[TS::CS + nb[par][n]], c = O[2 * TS::CS + nb[par][n]];
-            fma_f16_pair(hf.x[0], a.x, jh[par][n]);
-            fma_f16_pair(hf.x[1], a.y, jh[par][n]);
-            fma_f16_pair(hf.y[0], b.x, jh[par][n]);
-            fma_f16_pair(hf.y[1], b.y, jh[par][n]);
-            fma_f16_pair(hf.z[0], c.x, jh[par][n]);
-            fma_f16_pair(hf.z[1], c.y, jh[par][n]);
+            for (int q = 0; q < VEC / 2; ++q) hf.x[q] = hf.y[q] = hf.z[q] = make_float2(0.0f, 0.0f);
+          }
+          fma_f16_pair(hf.x[0], a.x, jh[par][n]);
+          fma_f16_pair(hf.x[1], a.y, jh[par][n]);
+          fma_f16_pair(hf.y[0], b.x, jh[par][n]);
+          fma_f16_pair(hf.y[1], b.y, jh[par][n]);
+          fma_f16_pair(hf.z[0], c.x, jh[par][n]);
+          fma_f16_pair(hf.z[1], c.y, jh[par][n]);
+        };
+        auto add_at = [&](int n, int q) {        // the neighbour at entry q
+          if constexpr (MIXED) {
+            add_raw(n, O[q], O[TS::CS + q], O[2 * TS::CS + q]);
+          } else {
+            Spins<VEC> v;
+            sh_read<F>(O, TS::CS, q, v);
+            add_spins(n, v);
+          }
+        };
+        auto add_other = [&](int n) {            // the thread's other site
+          if constexpr (MIXED) {
+            add_raw(n, keep[par ^ 1][0], keep[par ^ 1][1], keep[par ^ 1][2]);
+          } else if constexpr (KEPT) {
+            Spins<VEC> v;
+            decode<F>(keep[par ^ 1], v);
+            add_spins(n, v);
+          } else {
+            add_at(n, e0);
+          }
+        };
+        const bool f = (par + y + z) & 1;        // (uniform over the warp for T = 8)
+        if constexpr (T == 8) {
+          if (f) {
+            add_at(0, side[par]);
+            add_other(1);
+          } else {
+            add_other(0);
+            add_at(1, side[par]);
           }
         } else {
-          {
-            Spins<VEC> nbv;
-            sh_read<F>(O, TS::CS, nb[par][0], nbv);
-            const float2 jj = f2(j6[par][0]);
-#pragma unroll
-            for (int q = 0; q < VEC / 2; ++q) {
-              hf.x[q] = mul2(jj, nbv.x[q]);
-              hf.y[q] = mul2(jj, nbv.y[q]);
-              hf.z[q] = mul2(jj, nbv.z[q]);
-            }
-          }
-#pragma unroll
-          for (int n = 1; n < 6; ++n) {
-            Spins<VEC> nbv;
-            sh_read<F>(O, TS::CS, nb[par][n], nbv);
-            const float2 jj = f2(j6[par][n]);
-#pragma unroll
-            for (int q = 0; q < VEC / 2; ++q) {
-              hf.x[q] = fma2(jj, nbv.x[q], hf.x[q]);
-              hf.y[q] = fma2(jj, nbv.y[q], hf.y[q]);
-              hf.z[q] = fma2(jj, nbv.z[q], hf.z[q]);
-            }
-          }
+          add_at(0, f ? side[par] : e0);
+          add_at(1, f ? e0 : side[par]);
         }
+        add_at(2, e0 + HX);
+        add_at(3, e0 - HX);
+        add_at(4, e0 + HX * TS::P);
+        add_at(5, e0 - HX * TS::P);
         {
           const float2 hx = f2(h3[par][0]), hy = f2(h3[par][1]), hz = f2(h3[par][2]);
 #pragma unroll
@@ -244,7 +290,8 @@ __global__ void __launch_bounds__(TileShape<T>::NT, multihit_min_blocks<F, T>())
           }
         }
         Spins<VEC> s;
-        sh_read<F>(A[par], TS::CS, own[par], s);
+        if constexpr (KEPT) decode<F>(keep[par], s);
+        else sh_read<F>(A[par], TS::CS, e0, s);
         if (hb) {
 #pragma unroll
           for (int q = 0; q < VEC / 2; ++q) {
@@ -261,7 +308,7 @@ __global__ void __launch_bounds__(TileShape<T>::NT, multihit_min_blocks<F, T>())
         }
         // through the storage codec, as a stored spin would be
         encode<F>(s, keep[par]);
-        sh_write<F>(A[par], TS::CS, own[par], keep[par]);
+        sh_write<F>(A[par], TS::CS, e0, keep[par]);
         __syncthreads();
       }
     }
