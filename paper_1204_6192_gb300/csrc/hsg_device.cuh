@@ -521,17 +521,35 @@ __device__ __forceinline__ void hb_poles(float a, float u1, float& dm, float& dp
     } else {
       // the hardware exp's relative error (<~ 2a * 6e-8) enters 1 - cos t as
       // <~ 1.2e-7 absolute
-      dm = (a >= 0.35f) ? __fmul_rn(-logf(__fmaf_rn(om, __expf(-2.0f * a), u1)), inv_a)
-                        : __fmul_rn(-log1pf(__fmul_rn(om, expm1f(-2.0f * a))), inv_a);
-      dp = __fsub_rn(2.0f, dm);                     // accurate while cos t >= 0
-      if (dm > 1.0f && a < 40.0f) {
-        // southern hemisphere: dp from its own form, and dm = 2 - dp (in [1, 2],
-        // so accurate); the direct dm cancels there when u1 is small, since
-        // 1 + (1 - u1) expm1(-2a) is then close to u1 (a = 7.7, u1 = 1.6e-5:
-        // ~1e-3 relative in dm, which reached the spin through sin t)
-        const float ep = (a >= 0.35f) ? __fsub_rn(__expf(2.0f * a), 1.0f) : expm1f(2.0f * a);
-        dp = __fmul_rn(log1pf(__fmul_rn(u1, ep)), inv_a);
-        dm = __fsub_rn(2.0f, dp);
+      if (a >= 0.35f) {
+        dm = __fmul_rn(-logf(__fmaf_rn(om, __expf(-2.0f * a), u1)), inv_a);
+        dp = __fsub_rn(2.0f, dm);                     // accurate while cos t >= 0
+        if (dm > 1.0f && a < 40.0f) {
+          // southern hemisphere: dp from its own form, and dm = 2 - dp (in [1, 2],
+          // so accurate); the direct dm cancels there when u1 is small, since
+          // 1 + (1 - u1) expm1(-2a) is then close to u1 (a = 7.7, u1 = 1.6e-5:
+          // ~1e-3 relative in dm, which reached the spin through sin t)
+          dp = __fmul_rn(log1pf(__fmul_rn(u1, __fsub_rn(__expf(2.0f * a), 1.0f))), inv_a);
+          dm = __fsub_rn(2.0f, dp);
+        }
+      } else {
+        // The same two forms with log1p and expm1.  Here both hemispheres take about
+        // half of the draws, so a warp would evaluate both forms for every lane.  Which
+        // one dm > 1 picks is known beforehand unless u1 is close to the equator's
+        // u* = 1 / (1 + e^a) = 1/2 - a/4 + a^3/48 (truncated below 1.1e-5): dm moves by
+        // at least 2 per unit of u1 there and its rounding error is below 1e-5, so
+        // beyond 4e-5 of u* each lane evaluates its own form once.  (Measured on 256
+        // systems of L = 32 at T = 100, FP32: 44 -> 38 us per half-sweep.)
+        const float us = __fmaf_rn(a, __fmaf_rn(__fmul_rn(a, a), 1.0f / 48.0f, -0.25f), 0.5f);
+        const bool sure = fabsf(__fsub_rn(u1, us)) > 4e-5f;
+        bool south = sure && u1 < us;
+        float d = __fmul_rn(log1pf(__fmul_rn(south ? u1 : om, expm1f(south ? 2.0f * a : -2.0f * a))), inv_a);
+        if (!sure && -d > 1.0f) {
+          south = true;
+          d = __fmul_rn(log1pf(__fmul_rn(u1, expm1f(2.0f * a))), inv_a);
+        }
+        dp = south ? d : __fadd_rn(2.0f, d);
+        dm = south ? __fsub_rn(2.0f, d) : -d;
       }
     }
   } else {
