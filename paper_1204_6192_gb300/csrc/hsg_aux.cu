@@ -13,19 +13,22 @@ namespace hsg {
 // ---------------------------------------------------------------------------
 // Energies.  Every bond joins an odd and an even site, so
 //   E = - sum_{odd i} s_i . h_i  - sum_{even j} H_j . s_j
-// with h_i the full local field (bonds + field) of the odd site i.
+// with h_i the full local field (bonds + field) of the odd site i.  Latency-bound:
+// 64 registers keep 32 warps on an SM and the eight warp sums of a chunk take 12
+// shuffles instead of 40 (L = 64, BF16, 64 systems: 74 -> 33 us; its bytes take 15).
 // ---------------------------------------------------------------------------
 template <int F, bool J16>
-__global__ void __launch_bounds__(RED_BS) k_energy(const EnergyParams p) {
+__global__ void __launch_bounds__(RED_BS, F == FMT_YX4 ? 0 : 4) k_energy(const EnergyParams p) {
   constexpr int VEC = FmtInfo<F>::VEC, PL = FmtInfo<F>::PLANES;
+  constexpr uint32_t CH = FmtInfo<F>::CHUNK;
   using Chunk = typename FmtInfo<F>::Chunk;
   extern __shared__ float esum[];                 // [2][RED_BS / 32][GPT * VEC]
   chain_trigger();
   const int4 blk = p.blocks[blockIdx.x];
   const SampleDev& sd = p.samples[blk.x];
-  const uint32_t h = (uint32_t)blk.z + threadIdx.x;
   const uint32_t half_n = (uint32_t)sd.N >> 1;
-  const bool active = h < half_n;
+  const bool active = (uint32_t)blk.z + threadIdx.x < half_n;
+  const uint32_t h = min((uint32_t)blk.z + threadIdx.x, half_n - 1);   // (idle threads: the last site, unused)
   const int g0 = blk.y * p.GPT;
   const int g1 = min(p.G, g0 + p.GPT);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -33,75 +36,62 @@ __global__ void __launch_bounds__(RED_BS) k_energy(const EnergyParams p) {
   float* esum_even = esum;
   float* esum_odd = esum + (RED_BS / 32) * stride;
 
-  SiteGeom gm;                                   // the odd site with half-index h
-  float j6[6], h3[3], je[6], he[3];
-  long long nb_off[6], odd_off = 0, even_off = 0;
   const unsigned char* base = p.spins + sd.spin_off;
   const long long ps = sd.plane_stride;
-  const long long gstride = (long long)sd.N * FmtInfo<F>::CHUNK;
-  if (active) {
-    gm = site_geom(sd, h, 1);
-    load_record<J16>(p.rec, sd.rec_off + gm.own, j6, h3);
-    load_record<J16>(p.rec, sd.rec_off + h, je, he);   // even site with the same half-index
+  const long long gstride = (long long)sd.N * CH;
+  float j6[6], h3[3], je[6], he[3];
+  const SiteGeom gm = site_geom(sd, h, 1);       // the odd site with half-index h
+  load_record<J16>(p.rec, sd.rec_off + gm.own, j6, h3);
+  load_record<J16>(p.rec, sd.rec_off + h, je, he);   // even site with the same half-index
+  uint32_t nb_off[6];
 #pragma unroll
-    for (int n = 0; n < 6; ++n) nb_off[n] = chunk_offset<F>(sd, g0, gm.nb[n]);
-    odd_off = chunk_offset<F>(sd, g0, gm.own);
-    even_off = chunk_offset<F>(sd, g0, h);
-  }
+  for (int n = 0; n < 6; ++n) nb_off[n] = gm.nb[n] * CH;
   chain_wait();
   for (int g = g0; g < g1; ++g) {
-    float eo[VEC], ee[VEC];
+    const unsigned char* base_g = base + (long long)g * gstride;
+    Chunk nc[6][PL], co[PL], ce[PL];
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) { eo[v] = 0.0f; ee[v] = 0.0f; }
-    if (active) {
-      const long long dg = (long long)(g - g0) * gstride;
-      Chunk nc[6][PL], co[PL], ce[PL];
+    for (int n = 0; n < 6; ++n) load_chunks_at<F, LD_PLAIN>(base_g, ps, nb_off[n], nc[n]);
+    load_chunks_at<F, LD_PLAIN>(base_g, ps, gm.own * CH, co);
+    load_chunks_at<F, LD_PLAIN>(base_g, ps, h * CH, ce);
+    Spins<VEC> hf, t;
+    decode<F>(nc[0], t);
 #pragma unroll
-      for (int n = 0; n < 6; ++n) load_chunks<F, LD_PLAIN>(base + nb_off[n] + dg, ps, nc[n]);
-      load_chunks<F, LD_PLAIN>(base + odd_off + dg, ps, co);
-      load_chunks<F, LD_PLAIN>(base + even_off + dg, ps, ce);
-      Spins<VEC> hf, t;
-      decode<F>(nc[0], t);
-#pragma unroll
-      for (int q = 0; q < VEC / 2; ++q) {
-        hf.x[q] = mul2(f2(j6[0]), t.x[q]);
-        hf.y[q] = mul2(f2(j6[0]), t.y[q]);
-        hf.z[q] = mul2(f2(j6[0]), t.z[q]);
-      }
-#pragma unroll
-      for (int n = 1; n < 6; ++n) {
-        decode<F>(nc[n], t);
-#pragma unroll
-        for (int q = 0; q < VEC / 2; ++q) {
-          hf.x[q] = fma2(f2(j6[n]), t.x[q], hf.x[q]);
-          hf.y[q] = fma2(f2(j6[n]), t.y[q], hf.y[q]);
-          hf.z[q] = fma2(f2(j6[n]), t.z[q], hf.z[q]);
-        }
-      }
-      Spins<VEC> so, se;
-      decode<F>(co, so);
-      decode<F>(ce, se);
-#pragma unroll
-      for (int q = 0; q < VEC / 2; ++q) {
-        const float2 hx2 = add2(hf.x[q], f2(h3[0]));
-        const float2 hy2 = add2(hf.y[q], f2(h3[1]));
-        const float2 hz2 = add2(hf.z[q], f2(h3[2]));
-        const float2 o = dot3_2(so.x[q], so.y[q], so.z[q], hx2, hy2, hz2);
-        const float2 e = dot3_2(se.x[q], se.y[q], se.z[q], f2(he[0]), f2(he[1]), f2(he[2]));
-        eo[2 * q] = -o.x;
-        eo[2 * q + 1] = -o.y;
-        ee[2 * q] = -e.x;
-        ee[2 * q + 1] = -e.y;
-      }
+    for (int q = 0; q < VEC / 2; ++q) {
+      hf.x[q] = mul2(f2(j6[0]), t.x[q]);
+      hf.y[q] = mul2(f2(j6[0]), t.y[q]);
+      hf.z[q] = mul2(f2(j6[0]), t.z[q]);
     }
 #pragma unroll
-    for (int v = 0; v < VEC; ++v) {
-      const float to = warp_sum(eo[v]);
-      const float te = warp_sum(ee[v]);
-      if (lane == 0) {
-        esum_odd[warp * stride + (g - g0) * VEC + v] = to;
-        esum_even[warp * stride + (g - g0) * VEC + v] = te;
+    for (int n = 1; n < 6; ++n) {
+      decode<F>(nc[n], t);
+#pragma unroll
+      for (int q = 0; q < VEC / 2; ++q) {
+        hf.x[q] = fma2(f2(j6[n]), t.x[q], hf.x[q]);
+        hf.y[q] = fma2(f2(j6[n]), t.y[q], hf.y[q]);
+        hf.z[q] = fma2(f2(j6[n]), t.z[q], hf.z[q]);
       }
+    }
+    Spins<VEC> so, se;
+    decode<F>(co, so);
+    decode<F>(ce, se);
+    float eo[VEC], ee[VEC];
+#pragma unroll
+    for (int q = 0; q < VEC / 2; ++q) {
+      const float2 hx2 = add2(hf.x[q], f2(h3[0]));
+      const float2 hy2 = add2(hf.y[q], f2(h3[1]));
+      const float2 hz2 = add2(hf.z[q], f2(h3[2]));
+      const float2 o = dot3_2(so.x[q], so.y[q], so.z[q], hx2, hy2, hz2);
+      const float2 e = dot3_2(se.x[q], se.y[q], se.z[q], f2(he[0]), f2(he[1]), f2(he[2]));
+      eo[2 * q] = active ? -o.x : 0.0f;
+      eo[2 * q + 1] = active ? -o.y : 0.0f;
+      ee[2 * q] = active ? -e.x : 0.0f;
+      ee[2 * q + 1] = active ? -e.y : 0.0f;
+    }
+    const float to = warp_sum4_scatter(eo, lane), te = warp_sum4_scatter(ee, lane);
+    if ((lane & 7) == 0) {
+      esum_odd[warp * stride + (g - g0) * VEC + (lane >> 3)] = to;
+      esum_even[warp * stride + (g - g0) * VEC + (lane >> 3)] = te;
     }
   }
   __syncthreads();
@@ -132,8 +122,8 @@ __global__ void __launch_bounds__(RED_BS) k_energy(const EnergyParams p) {
 // (j <= k) decisions are taken at once, one warp per pair and 32 values of j, each
 // exactly as the sequential walk would take it.  What is left of the sequential
 // walk is one bit test per pair.  (R_T = 32: the walk with its FP64 arithmetic and
-// exponentials in the chain took 18 us, this launch with the sums takes 5; measured
-// on L32_fp32.)
+// exponentials in the chain took 18 us and the sums before it 2.4; one launch now
+// takes 11.8; L32_fp32.)
 // ---------------------------------------------------------------------------
 constexpr int TAIL_BS = 256;
 constexpr int TAIL_MASKS = 4096;      // decision words in shared memory: the chains run in batches
