@@ -43,9 +43,13 @@ struct hsg_ctx {
   // device state
   unsigned char* spins = nullptr;
   size_t spin_bytes = 0;
-  // packed formats: the opposite parity decoded to binary32 before each half-sweep
-  bool dec_once = false;
-  unsigned char* dec = nullptr;
+  // packed formats: the spins decoded to binary32 for their six neighbours.  One
+  // buffer per parity: a half-sweep reads its neighbours from the other parity's and
+  // leaves its own spins decoded in its own (dec_both; where the second buffer does
+  // not fit, one buffer, filled before each half-sweep)
+  bool dec_once = false, dec_both = false;
+  bool dec_fresh = false;             // the next half-sweep's neighbours are in dec
+  unsigned char* dec = nullptr;       // [parity][dec_bytes], or [dec_bytes]
   size_t dec_bytes = 0;
   void* rec = nullptr;
   size_t rec_bytes = 0;
@@ -242,7 +246,8 @@ SweepParams sweep_params(hsg_ctx* c, int parity, int sweep_offset) {
   p.blk_base = 0;
   p.n_launch = c->n_sweep_blocks;
   p.reverse = 0;
-  p.dec = c->dec;
+  p.dec = c->dec_both ? c->dec + (1 - parity) * c->dec_bytes : c->dec;
+  p.dec_out = c->dec_both ? c->dec + parity * c->dec_bytes : nullptr;
   p.stage_bytes = c->staged_possible ? staged_stage_bytes(c->fmt, c->Lh_max) : 0;
   p.stage_off = 0;
   p.err = c->d_bar + 5;
@@ -374,9 +379,11 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
     // of a launch are independent, so the order changes no result): each
     // launch starts on the planes whose spins the previous one left in L2.
     // Packed formats: the decode launch runs forward, the sweep backward.
-    p.reverse = c->dec_once ? 1 : parity;
-    // packed formats: decode the other parity once for the six neighbour loads
-    if (c->dec_once) HSG_CUDA(c, launch_decode_parity(c->fmt, p, 1 - parity, b1 - b0, c->stream));
+    p.reverse = c->dec_once && !c->dec_both ? 1 : parity;
+    // packed formats: decode the other parity once for the six neighbour loads,
+    // unless the half-sweep before this one left it decoded
+    if (c->dec_once && !c->dec_fresh) HSG_CUDA(c, launch_decode_parity(c->fmt, p, 1 - parity, b1 - b0, c->stream));
+    c->dec_fresh = c->dec_both;
     HSG_CUDA(c, launch_half_sweep(c->fmt, hb, c->j16, c->opt.fast_math != 0, energy, c->dec_once, p,
                                   b1 - b0, c->stream));
   }
@@ -517,6 +524,7 @@ hsg_status fused_sweep_pairs(hsg_ctx* c, int pairs) {
 // n OR sweeps outside a step: fused pairs where in use, the rest per half-sweep.
 hsg_status or_sweeps(hsg_ctx* c, int n, int sweep_offset) {
   int k = 0;
+  c->dec_fresh = false;
   if (c->use_fused && n >= 2) {
     HSG_TRY(fused_sweep_pairs(c, n / 2));
     k = 2 * (n / 2);
@@ -534,6 +542,7 @@ hsg_status enqueue_step(hsg_ctx* c) {
   const int np = (int)c->pass_bound.size() - 1;
   for (int ps = 0; ps < np; ++ps) {
     const int b0 = c->pass_bound[ps], b1 = c->pass_bound[ps + 1];
+    c->dec_fresh = false;
     for (int k = 0; k < nhb; ++k) HSG_TRY(half_sweeps(c, true, k, false, b0, b1));
     int k = 0;
     if (c->use_fused && np == 1) {
@@ -542,6 +551,7 @@ hsg_status enqueue_step(hsg_ctx* c) {
       const int pairs = (nor - 1) / 2;
       HSG_TRY(fused_sweep_pairs(c, pairs));
       k = 2 * pairs;
+      c->dec_fresh = false;
     }
     for (; k < nor; ++k) HSG_TRY(half_sweeps(c, false, nhb + k, k == nor - 1, b0, b1));
   }
@@ -1182,7 +1192,16 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
   HSG_ALLOC(c->spins, c->spin_bytes);
   c->dec_once = fmt_decodes_once(fmt);
   if (c->dec_once) {
-    HSG_ALLOC(c->dec, c->dec_bytes);
+    // both parities if they fit (not counted as an allocation that has to succeed)
+    void* both = nullptr;
+    c->dec_both = opt.inject_alloc_fault == 0 && cudaMalloc(&both, 2 * c->dec_bytes) == cudaSuccess;
+    if (c->dec_both) {
+      c->allocations.push_back(both);
+      c->dec = (unsigned char*)both;
+    } else {
+      cudaGetLastError();
+      HSG_ALLOC(c->dec, c->dec_bytes);
+    }
   }
   HSG_ALLOC(c->rec, c->rec_bytes);
   HSG_ALLOC(c->d_sd, sizeof(SampleDev) * n_samples);
@@ -1352,6 +1371,7 @@ hsg_status hsg_sweep_hb(hsg_ctx* c, int n) {
   if (n == 0) return HSG_OK;
   HSG_CUDA(c, cudaSetDevice(c->device));
   c->e_valid = false;
+  c->dec_fresh = false;
   for (int k = 0; k < n; ++k) HSG_TRY(half_sweeps(c, true, k));
   HSG_CUDA(c, launch_bump(c->d_counters, c->d_active, c->ns, n, 0, c->stream));
   return HSG_OK;

@@ -86,6 +86,7 @@ struct SweepParams {
                             // (so a launch starts on the planes the previous one ended with)
   uint32_t rk[20];          // Philox round keys of the seed
   const unsigned char* dec; // packed formats: the opposite parity as binary32 (see SampleDev)
+  unsigned char* dec_out;   // packed formats: where the updated spins go as binary32 (null: nowhere)
   // staged sweeps (hsg_wave.cu): bytes of one stage of neighbour rows, offset of
   // stage 0 in dynamic shared memory, the error word of their bounded waits
   int stage_bytes, stage_off;

@@ -8,6 +8,13 @@
 
 namespace hsg {
 
+// Four decoded systems of a site into the buffer of decoded neighbours.
+__device__ __forceinline__ void store_decoded(unsigned char* p, long long plane_stride, const Spins<4>& s) {
+  typename FmtInfo<FMT_F32>::Chunk c[3];
+  encode<FMT_F32>(s, c);
+  store_chunks<FMT_F32>(p, plane_stride, c);
+}
+
 // One block's share of a half-sweep: virtual block `bidx` of the sweep block
 // table.  CG: every load of data written during the launch bypasses L1 (for
 // the persistent kernel, whose blocks see each other's writes across grid
@@ -177,12 +184,17 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
       }
       encode<F>(s, c);
       if (!EN || active) store_chunks_at<F>(own_b, ps, own_off, c);
+      Spins<VEC> st;                  // the stored values
+      if constexpr (EN || DEC) decode<F>(c, st);
+      if constexpr (DEC) {
+        if (p.dec_out && (!EN || active))   // the next half-sweep's neighbours, decoded
+          store_decoded(p.dec_out + sd.dec_off + (long long)g * half_n * 16 + (size_t)(gm.own - (half_n - ob)) * 16,
+                        dps, st);
+      }
 
       if (EN) {
         // energy of the new state from the stored values: every bond joins one
         // odd and one even site, E = - sum_odd s_i.h_i - sum_even H_j.s_j
-        Spins<VEC> st;
-        decode<F>(c, st);
 #pragma unroll
         for (int k = 0; k < VEC / 2; ++k) {
           float2 d;

@@ -19,14 +19,15 @@ namespace hsg {
 // loads in flight.  Bounded to 64 registers, i.e. 4 blocks (32 warps) per SM,
 // every storage format but YX4 compiles with at most a few bytes of spill and
 // runs 2-15 % faster than at its natural 74-104 registers (2-3 blocks per SM).
-// The YX4 decode needs ~120 registers and spills heavily under any bound.
-template <int F, bool HB, bool J16, bool EN>
+// The YX4 decode of six neighbours needs ~120 registers and spills heavily under any
+// bound; with decoded neighbours its plain over-relaxation sweep takes 66.
+template <int F, bool HB, bool EN, bool DEC>
 constexpr int sweep_min_blocks() {
-  return F == FMT_YX4 ? 0 : 4;
+  return F == FMT_YX4 && (!DEC || HB || EN) ? 0 : 4;
 }
 
 template <int F, bool HB, bool J16, bool FAST, bool EN, bool DEC>
-__global__ void __launch_bounds__(SWEEP_BS, sweep_min_blocks<F, HB, J16, EN>()) k_half_sweep(const SweepParams p) {
+__global__ void __launch_bounds__(SWEEP_BS, sweep_min_blocks<F, HB, EN, DEC>()) k_half_sweep(const SweepParams p) {
   extern __shared__ float esum[];
   chain_trigger();
   const int k = p.reverse ? p.n_launch - 1 - (int)blockIdx.x : (int)blockIdx.x;
@@ -57,14 +58,7 @@ __global__ void __launch_bounds__(SWEEP_BS) k_decode_parity(const SweepParams p,
     load_chunks<F, LD_PLAIN>(src + (long long)g * gstride, sd.plane_stride, c);
     Spins<4> s;
     decode<F>(c, s);
-    uint4* d = reinterpret_cast<uint4*>(dst + (long long)g * half_n * 16);
-    const long long ps = sd.dec_plane_stride / 16;
-    d[0] = make_uint4(__float_as_uint(s.x[0].x), __float_as_uint(s.x[0].y), __float_as_uint(s.x[1].x),
-                      __float_as_uint(s.x[1].y));
-    d[ps] = make_uint4(__float_as_uint(s.y[0].x), __float_as_uint(s.y[0].y), __float_as_uint(s.y[1].x),
-                       __float_as_uint(s.y[1].y));
-    d[2 * ps] = make_uint4(__float_as_uint(s.z[0].x), __float_as_uint(s.z[0].y), __float_as_uint(s.z[1].x),
-                           __float_as_uint(s.z[1].y));
+    store_decoded(dst + (long long)g * half_n * 16, sd.dec_plane_stride, s);
   }
 }
 
