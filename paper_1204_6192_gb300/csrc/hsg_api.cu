@@ -141,6 +141,12 @@ struct hsg_ctx {
   long long pass_bytes = 0;             // resolved footprint bound (0: one pass)
   int max_passes = 1;
 
+  // results on their way to the caller (device -> here -> caller's memory), pinned;
+  // grows to the largest result asked for, at most RESULT_MAX
+  unsigned char* results = nullptr;
+  size_t results_bytes = 0;
+  std::vector<unsigned char> results_large;   // of one call beyond RESULT_MAX, or without pinned memory
+
   hsg_status err = HSG_OK;
   std::string msg;
   std::vector<void*> allocations;
@@ -563,16 +569,65 @@ hsg_status enqueue_step(hsg_ctx* c) {
   return HSG_OK;
 }
 
-// A bounded device wait that ran out (persistent schedule, staged measurement)
-// after the stream has been synchronised.
-hsg_status poll_device_error(hsg_ctx* c) {
-  unsigned int err[5] = {0u, 0u, 0u, 0u, 0u};
-  HSG_CUDA(c, cudaMemcpy(err, c->d_bar + 2, sizeof(err), cudaMemcpyDeviceToHost));
+// The error words of bounded device waits (persistent schedule, staged measurement,
+// fused and wave sweeps) and of the checked build.
+constexpr int ERR_WORDS = 5;
+hsg_status device_error(hsg_ctx* c, const unsigned int* err) {
   if (err[4]) return fail(c, HSG_ESTATE, "a device bounds check of a sweep kernel failed (HSG_CHECK build)");
   if (err[0]) return fail(c, HSG_ETIMEOUT, "a grid barrier wait of the persistent step kernel timed out");
   if (err[1]) return fail(c, HSG_ETIMEOUT, "a wait for a staged spin copy of a measurement kernel timed out");
   if (err[2]) return fail(c, HSG_ETIMEOUT, "a wait for a staged plane copy of the fused sweep kernel timed out");
   if (err[3]) return fail(c, HSG_ETIMEOUT, "a wait of the wave sweep kernel for its even blocks timed out");
+  return HSG_OK;
+}
+
+// After the stream has been synchronised.
+hsg_status poll_device_error(hsg_ctx* c) {
+  unsigned int err[ERR_WORDS] = {0u, 0u, 0u, 0u, 0u};
+  HSG_CUDA(c, cudaMemcpy(err, c->d_bar + 2, sizeof(err), cudaMemcpyDeviceToHost));
+  return device_error(c, err);
+}
+
+// Wait for the stream and bring device arrays and the error words to the host: the
+// copies go to the context's pinned buffer behind the kernels, so one
+// synchronisation serves them all (copies to pageable memory each waited for the
+// stream, and the error words for another round trip).  host[k] points to the
+// bytes of the k-th source until the next call.
+constexpr size_t RESULT_MAX = 64u << 20;
+struct ResultCopy {
+  const void* src;
+  size_t bytes;
+};
+hsg_status fetch_results(hsg_ctx* c, const std::vector<ResultCopy>& src, const unsigned char** host) {
+  size_t need = 64;
+  for (const auto& r : src) need += (r.bytes + 63) / 64 * 64;
+  if (need > c->results_bytes && need <= RESULT_MAX) {
+    if (c->results) cudaFreeHost(c->results);
+    c->results = nullptr;
+    c->results_bytes = 0;
+    if (cudaMallocHost(&c->results, need) == cudaSuccess) c->results_bytes = need;
+    else cudaGetLastError();
+  }
+  unsigned char* buf = c->results;
+  c->results_large = std::vector<unsigned char>(need > c->results_bytes ? need : 0);
+  if (need > c->results_bytes) buf = c->results_large.data();
+  size_t off = 64;
+  for (size_t k = 0; k < src.size(); ++k) {
+    HSG_CUDA(c, cudaMemcpyAsync(buf + off, src[k].src, src[k].bytes, cudaMemcpyDeviceToHost, c->stream));
+    host[k] = buf + off;
+    off += (src[k].bytes + 63) / 64 * 64;
+  }
+  HSG_CUDA(c, cudaMemcpyAsync(buf, c->d_bar + 2, sizeof(unsigned int) * ERR_WORDS, cudaMemcpyDeviceToHost, c->stream));
+  HSG_CUDA(c, cudaStreamSynchronize(c->stream));
+  return device_error(c, reinterpret_cast<const unsigned int*>(buf));
+}
+
+// [ns][Wp] energies of the context to [ns][W] of the caller
+hsg_status fetch_energies(hsg_ctx* c, double* E_sys) {
+  const unsigned char* host = nullptr;
+  HSG_TRY(fetch_results(c, {{c->d_E, sizeof(double) * c->ns * (size_t)c->Wp}}, &host));
+  for (int s = 0; s < c->ns; ++s)
+    std::memcpy(E_sys + (size_t)s * c->W, host + sizeof(double) * s * (size_t)c->Wp, sizeof(double) * c->W);
   return HSG_OK;
 }
 
@@ -1483,22 +1538,14 @@ hsg_status hsg_energies(hsg_ctx* c, double* E_sys) {
   HSG_CUDA(c, cudaSetDevice(c->device));
   HSG_TRY(enqueue_energy(c));
   c->e_valid = true;
-  HSG_CUDA(c, cudaMemcpy2DAsync(E_sys, sizeof(double) * c->W, c->d_E, sizeof(double) * c->Wp,
-                                sizeof(double) * c->W, c->ns, cudaMemcpyDeviceToHost, c->stream));
-  HSG_CUDA(c, cudaStreamSynchronize(c->stream));
-  HSG_TRY(poll_device_error(c));
-  return HSG_OK;
+  return fetch_energies(c, E_sys);
 }
 
 hsg_status hsg_last_energies(hsg_ctx* c, double* E_sys) {
   HSG_CHECK_CTX(c);
   if (!E_sys) return bad_arg(c, "E_sys is NULL");
   HSG_CUDA(c, cudaSetDevice(c->device));
-  HSG_CUDA(c, cudaMemcpy2DAsync(E_sys, sizeof(double) * c->W, c->d_E, sizeof(double) * c->Wp,
-                                sizeof(double) * c->W, c->ns, cudaMemcpyDeviceToHost, c->stream));
-  HSG_CUDA(c, cudaStreamSynchronize(c->stream));
-  HSG_TRY(poll_device_error(c));
-  return HSG_OK;
+  return fetch_energies(c, E_sys);
 }
 
 // Parameters common to the measurement launches; g.ok selects the staged
@@ -1551,20 +1598,18 @@ hsg_status hsg_measure(hsg_ctx* c, hsg_obs* o) {
     p.n_tiles = n_tiles;
     HSG_CUDA(c, launch_qtensor(c->fmt, p, c->stream));
   }
-  std::vector<double> E((size_t)c->ns * c->Wp);
-  std::vector<int> perm((size_t)c->ns * c->R_O * c->R_T);
-  HSG_CUDA(c, cudaMemcpyAsync(E.data(), c->d_E, sizeof(double) * E.size(), cudaMemcpyDeviceToHost,
-                              c->stream));
-  HSG_CUDA(c, cudaMemcpyAsync(perm.data(), c->d_perm, sizeof(int) * perm.size(),
-                              cudaMemcpyDeviceToHost, c->stream));
-  if (pairs && o->q)
-    HSG_CUDA(c, cudaMemcpyAsync(o->q, c->d_q, sizeof(double) * c->ns * c->R_T * 9,
-                                cudaMemcpyDeviceToHost, c->stream));
-  if (pairs && o->qk)
-    HSG_CUDA(c, cudaMemcpyAsync(o->qk, c->d_qk, sizeof(double) * c->ns * c->R_T * 54,
-                                cudaMemcpyDeviceToHost, c->stream));
-  HSG_CUDA(c, cudaStreamSynchronize(c->stream));
-  HSG_TRY(poll_device_error(c));
+  const size_t q_bytes = pairs && o->q ? sizeof(double) * c->ns * c->R_T * 9 : 0;
+  const size_t qk_bytes = pairs && o->qk ? sizeof(double) * c->ns * c->R_T * 54 : 0;
+  const unsigned char* host[4];
+  std::vector<ResultCopy> src{{c->d_E, sizeof(double) * c->ns * (size_t)c->Wp},
+                              {c->d_perm, sizeof(int) * c->ns * (size_t)c->R_O * c->R_T}};
+  if (q_bytes) src.push_back({c->d_q, q_bytes});
+  if (qk_bytes) src.push_back({c->d_qk, qk_bytes});
+  HSG_TRY(fetch_results(c, src, host));
+  const double* E = reinterpret_cast<const double*>(host[0]);
+  const int* perm = reinterpret_cast<const int*>(host[1]);
+  if (q_bytes) std::memcpy(o->q, host[2], q_bytes);
+  if (qk_bytes) std::memcpy(o->qk, host[q_bytes ? 3 : 2], qk_bytes);
   for (int s = 0; s < c->ns; ++s)
     for (int r = 0; r < c->R_O; ++r)
       for (int t = 0; t < c->R_T; ++t) {
@@ -1677,14 +1722,14 @@ hsg_status hsg_measure_overlaps(hsg_ctx* c, double* D, double* C) {
     p.n_tiles = staged ? g.n_tiles : n_tiles;
     HSG_CUDA(c, launch_overlaps(c->fmt, p, direct_c, c->stream));
   }
-  if (D)
-    HSG_CUDA(c, cudaMemcpyAsync(D, c->d_D, sizeof(double) * c->ns * c->R_T * n_pairs * 8,
-                                cudaMemcpyDeviceToHost, c->stream));
-  if (C)
-    HSG_CUDA(c, cudaMemcpyAsync(C, c->d_C, sizeof(double) * c->ns * c->R_T * n_pairs * 24,
-                                cudaMemcpyDeviceToHost, c->stream));
-  HSG_CUDA(c, cudaStreamSynchronize(c->stream));
-  HSG_TRY(poll_device_error(c));
+  const size_t n = sizeof(double) * c->ns * (size_t)c->R_T * n_pairs;
+  const unsigned char* host[2];
+  std::vector<ResultCopy> src;
+  if (D) src.push_back({c->d_D, 8 * n});
+  if (C) src.push_back({c->d_C, 24 * n});
+  HSG_TRY(fetch_results(c, src, host));
+  if (D) std::memcpy(D, host[0], 8 * n);
+  if (C) std::memcpy(C, host[D ? 1 : 0], 24 * n);
   return HSG_OK;
 }
 
@@ -1722,10 +1767,10 @@ hsg_status hsg_get_perm(hsg_ctx* c, int32_t* perm) {
   HSG_CHECK_CTX(c);
   if (!perm) return bad_arg(c, "perm is NULL");
   HSG_CUDA(c, cudaSetDevice(c->device));
-  HSG_CUDA(c, cudaMemcpyAsync(perm, c->d_perm, sizeof(int) * c->ns * c->R_O * c->R_T,
-                              cudaMemcpyDeviceToHost, c->stream));
-  HSG_CUDA(c, cudaStreamSynchronize(c->stream));
-  HSG_TRY(poll_device_error(c));
+  const size_t bytes = sizeof(int) * c->ns * (size_t)c->R_O * c->R_T;
+  const unsigned char* host = nullptr;
+  HSG_TRY(fetch_results(c, {{c->d_perm, bytes}}, &host));
+  std::memcpy(perm, host, bytes);
   return HSG_OK;
 }
 
@@ -1964,6 +2009,7 @@ void hsg_destroy(hsg_ctx* c) {
   if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
   if (c->graph) cudaGraphDestroy(c->graph);
   for (void* p : c->allocations) cudaFree(p);
+  if (c->results) cudaFreeHost(c->results);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;
 }
