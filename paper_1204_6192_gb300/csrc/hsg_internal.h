@@ -148,6 +148,7 @@ struct OverlapParams {
   // staged kernels only (sub > 0): storage sites per stage and per block, chunk
   // groups staged, padded bytes per staged (plane, group) row; bounded waits
   int sub, tile_ss, Gu, grow;
+  int red_floats;           // floats of dynamic shared memory (the block's reduction reuses the stages)
   unsigned int* err;        // set when a wait for a staged copy ran out
   unsigned long long timeout_ns;
 };

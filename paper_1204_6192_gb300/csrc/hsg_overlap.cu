@@ -253,20 +253,27 @@ template <int MODE, int NR>
 __host__ __device__ constexpr int staged_products() {
   return MODE == MEAS_QTENSOR ? 9 : (MODE == MEAS_CHIRAL ? 3 : 1) * (NR * (NR - 1) / 2);
 }
+// warp groups of a block.  The chiralities' components share no product and no
+// value, so three groups of 8 warps walk the same sites with a third of the sums
+// each: up to 42 accumulators a lane instead of 126, which left 8 warps on an SM.
+// (The tensor's rows all read replica 1: three groups decode it three times, 780 us
+// against 413 us at L = 128.)
+template <int MODE>
+__host__ __device__ constexpr int staged_groups() { return MODE == MEAS_CHIRAL ? 3 : 1; }
 
 }  // namespace
 
 template <int F, int MODE, int NR>
-__global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) {
+__global__ void __launch_bounds__(MEAS_BS * staged_groups<MODE>()) k_meas_staged(const OverlapParams p) {
   using FI = FmtInfo<F>;
-  constexpr int NQ = staged_products<MODE, NR>();
+  constexpr int NG = staged_groups<MODE>(), BS = MEAS_BS * NG;
+  constexpr int NQ = staged_products<MODE, NR>(), NQG = NQ / NG;   // products of the block, of a group
   constexpr int NV = NQ * NM;
-  constexpr int NW = MEAS_BS / 32;
+  constexpr int NW = MEAS_BS / 32;       // warps of a group
   extern __shared__ __align__(128) unsigned char stage[];
   __shared__ uint64_t full[MS_STAGES];   // a stage's copies have landed
   __shared__ uint64_t empty[MS_STAGES];  // every warp is done with a stage's buffer
   __shared__ float2 tw[512];             // (cos, sin)(2 pi x / L)
-  __shared__ float red[NV][32];          // the block's sums per (value, slot of the round)
   chain_trigger();
   const int s = blockIdx.z, round = blockIdx.y;
   // the sample's geometry in registers: the loop's barrier operations are
@@ -281,19 +288,19 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
   const uint32_t b1 = min(N, b0 + (uint32_t)p.tile_ss);
   const int sub = p.sub;
   const int n_sub = (int)((b1 - b0 + (uint32_t)sub - 1) / (uint32_t)sub);
-  const long long PS = (long long)p.Gu * p.grow;           // shared bytes between planes
-  const int stage_bytes = FI::PLANES * (int)PS;
+  const int PS = p.Gu * p.grow;                            // shared bytes between planes
+  const int stage_bytes = FI::PLANES * PS;
   const unsigned char* gsp = p.spins + sd.spin_off;
   const int L = sd.L, R_T = p.R_T;
 
   if (threadIdx.x == 0) {
     for (int k = 0; k < MS_STAGES; ++k) {
       mbar_init(&full[k], 1);
-      mbar_init(&empty[k], NW);
+      mbar_init(&empty[k], BS / 32);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  for (int x = threadIdx.x; x < L; x += blockDim.x) {
+  for (int x = threadIdx.x; x < L; x += BS) {
     float sn, cs;
     sincospif(2.0f * (float)x / (float)L, &sn, &cs);
     tw[x] = make_float2(cs, sn);
@@ -301,10 +308,11 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
   chain_wait();      // spins and permutations of the kernels before it from here on
   __syncthreads();
 
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) % NW, group = threadIdx.x / MEAS_BS;
+  const bool issuer = threadIdx.x < 32;
   // stage k of the run: sub-run k into buffer k % MS_STAGES, one copy per
-  // (plane, chunk group) row, issued by the lanes of warp 0 after lane 0 has
-  // announced the stage's bytes
+  // (plane, chunk group) row, issued by the lanes of the block's first warp after
+  // lane 0 has announced the stage's bytes
   const int rows = FI::PLANES * p.Gu;
   auto issue = [&](int k) {
     const int b = k % MS_STAGES;
@@ -315,12 +323,12 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
     unsigned char* dst = stage + b * stage_bytes;
     for (int row = lane; row < rows; row += 32) {
       const int pl = row / p.Gu, g = row - pl * p.Gu;
-      bulk_copy_g2s(dst + pl * PS + (long long)g * p.grow,
+      bulk_copy_g2s(dst + pl * PS + g * p.grow,
                     gsp + pl * sd.plane_stride + ((long long)g * N + ss0) * FI::CHUNK, bytes, &full[b]);
     }
   };
-  int issued = min(MS_STAGES, n_sub);   // stages issued so far (warp 0)
-  if (warp == 0)
+  int issued = min(MS_STAGES, n_sub);   // stages issued so far
+  if (issuer)
     for (int k = 0; k < issued; ++k) issue(k);
 
   // lanes: TL slots per site group, 32 / TL site groups per warp
@@ -338,18 +346,18 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
     off[r] = (w >> 2) * p.grow;
     jw[r] = w & 3;
   }
-  float a0[NQ];
-  float2 ak[NQ][3];
+  float a0[NQG];
+  float2 ak[NQG][3];
 #pragma unroll
-  for (int q = 0; q < NQ; ++q) {
+  for (int q = 0; q < NQG; ++q) {
     a0[q] = 0.0f;
 #pragma unroll
     for (int d = 0; d < 3; ++d) ak[q][d] = make_float2(0.0f, 0.0f);
   }
 
   // No block-wide barrier in the loop: a warp waits for a stage's copies
-  // (full) and, after its sites, arrives on the stage's empty barrier; warp 0
-  // refills a buffer once every warp has arrived.  Decisions on a wait that
+  // (full) and, after its sites, arrives on the stage's empty barrier; the first
+  // warp refills a buffer once every warp has arrived.  Decisions on a wait that
   // ran out are taken per warp, so a warp leaves the loop as a whole.
   bool ok = true;
   int k = 0;
@@ -363,41 +371,56 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
     const uint32_t ss0 = b0 + (uint32_t)k * (uint32_t)sub;
     const int n = (int)min((uint32_t)sub, b1 - ss0);
     const unsigned char* st = stage + b * stage_bytes;
-    for (int j = warp * SPW + grp; j < n; j += NW * SPW) {
-      const uint32_t ss = ss0 + (uint32_t)j;
+    // coordinates x | y << 10 | z << 20 of the stage's sites, lane l's for the l-th
+    // step of the warp's site group 0 and its neighbours: each site's division once,
+    // not once per slot (sub <= 64 sites: at most 64 / 32 rounds of 32 sites)
+    uint32_t xyz = 0;
+    auto locate = [&](int j) {
+      const uint32_t ss = ss0 + (uint32_t)min(j, n - 1);
       const uint32_t par = ss >= Nh ? 1u : 0u;
       const uint32_t h = ss - par * Nh;                                  // site >> 1
       const uint32_t r = (__umulhi(h, sd.fdLh_m) + h) >> sd.fdLh_s;       // h / (L / 2)
       const uint32_t zz = (__umulhi(r, sd.fdL_m) + r) >> sd.fdL_s;        // r / L
       const uint32_t y = r - zz * (uint32_t)L;
       const uint32_t x = 2u * (h - r * (uint32_t)sd.Lh) + ((par + y + zz) & 1u);
-      const float2 tk[3] = {tw[x], tw[y], tw[zz]};
-      if (!live) continue;
-      V3 S[NR];
-#pragma unroll
-      for (int rr = 0; rr < NR; ++rr)
-        decode_one<F>(st + off[rr] + j * FI::CHUNK, PS, jw[rr], S[rr].x, S[rr].y, S[rr].z);
-      float P[NQ];
+      return x | (y << 10) | (zz << 20);
+    };
+    // the warp's sites are warp * SPW + grp + i NW SPW; lane m holds site (m / SPW, m % SPW)
+    xyz = locate(warp * SPW + (lane % SPW) + (lane / SPW) * NW * SPW);
+    for (int i = 0, j = warp * SPW + grp; i * NW * SPW + warp * SPW < n; ++i, j += NW * SPW) {
+      const uint32_t c = __shfl_sync(0xffffffffu, xyz, i * SPW + grp);
+      if (!live || j >= n) continue;
+      const float2 tk[3] = {tw[c & 1023u], tw[(c >> 10) & 1023u], tw[c >> 20]};
+      const unsigned char* sj = st + j * FI::CHUNK;
+      float P[NQG];
       if constexpr (MODE == MEAS_QTENSOR) {
+        V3 S[2];
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr)
+          decode_one<F>(sj + off[rr], PS, jw[rr], S[rr].x, S[rr].y, S[rr].z);
         const float A[3] = {S[0].x, S[0].y, S[0].z}, B[3] = {S[1].x, S[1].y, S[1].z};
 #pragma unroll
         for (int mu = 0; mu < 3; ++mu)
 #pragma unroll
           for (int nu = 0; nu < 3; ++nu) P[3 * mu + nu] = __fmul_rn(A[mu], B[nu]);
       } else if constexpr (MODE == MEAS_CHIRAL) {
-        // the staged "spins" are the chiralities (kappa^x, kappa^y, kappa^z):
-        // per pair, in the pair order below, the three products kappa^a kappa^b
+        // the staged "spins" are the chiralities (kappa^x, kappa^y, kappa^z): per pair,
+        // in the pair order below, the product of component a = group
+        float K[NR];
+#pragma unroll
+        for (int rr = 0; rr < NR; ++rr)
+          K[rr] = reinterpret_cast<const float*>(sj + off[rr] + group * PS)[jw[rr]];
         int q = 0;
 #pragma unroll
         for (int bb = 1; bb < NR; ++bb)
 #pragma unroll
-          for (int aa = 0; aa < bb; ++aa) {
-            P[q++] = __fmul_rn(S[aa].x, S[bb].x);
-            P[q++] = __fmul_rn(S[aa].y, S[bb].y);
-            P[q++] = __fmul_rn(S[aa].z, S[bb].z);
-          }
+          for (int aa = 0; aa < bb; ++aa) P[q++] = __fmul_rn(K[aa], K[bb]);
       } else {
         // pairs in the order (0,1) (0,2) (1,2) (0,3) (1,3) (2,3)
+        V3 S[NR];
+#pragma unroll
+        for (int rr = 0; rr < NR; ++rr)
+          decode_one<F>(sj + off[rr], PS, jw[rr], S[rr].x, S[rr].y, S[rr].z);
         int q = 0;
 #pragma unroll
         for (int bb = 1; bb < NR; ++bb)
@@ -405,7 +428,7 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
           for (int aa = 0; aa < bb; ++aa) P[q++] = dot3(S[aa], S[bb]);
       }
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) {
+      for (int q = 0; q < NQG; ++q) {
         a0[q] = __fadd_rn(a0[q], P[q]);
 #pragma unroll
         for (int d = 0; d < 3; ++d) ak[q][d] = fma2(f2(P[q]), tk[d], ak[q][d]);
@@ -413,7 +436,7 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(&empty[b]);
-    if (warp == 0 && k + MS_STAGES < n_sub) {
+    if (issuer && k + MS_STAGES < n_sub) {
       if (!__all_sync(0xffffffffu, mbar_wait(&empty[b], ph, p.timeout_ns))) {
         ok = false;
         break;
@@ -427,7 +450,7 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
     // a wait ran out: flag it and give the copies this block issued a
     // bounded time to land; the block's partials are not used
     if (lane == 0) atomicExch(p.err, 1u);
-    if (warp == 0)
+    if (issuer)
       for (int q = k; q < issued; ++q)
         mbar_wait(&full[q % MS_STAGES], (uint32_t)(q / MS_STAGES) & 1u, p.timeout_ns);
   }
@@ -435,7 +458,7 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
   // site groups of a warp share slots: add them (fixed butterfly order)
   for (int o = TL; o < 32; o <<= 1) {
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
+    for (int q = 0; q < NQG; ++q) {
       a0[q] += __shfl_xor_sync(0xffffffffu, a0[q], o);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
@@ -444,44 +467,81 @@ __global__ void __launch_bounds__(MEAS_BS) k_meas_staged(const OverlapParams p) 
       }
     }
   }
-  // warps in order, FP32 (GB300's FP64 rate is a small fraction of its FP32
-  // rate); the block's sums leave as FP64
-  for (int w = 0; w < NW; ++w) {
-    if (warp == w && grp == 0 && live) {
+  // The warps of a group in order, FP32 (GB300's FP64 rate is a small fraction of
+  // its FP32 rate); the block's sums leave as FP64.  The stage buffers are free:
+  // `batch` warps at a time write their sums there ([warp][value][slot]), and each
+  // (value, slot) is then added by one thread, so that no warp waits for another's
+  // additions.  Sums so far: in registers of the thread that owns the (value, slot).
+  float* red = reinterpret_cast<float*>(stage);
+  const int per_warp = NV * nt;              // floats of one warp index (all groups)
+  const int batch = max(1, min(NW, p.red_floats / per_warp));
+  constexpr int OWN = (NV * 32 + BS - 1) / BS;
+  float sum[OWN];
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        float* rv = &red[q * NM][lane];
+  for (int m = 0; m < OWN; ++m) sum[m] = 0.0f;
+  for (int w0 = 0; w0 < NW; w0 += batch) {
+    __syncthreads();
+    if (warp >= w0 && warp < w0 + batch && grp == 0 && live) {
+#pragma unroll
+      for (int q = 0; q < NQG; ++q) {
+        // product index in the output order (chiral: pair * 3 + component)
+        const int gq = MODE == MEAS_CHIRAL ? q * 3 + group : q;
+        float* rv = red + (warp - w0) * per_warp + gq * NM * nt + tl;
         const float v[NM] = {a0[q], ak[q][0].x, ak[q][0].y, ak[q][1].x, ak[q][1].y, ak[q][2].x, ak[q][2].y};
 #pragma unroll
-        for (int m = 0; m < NM; ++m) rv[m * 32] = (w == 0 ? 0.0f : rv[m * 32]) + v[m];
+        for (int m = 0; m < NM; ++m) rv[m * nt] = v[m];
       }
     }
     __syncthreads();
+#pragma unroll
+    for (int m = 0; m < OWN; ++m) {
+      const int i = (int)threadIdx.x + m * BS;
+      if (i < per_warp)
+        for (int w = 0; w < min(batch, NW - w0); ++w) sum[m] += red[w * per_warp + i];
+    }
   }
+  // partials [value][slot of the round] of this block
   double* out = p.partials + (((long long)s * p.n_tiles + blockIdx.x) * R_T + 32 * round) * NV;
-  for (int i = threadIdx.x; i < nt * NV; i += MEAS_BS) out[i] = (double)red[i % NV][i / NV];
+#pragma unroll
+  for (int m = 0; m < OWN; ++m) {
+    const int i = (int)threadIdx.x + m * BS;
+    if (i < per_warp) out[i] = (double)sum[m];
+  }
 }
 
-// One warp per (sample, slot, value): lane l adds the partials of blocks
-// l, l + 32, ... in that order, then the lanes are added in a fixed butterfly;
-// the total times 1/N.  Eight values per block of 256 threads.
+// The blocks' partials of one (sample, round of slots), FP64: a block adds 32
+// consecutive columns (value, slot) with 32 lanes of blocks each (lane l adds
+// blocks l, l + 32, ... in that order), then the lanes in order; the total times
+// 1/N.  (Columns are contiguous in a block's partials, so a warp reads 256
+// consecutive bytes.)
+constexpr int MF_ROWS = 32;
 template <int MODE>
-__global__ void __launch_bounds__(256) k_meas_final_staged(const OverlapParams p, int NV) {
+__global__ void __launch_bounds__(32 * MF_ROWS) k_meas_final_staged(const OverlapParams p, int NV) {
+  __shared__ double red[MF_ROWS][33];
   chain_trigger();
-  chain_wait();
-  const int t = blockIdx.x % p.R_T, s = blockIdx.x / p.R_T;
-  const int v = blockIdx.y * 8 + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (v >= NV) return;
+  const int s = blockIdx.z, round = blockIdx.y;
+  const int nt = min(32, p.R_T - 32 * round);
+  const int col = blockIdx.x * 32 + (threadIdx.x & 31), row = threadIdx.x >> 5;
   const SampleDev& sd = p.samples[s];
   const int n_tiles = (int)(((long long)sd.N + p.tile_ss - 1) / p.tile_ss);
   const long long stride = (long long)p.R_T * NV;
-  const double* src = p.partials + ((long long)s * p.n_tiles * p.R_T + t) * NV + v;
+  chain_wait();
   double acc = 0.0;
+  if (col < nt * NV) {
+    const double* src = p.partials + (long long)s * p.n_tiles * stride + (long long)32 * round * NV + col;
 #pragma unroll 4
-  for (int k = lane; k < n_tiles; k += 32) acc += src[k * stride];
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane != 0) return;
-  const double val = acc / (double)sd.N;
+    for (int k = row; k < n_tiles; k += MF_ROWS) acc += src[k * stride];
+  }
+  red[row][threadIdx.x & 31] = acc;
+  __syncthreads();
+  // warp w adds columns w: lanes hold the rows
+  const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double val = red[lane][c];
+  for (int o = 16; o > 0; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
+  const int mine = blockIdx.x * 32 + c;
+  if (lane != 0 || mine >= nt * NV) return;
+  val /= (double)sd.N;
+  const int v = mine / nt, t = 32 * round + mine % nt;
   const int q = v / NM, m = v % NM;
   if constexpr (MODE == MEAS_QTENSOR) {
     if (m == 0) {
@@ -506,16 +566,21 @@ __global__ void __launch_bounds__(256) k_meas_final_staged(const OverlapParams p
 }
 
 template <int F, int MODE, int NR>
-static cudaError_t staged_launch(const OverlapParams& p, cudaStream_t st) {
+static cudaError_t staged_launch(OverlapParams p, cudaStream_t st) {
   constexpr int NV = staged_products<MODE, NR>() * NM;
-  const int smem = MS_STAGES * FmtInfo<F>::PLANES * p.Gu * p.grow;
+  // the stages, or at least one warp's sums for the block's reduction
+  const int stages = MS_STAGES * FmtInfo<F>::PLANES * p.Gu * p.grow;
+  const int smem = max(stages, NV * 32 * (int)sizeof(float));
+  p.red_floats = smem / (int)sizeof(float);
   cudaError_t e = cudaFuncSetAttribute(k_meas_staged<F, MODE, NR>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const dim3 grid(p.n_tiles, (p.R_T + 31) / 32, p.n_samples);
-  e = launch_chained(k_meas_staged<F, MODE, NR>, grid, MEAS_BS, smem, st, p);
+  const int rounds = (p.R_T + 31) / 32;
+  e = launch_chained(k_meas_staged<F, MODE, NR>, dim3(p.n_tiles, rounds, p.n_samples),
+                     MEAS_BS * staged_groups<MODE>(), smem, st, p);
   if (e != cudaSuccess) return e;
-  return launch_chained(k_meas_final_staged<MODE>, dim3(p.n_samples * p.R_T, (NV + 7) / 8), 256, 0, st, p, NV);
+  return launch_chained(k_meas_final_staged<MODE>, dim3((min(32, p.R_T) * NV + 31) / 32, rounds, p.n_samples),
+                        32 * MF_ROWS, 0, st, p, NV);
 }
 
 template <int F, int MODE>
