@@ -509,19 +509,19 @@ __global__ void __launch_bounds__(MEAS_BS * staged_groups<MODE>()) k_meas_staged
   }
 }
 
-// The blocks' partials of one (sample, round of slots), FP64: a block adds 32
-// consecutive columns (value, slot) with 32 lanes of blocks each (lane l adds
-// blocks l, l + 32, ... in that order), then the lanes in order; the total times
-// 1/N.  (Columns are contiguous in a block's partials, so a warp reads 256
-// consecutive bytes.)
-constexpr int MF_ROWS = 32;
+// The blocks' partials of one (sample, round of slots), FP64: a block adds MF_COLS
+// consecutive columns (value, slot) with 32 lanes of tiles each (lane l adds tiles
+// l, l + 32, ... in that order), then the lanes in a fixed butterfly; the total times
+// 1/N.  Columns are contiguous in a tile's partials.  Bound by the FP64 additions (two
+// a clock and SM), so the columns are spread over as many SMs as there are.
+constexpr int MF_ROWS = 32, MF_COLS = 8;
 template <int MODE>
-__global__ void __launch_bounds__(32 * MF_ROWS) k_meas_final_staged(const OverlapParams p, int NV) {
-  __shared__ double red[MF_ROWS][33];
+__global__ void __launch_bounds__(MF_COLS * MF_ROWS) k_meas_final_staged(const OverlapParams p, int NV) {
+  __shared__ double red[MF_ROWS][MF_COLS + 1];
   chain_trigger();
   const int s = blockIdx.z, round = blockIdx.y;
   const int nt = min(32, p.R_T - 32 * round);
-  const int col = blockIdx.x * 32 + (threadIdx.x & 31), row = threadIdx.x >> 5;
+  const int col = blockIdx.x * MF_COLS + threadIdx.x % MF_COLS, row = threadIdx.x / MF_COLS;
   const SampleDev& sd = p.samples[s];
   const int n_tiles = (int)(((long long)sd.N + p.tile_ss - 1) / p.tile_ss);
   const long long stride = (long long)p.R_T * NV;
@@ -529,16 +529,23 @@ __global__ void __launch_bounds__(32 * MF_ROWS) k_meas_final_staged(const Overla
   double acc = 0.0;
   if (col < nt * NV) {
     const double* src = p.partials + (long long)s * p.n_tiles * stride + (long long)32 * round * NV + col;
-#pragma unroll 4
-    for (int k = row; k < n_tiles; k += MF_ROWS) acc += src[k * stride];
+    int k = row;
+    for (; k + 11 * MF_ROWS < n_tiles; k += 12 * MF_ROWS) {   // twelve loads in flight
+      double v[12];
+#pragma unroll
+      for (int u = 0; u < 12; ++u) v[u] = src[(k + u * MF_ROWS) * stride];
+#pragma unroll
+      for (int u = 0; u < 12; ++u) acc += v[u];
+    }
+    for (; k < n_tiles; k += MF_ROWS) acc += src[k * stride];
   }
-  red[row][threadIdx.x & 31] = acc;
+  red[row][threadIdx.x % MF_COLS] = acc;
   __syncthreads();
-  // warp w adds columns w: lanes hold the rows
+  // warp c adds column c: lanes hold the rows
   const int c = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double val = red[lane][c];
   for (int o = 16; o > 0; o >>= 1) val += __shfl_xor_sync(0xffffffffu, val, o);
-  const int mine = blockIdx.x * 32 + c;
+  const int mine = blockIdx.x * MF_COLS + c;
   if (lane != 0 || mine >= nt * NV) return;
   val /= (double)sd.N;
   const int v = mine / nt, t = 32 * round + mine % nt;
@@ -579,8 +586,8 @@ static cudaError_t staged_launch(OverlapParams p, cudaStream_t st) {
   e = launch_chained(k_meas_staged<F, MODE, NR>, dim3(p.n_tiles, rounds, p.n_samples),
                      MEAS_BS * staged_groups<MODE>(), smem, st, p);
   if (e != cudaSuccess) return e;
-  return launch_chained(k_meas_final_staged<MODE>, dim3((min(32, p.R_T) * NV + 31) / 32, rounds, p.n_samples),
-                        32 * MF_ROWS, 0, st, p, NV);
+  return launch_chained(k_meas_final_staged<MODE>, dim3((min(32, p.R_T) * NV + MF_COLS - 1) / MF_COLS, rounds, p.n_samples),
+                        MF_COLS * MF_ROWS, 0, st, p, NV);
 }
 
 template <int F, int MODE>
@@ -632,7 +639,7 @@ static cudaError_t meas_dispatch(int fmt, const OverlapParams& p, int mode, cuda
 // launch per parity over the sweep block table; a thread owns one site and
 // walks its chunk groups, as the sweeps do.
 template <int F>
-__global__ void __launch_bounds__(SWEEP_BS) k_chirality(const ChiralityParams p) {
+__global__ void __launch_bounds__(SWEEP_BS, F == FMT_YX4 || F == FMT_F32 ? 0 : 4) k_chirality(const ChiralityParams p) {
   constexpr int VEC = 4, PL = FmtInfo<F>::PLANES;
   using Chunk = typename FmtInfo<F>::Chunk;
   chain_trigger();
@@ -649,19 +656,20 @@ __global__ void __launch_bounds__(SWEEP_BS) k_chirality(const ChiralityParams p)
   const SampleDev& kd = p.ksamples[blk.x];
   unsigned char* kb = p.kappa + kd.spin_off;
   const long long kps = kd.plane_stride;
+  constexpr uint32_t CH = FmtInfo<F>::CHUNK;
   for (int g = g0; g < g1; ++g) {
-    Chunk c[PL];
-    load_chunks<F, LD_PLAIN>(base + chunk_offset<F>(sd, g, gm.own), ps, c);
+    const unsigned char* base_g = base + (long long)g * sd.N * CH;
+    Chunk c[PL], nc[6][PL];
+    load_chunks_at<F, LD_PLAIN>(base_g, ps, gm.own * CH, c);
+#pragma unroll
+    for (int n = 0; n < 6; ++n) load_chunks_at<F, LD_PLAIN>(base_g, ps, gm.nb[n] * CH, nc[n]);
     Spins<VEC> s0;
     decode<F>(c, s0);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      Chunk cp[PL], cm[PL];
-      load_chunks<F, LD_PLAIN>(base + chunk_offset<F>(sd, g, gm.nb[2 * a]), ps, cp);
-      load_chunks<F, LD_PLAIN>(base + chunk_offset<F>(sd, g, gm.nb[2 * a + 1]), ps, cm);
       Spins<VEC> sp, sm;
-      decode<F>(cp, sp);
-      decode<F>(cm, sm);
+      decode<F>(nc[2 * a], sp);
+      decode<F>(nc[2 * a + 1], sm);
       float k4[VEC];
 #pragma unroll
       for (int v = 0; v < VEC; ++v) {

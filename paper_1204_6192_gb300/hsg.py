@@ -270,7 +270,8 @@ class Context:
         """Replica-pair overlaps D [ns, R_T, P, 4, 2] and chiral overlaps
         C [ns, R_T, P, 3, 4, 2] (modes k = 0, kx, ky, kz; re, im) for the P pairs
         (0,1) (0,2) (1,2) (0,3) (1,3) (2,3) of the first min(R_O, 4) replicas."""
-        P = self.info().n_overlap_pairs
+        r = min(self.n_replicas, 4)
+        P = r * (r - 1) // 2
         ns, R_T = self.n_samples, self.n_temps
         D = np.zeros((ns, R_T, P, 4, 2)) if spin else None
         C = np.zeros((ns, R_T, P, 3, 4, 2)) if chiral else None
