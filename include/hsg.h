@@ -147,7 +147,11 @@ enum {
   HSG_SWEEP_HALF = 1,         /* one launch per half-sweep */
   HSG_SWEEP_FUSED = 2,        /* one launch per sweep through shared memory (pairs of OR sweeps) */
   HSG_SWEEP_WAVE = 3,         /* one launch per sweep, odd blocks trailing even blocks in L2 */
-  HSG_SWEEP_STAGED = 4        /* one launch per half-sweep, neighbour rows staged in shared memory */
+  HSG_SWEEP_STAGED = 4,       /* one launch per half-sweep, neighbour rows staged in shared memory */
+  HSG_SWEEP_RESIDENT = 5      /* hsg_info only (not an option): hsg_step runs all sweeps of a step in
+                                 one launch, each pair of systems in the shared memory of one block;
+                                 where every L <= 12 and no sweep kernel, pass footprint or chunks
+                                 per thread is asked for.  hsg_sweep_or then uses HSG_SWEEP_HALF. */
 };
 
 enum {

@@ -136,6 +136,10 @@ struct hsg_ctx {
   unsigned int* d_wave_flags = nullptr; // [max_sweep_blocks] completion flags of the even blocks
   unsigned int* d_wave_state = nullptr; // tickets taken, blocks finished, epoch
 
+  // resident sweeps: all sweeps of a step in one launch, each pair of systems in
+  // the shared memory of one block
+  bool use_resident = false;            // resolved choice of the schedule
+
   std::vector<int> pass_bound{0, 0};    // [n_passes + 1] block table bounds
   int* d_pass_bound = nullptr;
   long long pass_bytes = 0;             // resolved footprint bound (0: one pass)
@@ -539,12 +543,40 @@ hsg_status or_sweeps(hsg_ctx* c, int n, int sweep_offset) {
   return HSG_OK;
 }
 
+// All sweeps of a step, and the energies of its final state (n_or > 0).
+hsg_status resident_sweeps(hsg_ctx* c) {
+  const SweepParams sp = sweep_params(c, 0, 0);
+  ResidentParams p{};
+  p.spins = c->spins;
+  p.rec = c->rec;
+  p.samples = c->d_sd;
+  p.beta = c->d_beta;
+  p.counters = c->d_counters;
+  p.active = c->d_active;
+  p.E = c->d_E;
+  p.n_samples = c->ns;
+  p.n_pairs = c->Wp / 2;
+  p.Wp = c->Wp;
+  p.n_hb = c->opt.n_hb_per_step;
+  p.n_or = c->opt.n_or_per_step;
+  p.max_half_sites = c->Lmax * c->Lmax * c->Lmax / 2;
+  for (int r = 0; r < 20; ++r) p.rk[r] = sp.rk[r];
+  HSG_CUDA(c, launch_resident(c->fmt, c->j16, c->opt.fast_math != 0, p, c->stream));
+  return HSG_OK;
+}
+
 // A step: n_hb HB sweeps, n_or OR sweeps (the last one also produces the
 // energy partials of the final state), the energy sums and one PT pass.  The
 // sweeps run pass by pass; systems are independent and every random number is
 // keyed by (site, system, sweep), so the order of the passes changes nothing.
 hsg_status enqueue_step(hsg_ctx* c) {
   const int nhb = c->opt.n_hb_per_step, nor = c->opt.n_or_per_step;
+  if (c->use_resident) {
+    HSG_TRY(resident_sweeps(c));
+    if (nor == 0) return enqueue_energy(c, true, nhb);
+    HSG_CUDA(c, launch_pt(pt_params(c, nhb + nor), c->stream));
+    return HSG_OK;
+  }
   const int np = (int)c->pass_bound.size() - 1;
   for (int ps = 0; ps < np; ++ps) {
     const int b0 = c->pass_bound[ps], b1 = c->pass_bound[ps + 1];
@@ -852,6 +884,7 @@ hsg_status configure_schedule(hsg_ctx* c, int variant, int gpt, long long pass_b
     HSG_TRY(plan_wave(c, blocks, lag));
     c->use_wave = true;
   }
+  c->use_resident = sweep == HSG_SWEEP_RESIDENT && variant == HSG_VARIANT_TWO_PASS;
   if (variant == HSG_VARIANT_PERSISTENT) {
     c->persist_smem = sizeof(float) * (SWEEP_BS / 32) * c->GPT * c->VEC;
     int max_grid = 0;
@@ -924,6 +957,15 @@ hsg_status copy_chain_state(hsg_ctx* c, unsigned char* host, bool to_host) {
     off += r.second;
   }
   return HSG_OK;
+}
+
+// Whether the resident sweeps can serve hsg_step: every lattice within a block's
+// threads, some sweeps, and no sweep kernel, pass footprint or chunks per thread
+// asked for.
+bool resident_possible(const hsg_ctx* c) {
+  return c->Lmax * c->Lmax * c->Lmax / 2 <= RES_MAX_HALF_SITES &&
+         c->opt.n_hb_per_step + c->opt.n_or_per_step > 0 && c->opt.sweep_kernel == HSG_SWEEP_AUTO &&
+         c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0;
 }
 
 // Autotuner: the schedules, sweep kernels and chunks-per-thread settings
@@ -999,6 +1041,8 @@ hsg_status autotune(hsg_ctx* c) {
   }
   if ((sk == HSG_SWEEP_AUTO || sk == HSG_SWEEP_STAGED) && c->staged_possible)
     sweeps.push_back({HSG_SWEEP_STAGED, 0});
+  const int gpt0 = c->GPT;
+  if (resident_possible(c)) sweeps.push_back({HSG_SWEEP_RESIDENT, 0});
   if (sweeps.empty()) sweeps.push_back({HSG_SWEEP_HALF, 0});
   cudaEvent_t e0, e1;
   HSG_CUDA(c, cudaEventCreate(&e0));
@@ -1025,8 +1069,9 @@ hsg_status autotune(hsg_ctx* c) {
         // the fused sweep runs in the two-pass schedule with one pass only, the
         // wave sweep in the two-pass schedule; the persistent schedule has its own
         if (sw.first != HSG_SWEEP_HALF && v != HSG_VARIANT_TWO_PASS) continue;
-        if (sw.first == HSG_SWEEP_FUSED && pb != 0) continue;
+        if ((sw.first == HSG_SWEEP_FUSED || sw.first == HSG_SWEEP_RESIDENT) && pb != 0) continue;
         for (int g : gpts) {
+          if (sw.first == HSG_SWEEP_RESIDENT && g != gpt0) continue;   // (no use of it there)
           HSG_TRY(configure_schedule(c, v, g, pb, sw.first, sw.second));
           if (sw.first == HSG_SWEEP_FUSED && !c->use_fused) continue;
           HSG_TRY(run_steps(c, 1));
@@ -1359,7 +1404,10 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
       c->staged_possible = c->staged_possible && lattice_has_staged(L[s]);
       c->Lh_max = std::max(c->Lh_max, L[s] / 2);
     }
-    const int sweep = opt.sweep_kernel == HSG_SWEEP_AUTO ? HSG_SWEEP_HALF : opt.sweep_kernel;
+    int sweep = opt.sweep_kernel == HSG_SWEEP_AUTO ? HSG_SWEEP_HALF : opt.sweep_kernel;
+    // the two-pass schedule as an explicit choice: resident where possible (the
+    // tuner, for an automatic one, times it against the others)
+    if (opt.variant == HSG_VARIANT_TWO_PASS && resident_possible(c)) sweep = HSG_SWEEP_RESIDENT;
     hsg_status st2 = configure_schedule(c, want, c->GPT, opt.pass_bytes, sweep, opt.wave_lag);
     if (st2 != HSG_OK) return cleanup_fail(st2);
   }
@@ -1936,7 +1984,8 @@ hsg_status hsg_get_info(hsg_ctx* c, hsg_info* info) {
   info->sweep_count = cnt[0];
   info->pt_count = cnt[1];
   info->stream = (void*)c->stream;
-  info->sweep_kernel = c->use_wave ? HSG_SWEEP_WAVE
+  info->sweep_kernel = c->use_resident ? HSG_SWEEP_RESIDENT
+                      : c->use_wave ? HSG_SWEEP_WAVE
                       : c->use_staged ? HSG_SWEEP_STAGED
                       : (c->use_fused ? HSG_SWEEP_FUSED : HSG_SWEEP_HALF);
   info->staged = (c->use_wave && c->staged_possible) || c->use_staged;

@@ -282,6 +282,24 @@ cudaError_t launch_wave(int fmt, bool j16, bool energy, bool staged, const WaveP
 cudaError_t launch_staged_half(int fmt, bool j16, bool energy, const SweepParams& p, int n_blocks,
                                size_t smem, cudaStream_t st);
 
+// The sweeps of a step with a pair of systems' lattice resident in a block's shared
+// memory (hsg_resident.cu), for lattices of at most RES_MAX_HALF_SITES sites of a parity.
+constexpr int RES_MAX_HALF_SITES = 896;   // L <= 12: 864
+struct ResidentParams {
+  unsigned char* spins;
+  const void* rec;
+  const SampleDev* samples;
+  const float* beta;        // [n_samples][Wp]
+  const unsigned long long* counters;   // [n_samples][2]: sweeps done, PT passes done
+  const unsigned char* active;          // [n_samples]
+  double* E;                // [n_samples][Wp]: energies of the final state (n_or > 0)
+  int n_samples, n_pairs;   // pairs of systems per sample (Wp / 2)
+  int Wp, n_hb, n_or;
+  int max_half_sites;       // of the context's largest lattice
+  uint32_t rk[20];          // Philox round keys of the seed
+};
+cudaError_t launch_resident(int fmt, bool j16, bool fast, const ResidentParams& p, cudaStream_t st);
+
 // The packed spin formats (one or two 32-bit words per system) decode each
 // neighbour spin once into a binary32 buffer before a half-sweep instead of
 // at every one of its six uses.
