@@ -141,6 +141,12 @@ struct hsg_ctx {
   bool use_resident = false;            // resolved choice of the schedule
 
   std::vector<int> pass_bound{0, 0};    // [n_passes + 1] block table bounds
+  // passes of a step on two branches of its graph (chains = 2), the odd ones on
+  // `side`: systems meet only in the PT pass, so while one branch's launch drains,
+  // the other's fills the GPU
+  int chains = 1;
+  cudaStream_t side = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int* d_pass_bound = nullptr;
   long long pass_bytes = 0;             // resolved footprint bound (0: one pass)
   int max_passes = 1;
@@ -565,6 +571,16 @@ hsg_status resident_sweeps(hsg_ctx* c) {
   return HSG_OK;
 }
 
+// The context's launches go to another stream while this object lives.
+struct OnStream {
+  hsg_ctx* c;
+  cudaStream_t own;
+  OnStream(hsg_ctx* ctx, cudaStream_t st) : c(ctx), own(ctx->stream) { c->stream = st; }
+  ~OnStream() { c->stream = own; }
+  OnStream(const OnStream&) = delete;
+  OnStream& operator=(const OnStream&) = delete;
+};
+
 // A step: n_hb HB sweeps, n_or OR sweeps (the last one also produces the
 // energy partials of the final state), the energy sums and one PT pass.  The
 // sweeps run pass by pass; systems are independent and every random number is
@@ -578,8 +594,17 @@ hsg_status enqueue_step(hsg_ctx* c) {
     return HSG_OK;
   }
   const int np = (int)c->pass_bound.size() - 1;
+  const bool fork = c->chains == 2 && np > 1;
+  if (fork) {
+    if (!c->side) HSG_CUDA(c, cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
+    if (!c->ev_fork) HSG_CUDA(c, cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
+    if (!c->ev_join) HSG_CUDA(c, cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
+    HSG_CUDA(c, cudaEventRecord(c->ev_fork, c->stream));
+    HSG_CUDA(c, cudaStreamWaitEvent(c->side, c->ev_fork, 0));
+  }
   for (int ps = 0; ps < np; ++ps) {
     const int b0 = c->pass_bound[ps], b1 = c->pass_bound[ps + 1];
+    const OnStream branch(c, fork && (ps & 1) ? c->side : c->stream);
     c->dec_fresh = false;
     for (int k = 0; k < nhb; ++k) HSG_TRY(half_sweeps(c, true, k, false, b0, b1));
     int k = 0;
@@ -592,6 +617,10 @@ hsg_status enqueue_step(hsg_ctx* c) {
       c->dec_fresh = false;
     }
     for (; k < nor; ++k) HSG_TRY(half_sweeps(c, false, nhb + k, k == nor - 1, b0, b1));
+  }
+  if (fork) {
+    HSG_CUDA(c, cudaEventRecord(c->ev_join, c->side));
+    HSG_CUDA(c, cudaStreamWaitEvent(c->stream, c->ev_join, 0));
   }
   if (nor > 0) {
     HSG_CUDA(c, launch_energy_sums_pt(energy_params(c), pt_params(c, nhb + nor), c->stream));
@@ -817,7 +846,7 @@ hsg_status plan_wave(hsg_ctx* c, const std::vector<int4>& blocks, int lag) {
 // chunk group), and set up the chosen step schedule (drops a captured graph:
 // its parameters change).
 hsg_status configure_schedule(hsg_ctx* c, int variant, int gpt, long long pass_bytes, int sweep,
-                              int lag) {
+                              int lag, int chains = 1) {
   gpt = std::max(1, std::min(c->G, gpt));
   const int n_gg = (c->G + gpt - 1) / gpt;
   const long long site_chunk_bytes = (long long)c->PL * c->VEC * c->ELEM;
@@ -871,6 +900,7 @@ hsg_status configure_schedule(hsg_ctx* c, int variant, int gpt, long long pass_b
     c->graph = nullptr;
   }
   c->variant = variant;
+  c->chains = chains;
   // the fused over-relaxation sweep serves the two-pass schedule in one pass,
   // the wave sweep the two-pass schedule with any passes
   c->use_fused = false;
@@ -978,7 +1008,7 @@ bool resident_possible(const hsg_ctx* c) {
 struct TuneChoice {
   int variant, gpt;
   long long pass_bytes;
-  int sweep, lag;
+  int sweep, lag, chains;
 };
 constexpr int TUNE_REPS = 5;
 std::mutex g_tune_mu;
@@ -1003,7 +1033,7 @@ hsg_status autotune(hsg_ctx* c) {
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end())
       return configure_schedule(c, it->second.variant, it->second.gpt, it->second.pass_bytes,
-                                it->second.sweep, it->second.lag);
+                                it->second.sweep, it->second.lag, it->second.chains);
   }
   // save the state the trial steps will change
   void* spins_copy = nullptr;
@@ -1062,7 +1092,32 @@ hsg_status autotune(hsg_ctx* c) {
     }
   }
   float best = 1e30f;
-  TuneChoice bestc{HSG_VARIANT_TWO_PASS, c->GPT, budgets[0], sweeps[0].first, sweeps[0].second};
+  TuneChoice bestc{HSG_VARIANT_TWO_PASS, c->GPT, budgets[0], sweeps[0].first, sweeps[0].second, 1};
+  // one warm-up step, then the median of TUNE_REPS timings of two steps; a
+  // candidate replaces the current choice only when it is at least 1% faster, so that
+  // timing noise between near-equal candidates does not decide (candidates are tried
+  // simplest first)
+  auto time_candidate = [&](const TuneChoice& t) -> hsg_status {
+    HSG_TRY(configure_schedule(c, t.variant, t.gpt, t.pass_bytes, t.sweep, t.lag, t.chains));
+    if (t.sweep == HSG_SWEEP_FUSED && !c->use_fused) return HSG_OK;
+    if (t.chains > 1 && c->pass_bound.size() < 3) return HSG_OK;
+    HSG_TRY(run_steps(c, 1));
+    float ms[TUNE_REPS];
+    for (int r = 0; r < TUNE_REPS; ++r) {
+      HSG_CUDA(c, cudaEventRecord(e0, st));
+      HSG_TRY(run_steps(c, 2));
+      HSG_CUDA(c, cudaEventRecord(e1, st));
+      HSG_CUDA(c, cudaEventSynchronize(e1));
+      HSG_CUDA(c, cudaEventElapsedTime(&ms[r], e0, e1));
+    }
+    HSG_TRY(poll_device_error(c));
+    std::sort(ms, ms + TUNE_REPS);
+    if (ms[TUNE_REPS / 2] < best * 0.99f) {
+      best = ms[TUNE_REPS / 2];
+      bestc = t;
+    }
+    return HSG_OK;
+  };
   for (long long pb : budgets) {
     for (int v : {HSG_VARIANT_TWO_PASS, HSG_VARIANT_PERSISTENT}) {
       for (const auto& sw : sweeps) {
@@ -1072,30 +1127,21 @@ hsg_status autotune(hsg_ctx* c) {
         if ((sw.first == HSG_SWEEP_FUSED || sw.first == HSG_SWEEP_RESIDENT) && pb != 0) continue;
         for (int g : gpts) {
           if (sw.first == HSG_SWEEP_RESIDENT && g != gpt0) continue;   // (no use of it there)
-          HSG_TRY(configure_schedule(c, v, g, pb, sw.first, sw.second));
-          if (sw.first == HSG_SWEEP_FUSED && !c->use_fused) continue;
-          HSG_TRY(run_steps(c, 1));
-          float t[TUNE_REPS];
-          for (int r = 0; r < TUNE_REPS; ++r) {
-            HSG_CUDA(c, cudaEventRecord(e0, st));
-            HSG_TRY(run_steps(c, 2));
-            HSG_CUDA(c, cudaEventRecord(e1, st));
-            HSG_CUDA(c, cudaEventSynchronize(e1));
-            HSG_CUDA(c, cudaEventElapsedTime(&t[r], e0, e1));
-          }
-          HSG_TRY(poll_device_error(c));
-          std::sort(t, t + TUNE_REPS);
-          const float ms = t[TUNE_REPS / 2];
-          // a candidate replaces the current choice only when it is at least
-          // 1% faster, so that timing noise between near-equal candidates does
-          // not decide (candidates are tried simplest first)
-          if (ms < best * 0.99f) {
-            best = ms;
-            bestc = TuneChoice{v, g, pb, sw.first, sw.second};
-          }
+          HSG_TRY(time_candidate({v, g, pb, sw.first, sw.second, 1}));
         }
       }
     }
+  }
+  // the half-sweeps in passes on two branches of the step's graph: halves of the
+  // systems, and the footprints above (two passes in flight)
+  if (c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 && bestc.variant == HSG_VARIANT_TWO_PASS &&
+      bestc.sweep == HSG_SWEEP_HALF) {
+    std::vector<int> near;
+    for (int g : {bestc.gpt, (bestc.gpt + 1) / 2, 2 * bestc.gpt})
+      if (g <= c->G && std::find(near.begin(), near.end(), g) == near.end()) near.push_back(g);
+    budgets[0] = (long long)(c->spin_bytes + 1) / 2 + (long long)c->rec_bytes;
+    for (long long pb : budgets)
+      for (int g : near) HSG_TRY(time_candidate({HSG_VARIANT_TWO_PASS, g, pb, HSG_SWEEP_HALF, 0, 2}));
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1109,7 +1155,7 @@ hsg_status autotune(hsg_ctx* c) {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     g_tune_cache[key] = bestc;
   }
-  return configure_schedule(c, bestc.variant, bestc.gpt, bestc.pass_bytes, bestc.sweep, bestc.lag);
+  return configure_schedule(c, bestc.variant, bestc.gpt, bestc.pass_bytes, bestc.sweep, bestc.lag, bestc.chains);
 }
 
 hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double* temps,
@@ -2057,6 +2103,9 @@ void hsg_destroy(hsg_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
   if (c->graph) cudaGraphDestroy(c->graph);
+  if (c->side) cudaStreamDestroy(c->side);
+  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  if (c->ev_join) cudaEventDestroy(c->ev_join);
   for (void* p : c->allocations) cudaFree(p);
   if (c->results) cudaFreeHost(c->results);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
