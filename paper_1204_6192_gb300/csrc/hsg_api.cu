@@ -345,6 +345,7 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
                        int b1 = -1) {
   if (b1 < 0) b1 = c->n_sweep_blocks;
   if (!hb && c->use_staged) {
+    const bool one_L = std::all_of(c->L.begin(), c->L.end(), [&](int L) { return L == c->L[0]; });
     int off = 0;
     const size_t smem = staged_smem(c->fmt, c->GPT, energy, c->Lh_max, &off);
     for (int parity = 0; parity < 2; ++parity) {
@@ -353,7 +354,8 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
       p.n_launch = b1 - b0;
       p.reverse = parity;
       p.stage_off = off;
-      HSG_CUDA(c, launch_staged_half(c->fmt, c->j16, energy, p, b1 - b0, smem, c->stream));
+      HSG_CUDA(c, launch_staged_half(c->fmt, c->j16, energy, one_L ? c->Lh_max : 0, p, b1 - b0, smem,
+                                     c->stream));
     }
     return HSG_OK;
   }

@@ -87,7 +87,7 @@ struct SweepParams {
   uint32_t rk[20];          // Philox round keys of the seed
   const unsigned char* dec; // packed formats: the opposite parity as binary32 (see SampleDev)
   unsigned char* dec_out;   // packed formats: where the updated spins go as binary32 (null: nowhere)
-  // staged sweeps (hsg_wave.cu): bytes of one stage of neighbour rows, offset of
+  // staged sweeps (hsg_wave.cu): bytes of one stage of rows, offset of
   // stage 0 in dynamic shared memory, the error word of their bounded waits
   int stage_bytes, stage_off;
   unsigned int* err;
@@ -267,10 +267,10 @@ struct WaveParams {
 bool fmt_has_wave(int fmt);
 // Staged sweeps: every block copies the opposite-parity rows its sites read
 // (plane z: rows y0-1 .. y0+R, planes z-1 and z+1: rows y0 .. y0+R-1; R = 256 /
-// (L/2)) into a two-stage shared-memory ring with cp.async.bulk, one chunk group
+// (L/2)) and its own rows into a two-stage shared-memory ring with cp.async.bulk, one chunk group
 // per stage.  Possible for every sample with L a power of 2, L >= 32.
 constexpr int STAGED_STAGES = 2;
-constexpr int STAGED_HEAD = 256;          // mbarriers and stage counters
+constexpr int STAGED_HEAD = 256;          // mbarriers
 bool lattice_has_staged(int L);
 int staged_stage_bytes(int fmt, int Lh_max);
 size_t staged_smem(int fmt, int gpt, bool energy, int Lh_max, int* stage_off);
@@ -278,8 +278,9 @@ size_t staged_smem(int fmt, int gpt, bool energy, int Lh_max, int* stage_off);
 cudaError_t wave_occupancy(int fmt, bool j16, bool staged, size_t smem, int* blocks_per_sm);
 cudaError_t launch_wave(int fmt, bool j16, bool energy, bool staged, const WaveParams& p, size_t smem,
                         cudaStream_t st);
-// one half-sweep (p.parity) of over-relaxation with the staged block body
-cudaError_t launch_staged_half(int fmt, bool j16, bool energy, const SweepParams& p, int n_blocks,
+// one half-sweep (p.parity) of over-relaxation with the staged block body; Lh: L / 2 if
+// every sample has the same, else 0
+cudaError_t launch_staged_half(int fmt, bool j16, bool energy, int Lh, const SweepParams& p, int n_blocks,
                                size_t smem, cudaStream_t st);
 
 // The sweeps of a step with a pair of systems' lattice resident in a block's shared

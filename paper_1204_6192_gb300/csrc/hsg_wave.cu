@@ -6,20 +6,33 @@
 // storage sites of one parity: R = 256 / (L/2) whole rows y0 .. y0+R-1 of one
 // plane z (L a power of 2, L >= 32).  Its sites read the opposite parity in
 // rows y0-1 .. y0+R of plane z (the +-x and +-y neighbours) and in rows
-// y0 .. y0+R-1 of planes z-1 and z+1.  Those rows are contiguous runs of the
-// parity-split layout, so per component plane and chunk group they reach
-// shared memory as six cp.async.bulk copies (the rows y0-1 and y0+R apart, as
-// they wrap in y).  The block walks its chunk groups through a two-stage ring:
-// while it computes chunk group g, the copies of g+1 are in flight.  Each stage
-// has a full mbarrier carrying the copies' bytes; a warp that has read its
-// neighbours of a stage counts itself out on the stage's counter, and the last
-// warp to do so issues the copies of the stage's next chunk group, so no warp
-// waits for another except through the data.  The spins a thread updates come
-// by a plain load issued before its wait; the update is the per-half-sweep
+// y0 .. y0+R-1 of planes z-1 and z+1.  Those rows, and the block's own, are
+// contiguous runs of the parity-split layout, so per component plane and chunk
+// group they reach shared memory as six cp.async.bulk copies (the rows y0-1 and
+// y0+R apart, as they wrap in y).  The block walks its chunk groups through a
+// two-stage ring: while it computes chunk group g, the copies of g+1 are in
+// flight.  Each stage has a full mbarrier carrying the copies' bytes and an empty
+// one that its warps arrive at once they have read it.  The copies of the stage's
+// next chunk group are issued by one warp, another in each iteration, at the end of
+// its own update, when the others have mostly read the stage: no warp waits there
+// for long, and none issues all of them.  The update is the per-half-sweep
 // kernel's, in the same operations and order, so the results are bit for bit
 // the same.  Every wait is bounded: one that runs out sets the error word, and
 // the block stops computing but keeps waiting (bounded) for the copies it
 // issued before it exits.
+//
+// What bounds it: at L = 128 the half-sweep's one pass over each parity in DRAM, at
+// smaller L the reads from L2 to the SMs (about 9 TB/s).  Against the kernel that
+// loads into registers, a block reads each row once from L2, and no registers wait
+// for it.  A half-sweep of 48 systems at L = 128: FP16 168.4 us in registers and 152.8
+// staged (149 at the measured copy rate; 168.4 as well while the own spins came by
+// plain loads and the last warp to read a stage refilled it), BF16 171 and 159, FP32
+// 290 and 288 (267).  At L = 64 both kernels take the same (28 us for 12 samples of
+// 32 systems), at L = 32 loading into registers is the faster: the tuner times both.
+// The L / 2 of 32 and 64 are compile-time, with the stages unrolled: the offsets are
+// then constants, which is what lets six neighbours and the own spins fit into the
+// registers.  Heat bath has no staged form: its registers spill (361 against 303 us
+// at L = 128).
 //
 // Wave launch.  One launch has one block per (block table entry, parity): the
 // blocks of the two per-half-sweep launches.  A block takes a ticket on entry
@@ -63,20 +76,23 @@ __device__ __forceinline__ bool wait_flag(const unsigned int* f, unsigned int wa
   return true;
 }
 
-// Chunks of one component plane of a stage: rows [y0-1 .. y0+R] of plane z,
-// then rows [y0 .. y0+R-1] of plane z-1, then of plane z+1 (R Lh = 256).
-__host__ __device__ constexpr int stage_plane_chunks(int Lh) { return 3 * SWEEP_BS + 2 * Lh; }
+// Chunks of one component plane of a stage: rows [y0-1 .. y0+R] of plane z, then rows
+// [y0 .. y0+R-1] of planes z-1 and z+1 of the opposite parity, then the block's own
+// sites (R Lh = 256).
+__host__ __device__ constexpr int stage_plane_chunks(int Lh) { return 4 * SWEEP_BS + 2 * Lh; }
 
-// One block of an over-relaxation half-sweep (parity p.parity) with staged
-// neighbour rows; smem: dynamic shared memory laid out as in staged_smem().
-template <int F, bool J16, bool EN>
+// One block of an over-relaxation half-sweep (parity p.parity) with staged rows;
+// smem: dynamic shared memory laid out as in staged_smem().  LH: L / 2 of every sample
+// of the context, or 0 (read from the sample).
+template <int F, bool J16, bool EN, int LH>
 __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, unsigned char* smem) {
   constexpr int VEC = FmtInfo<F>::VEC, PL = FmtInfo<F>::PLANES, CH = FmtInfo<F>::CHUNK;
   constexpr int S = STAGED_STAGES;
+  constexpr int KINDS = 6;              // copies per component plane
   using Chunk = typename FmtInfo<F>::Chunk;
   constexpr bool MIXED = (F == FMT_F16) && J16;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem);
-  int* cnt = reinterpret_cast<int*>(smem + 64);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem);          // a stage's copies have landed
+  uint64_t* empty = reinterpret_cast<uint64_t*>(smem + 64);    // every warp has read the stage
   float* esum = reinterpret_cast<float*>(smem + STAGED_HEAD);
   unsigned char* stages = smem + p.stage_off;
 
@@ -86,7 +102,7 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
     return;
   }
   const SampleDev& sd = p.samples[blk.x];
-  const int L = sd.L, Lh = sd.Lh, R = SWEEP_BS / Lh;
+  const int L = LH ? 2 * LH : sd.L, Lh = LH ? LH : sd.Lh, R = SWEEP_BS / Lh;
   const int par = p.parity;
   const uint32_t half_n = (uint32_t)sd.N >> 1;
   const int g0 = blk.y * p.GPT, g1 = min(p.G, g0 + p.GPT), ng = g1 - g0;
@@ -94,15 +110,16 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
   const int z = r0 / L, y0 = r0 - z * L;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int pc = stage_plane_chunks(Lh);
+  const int stage_bytes = LH ? PL * stage_plane_chunks(LH) * CH : p.stage_bytes;
   const long long gstride = (long long)sd.N * CH;
   const uint32_t tx_bytes = (uint32_t)(PL * pc * CH);
 
-  // the copy this lane issues for a stage (lanes 0 .. 6 PL - 1 of the issuing warp)
+  // the copy this lane issues for a stage (lanes 0 .. KINDS PL - 1 of the issuing warp)
   long long c_src = 0;
   uint32_t c_dst = 0, c_bytes = 0;
-  if (lane < 6 * PL) {
-    const int pl = lane / 6, kind = lane - 6 * (lane / 6);
-    const uint32_t ob = (uint32_t)(1 - par) * half_n;
+  if (lane < KINDS * PL) {
+    const int pl = lane / KINDS, kind = lane - KINDS * (lane / KINDS);
+    uint32_t ob = (uint32_t)(1 - par) * half_n;
     int row, dst, nrows = R;
     if (kind == 0) {
       row = (y0 == 0 ? L - 1 : y0 - 1) + L * z, dst = 0, nrows = 1;
@@ -112,34 +129,35 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
       row = (y0 + R == L ? 0 : y0 + R) + L * z, dst = (R + 1) * Lh, nrows = 1;
     } else if (kind == 3) {
       row = y0 + L * (z == 0 ? L - 1 : z - 1), dst = (R + 2) * Lh;
-    } else {
+    } else if (kind == 4) {
       row = y0 + L * (z + 1 == L ? 0 : z + 1), dst = (2 * R + 2) * Lh;
+    } else {
+      ob = (uint32_t)par * half_n;
+      row = r0, dst = (3 * R + 2) * Lh;
     }
-    if (kind < 5) {
-      c_src = sd.spin_off + (long long)pl * sd.plane_stride + (long long)(ob + (uint32_t)row * Lh) * CH;
-      c_dst = (uint32_t)((pl * pc + dst) * CH);
-      c_bytes = (uint32_t)(nrows * Lh * CH);
-      // HSG_CHECK builds: the rows within the opposite half, the copy within its
-      // stage (else copy the same number of bytes from the plane's start: the
-      // stage's byte count still completes, the results are flagged)
-      if (HSG_OUT_OF_BOUNDS(row >= 0 && (long long)(row + nrows) * Lh <= (long long)half_n &&
-                                c_dst + c_bytes <= (uint32_t)p.stage_bytes,
-                            p.bounds_err))
-        c_src = sd.spin_off + (long long)pl * sd.plane_stride;
-    }
+    c_src = sd.spin_off + (long long)pl * sd.plane_stride + (long long)(ob + (uint32_t)row * Lh) * CH;
+    c_dst = (uint32_t)((pl * pc + dst) * CH);
+    c_bytes = (uint32_t)(nrows * Lh * CH);
+    // HSG_CHECK builds: the rows within their half, the copy within its stage (else
+    // copy the same number of bytes from the plane's start: the stage's byte count
+    // still completes, the results are flagged)
+    if (HSG_OUT_OF_BOUNDS(row >= 0 && (long long)(row + nrows) * Lh <= (long long)half_n &&
+                              c_dst + c_bytes <= (uint32_t)stage_bytes,
+                          p.bounds_err))
+      c_src = sd.spin_off + (long long)pl * sd.plane_stride;
   }
   auto issue = [&](int i) {   // the copies of chunk group g0 + i into stage i % S (one warp)
     const int s = i % S;
     if (lane == 0) mbar_expect_tx(&full[s], tx_bytes);
     __syncwarp();
     if (c_bytes)
-      bulk_copy_g2s(stages + s * p.stage_bytes + c_dst, p.spins + c_src + (long long)(g0 + i) * gstride,
+      bulk_copy_g2s(stages + s * stage_bytes + c_dst, p.spins + c_src + (long long)(g0 + i) * gstride,
                     c_bytes, &full[s]);
   };
   if (tid == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
-      cnt[s] = 0;
+      mbar_init(&empty[s], NW);
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -185,26 +203,20 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
 
   bool ok = true;
   int i = 0;
-  for (; i < ng; ++i) {
-    const int s = i % S;
+  // chunk group g0 + i from stage s (constant in the unrolled loop below); false: a wait ran out
+  auto step = [&](int s) {
     const uint32_t ph = (uint32_t)(i / S) & 1u;
-    unsigned char* own_p = own_base + (long long)(g0 + i) * gstride;
-    Chunk c[PL];
-    load_chunks<F, LD_PLAIN>(own_p, ps, c);
-    float e[VEC];
-#pragma unroll
-    for (int v = 0; v < VEC; ++v) e[v] = 0.0f;
-    if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.timeout_ns))) {
-      ok = false;
-      break;
-    }
-    const unsigned char* st = stages + s * p.stage_bytes;
-    Chunk nc[6][PL];
+    if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.timeout_ns))) return false;
+    const unsigned char* st = stages + s * stage_bytes;
+    Chunk nc[6][PL], c[PL];
 #pragma unroll
     for (int n = 0; n < 6; ++n)
 #pragma unroll
       for (int pl = 0; pl < PL; ++pl)
         nc[n][pl] = *reinterpret_cast<const Chunk*>(st + (pl * pc + off[n]) * CH);
+#pragma unroll
+    for (int pl = 0; pl < PL; ++pl)
+      c[pl] = *reinterpret_cast<const Chunk*>(st + (pl * pc + (3 * R + 2) * Lh + tid) * CH);
 
     // local field h = sum_n J_n s_n + H, in the order +x, -x, +y, -y, +z, -z
     Spins<VEC> hf;
@@ -249,21 +261,11 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
         }
       }
     }
-    // every neighbour value is in registers: count this warp out of the stage;
-    // the last warp refills it with the chunk group S further on
-    {
-      int last = 0;
-      __syncwarp();
-      if (lane == 0) {
-        last = atomicAdd(&cnt[s], 1) == NW - 1;
-        if (last) atomicExch(&cnt[s], 0);
-      }
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (last && i + S < ng) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue(i + S);
-      }
-    }
+    Spins<VEC> sv;
+    decode<F>(c, sv);
+    // every staged value is in registers: this warp is done with the stage
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&empty[s]);
     {
       const float2 hx2 = f2(h3[0]), hy2 = f2(h3[1]), hz2 = f2(h3[2]);
 #pragma unroll
@@ -273,16 +275,15 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
         hf.z[k] = add2(hf.z[k], hz2);
       }
     }
-    Spins<VEC> sv;
-    decode<F>(c, sv);
 #pragma unroll
     for (int k = 0; k < VEC / 2; ++k) or_move2(sv.x[k], sv.y[k], sv.z[k], hf.x[k], hf.y[k], hf.z[k]);
     encode<F>(sv, c);
-    if (store_ok) store_chunks<F>(own_p, ps, c);
+    if (store_ok) store_chunks<F>(own_base + (long long)(g0 + i) * gstride, ps, c);
     if constexpr (EN) {
       // energy of the new state from the stored values: every bond joins one
       // odd and one even site, E = - sum_odd s_i.h_i - sum_even H_j.s_j
       Spins<VEC> stv;
+      float e[VEC];
       decode<F>(c, stv);
 #pragma unroll
       for (int k = 0; k < VEC / 2; ++k) {
@@ -299,6 +300,26 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
       const float t = warp_sum4_scatter(e, lane);
       if ((lane & 7) == 0) esum[warp * p.GPT * VEC + i * VEC + (lane >> 3)] = t;
     }
+    // refill the stage with the chunk group S further on, one warp after the other in
+    // turn: by the end of its own update the others have read the stage, as a rule
+    if (i + S < ng && warp == (i & (NW - 1))) {
+      if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ph, p.timeout_ns))) return false;
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      issue(i + S);
+    }
+    return true;
+  };
+  if constexpr (LH > 0) {   // unrolled over the stages: their offsets are constants
+    static_assert(S == 2, "two stages");
+    while (i < ng) {
+      if (!(ok = step(0))) break;
+      if (++i == ng) break;
+      if (!(ok = step(1))) break;
+      ++i;
+    }
+  } else {
+    for (; i < ng; ++i)
+      if (!(ok = step(i % S))) break;
   }
   if (!ok) {
     // a wait ran out: flag it and give the copies in flight a bounded time to
@@ -319,12 +340,12 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
   __syncthreads();   // the ring and its barriers are reused by nothing after this
 }
 
-template <int F, bool J16, bool EN>
+template <int F, bool J16, bool EN, int LH>
 __global__ void __launch_bounds__(SWEEP_BS, 4) k_staged_half(const SweepParams p) {
   extern __shared__ __align__(128) unsigned char smem[];
   chain_trigger();
   const int k = p.reverse ? p.n_launch - 1 - (int)blockIdx.x : (int)blockIdx.x;
-  staged_block<F, J16, EN>(p, p.blk_base + k, smem);
+  staged_block<F, J16, EN, LH>(p, p.blk_base + k, smem);
 }
 
 template <int F, bool J16, bool EN, bool STG>
@@ -346,7 +367,7 @@ __global__ void __launch_bounds__(SWEEP_BS, 4) k_wave_sweep(const WaveParams P) 
   if (!valid) {
     if (threadIdx.x == 0) atomicExch(P.err, 1u);
   } else if (parity == 0) {
-    if constexpr (STG) staged_block<F, J16, EN>(sp, b, smem);
+    if constexpr (STG) staged_block<F, J16, EN, 0>(sp, b, smem);
     else sweep_block<F, false, J16, false, EN, false>(sp, b, reinterpret_cast<float*>(smem));
   } else {
     // every even block of the planes this block reads or overwrites
@@ -362,7 +383,7 @@ __global__ void __launch_bounds__(SWEEP_BS, 4) k_wave_sweep(const WaveParams P) 
     if (__syncthreads_or(late)) {
       if (threadIdx.x == 0) atomicExch(P.err, 1u);
     } else {
-      if constexpr (STG) staged_block<F, J16, EN>(sp, b, smem);
+      if constexpr (STG) staged_block<F, J16, EN, 0>(sp, b, smem);
       else sweep_block<F, false, J16, false, EN, true>(sp, b, reinterpret_cast<float*>(smem));
     }
   }
@@ -404,18 +425,27 @@ cudaError_t launch_wf(bool j16, bool en, bool stg, const WaveParams& p, size_t s
   return en ? launch_w<F, false, true, false>(p, smem, st) : launch_w<F, false, false, false>(p, smem, st);
 }
 
-template <int F, bool J16, bool EN>
+template <int F, bool J16, bool EN, int LH>
 cudaError_t launch_h(const SweepParams& p, int n_blocks, size_t smem, cudaStream_t st) {
-  cudaError_t e = allow_smem(k_staged_half<F, J16, EN>, smem);
+  cudaError_t e = allow_smem(k_staged_half<F, J16, EN, LH>, smem);
   if (e != cudaSuccess) return e;
-  return launch_chained(k_staged_half<F, J16, EN>, n_blocks, SWEEP_BS, smem, st, p);
+  return launch_chained(k_staged_half<F, J16, EN, LH>, n_blocks, SWEEP_BS, smem, st, p);
+}
+
+template <int F, bool J16, bool EN>
+cudaError_t launch_hl(int Lh, const SweepParams& p, int n_blocks, size_t smem, cudaStream_t st) {
+  switch (Lh) {
+    case 32: return launch_h<F, J16, EN, 32>(p, n_blocks, smem, st);
+    case 64: return launch_h<F, J16, EN, 64>(p, n_blocks, smem, st);
+  }
+  return launch_h<F, J16, EN, 0>(p, n_blocks, smem, st);
 }
 
 template <int F>
-cudaError_t launch_hf(bool j16, bool en, const SweepParams& p, int n_blocks, size_t smem,
+cudaError_t launch_hf(bool j16, bool en, int Lh, const SweepParams& p, int n_blocks, size_t smem,
                       cudaStream_t st) {
-  if (j16) return en ? launch_h<F, true, true>(p, n_blocks, smem, st) : launch_h<F, true, false>(p, n_blocks, smem, st);
-  return en ? launch_h<F, false, true>(p, n_blocks, smem, st) : launch_h<F, false, false>(p, n_blocks, smem, st);
+  if (j16) return en ? launch_hl<F, true, true>(Lh, p, n_blocks, smem, st) : launch_hl<F, true, false>(Lh, p, n_blocks, smem, st);
+  return en ? launch_hl<F, false, true>(Lh, p, n_blocks, smem, st) : launch_hl<F, false, false>(Lh, p, n_blocks, smem, st);
 }
 
 template <int F>
@@ -471,13 +501,13 @@ cudaError_t launch_wave(int fmt, bool j16, bool energy, bool staged, const WaveP
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_staged_half(int fmt, bool j16, bool energy, const SweepParams& p, int n_blocks,
+cudaError_t launch_staged_half(int fmt, bool j16, bool energy, int Lh, const SweepParams& p, int n_blocks,
                                size_t smem, cudaStream_t st) {
   if (n_blocks <= 0) return cudaSuccess;
   switch (fmt) {
-    case FMT_F32: return launch_hf<FMT_F32>(j16, energy, p, n_blocks, smem, st);
-    case FMT_F16: return launch_hf<FMT_F16>(j16, energy, p, n_blocks, smem, st);
-    case FMT_BF16: return launch_hf<FMT_BF16>(j16, energy, p, n_blocks, smem, st);
+    case FMT_F32: return launch_hf<FMT_F32>(j16, energy, Lh, p, n_blocks, smem, st);
+    case FMT_F16: return launch_hf<FMT_F16>(j16, energy, Lh, p, n_blocks, smem, st);
+    case FMT_BF16: return launch_hf<FMT_BF16>(j16, energy, Lh, p, n_blocks, smem, st);
   }
   return cudaErrorInvalidValue;
 }

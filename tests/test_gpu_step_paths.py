@@ -1,8 +1,8 @@
 """The paths a step and its tail can take, against each other and the oracle: the
 resident sweeps (small lattices), the parallel-tempering pass with its decisions
 taken in parallel, the packed formats' decoded neighbours carried from one
-half-sweep to the next, and the heat bath's choice of hemisphere at small
-beta |h|."""
+half-sweep to the next, the staged half-sweeps, and the heat bath's choice of
+hemisphere at small beta |h|."""
 import numpy as np
 import pytest
 
@@ -141,3 +141,22 @@ def test_heat_bath_hemispheres_at_small_a(T):
     orc.sweep_hb(1)
     assert np.abs(ctx.get_spins()[0] - orc.spins()[0]).max() < 1e-5
     ctx.close()
+
+
+@pytest.mark.parametrize("Ls,n_temps,precision,j16", [
+    ((128,), 5, "fp32", False), ((128,), 5, "fp32", True), ((128,), 5, "fp16", False), ((128,), 9, "bf16", True),
+    ((64, 64), 3, "bf16", False), ((32, 64), 3, "fp32", False), ((32, 64), 3, "fp16", True), ((32,), 9, "fp16", False)])
+def test_staged_half_sweeps(Ls, n_temps, precision, j16):
+    """Staged over-relaxation half-sweeps (L / 2 of 64 and 32 in constants, any other
+    and mixed lattices at run time), odd and even numbers of chunk groups per block:
+    the same bits as half-sweeps that load into registers, energies included."""
+    samples = [inputs.small_sample(L, n_temps=n_temps, disorder_seed=L + k) for k, L in enumerate(Ls)]
+    out = []
+    for kernel in (hsg.SWEEP_HALF, hsg.SWEEP_STAGED):
+        ctx = hsg.Context(samples, 1, 5, precision=precision, j_fp16=j16, variant=hsg.VARIANT_TWO_PASS,
+                          sweep_kernel=kernel)
+        assert ctx.info().sweep_kernel == kernel
+        ctx.step(1)
+        out.append(state(ctx))
+        ctx.close()
+    same(out[0], out[1])
