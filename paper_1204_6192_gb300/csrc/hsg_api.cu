@@ -1135,15 +1135,19 @@ hsg_status autotune(hsg_ctx* c) {
     }
   }
   // the half-sweeps in passes on two branches of the step's graph: halves of the
-  // systems, and the footprints above (two passes in flight)
+  // systems, and half the footprints above, so that the two passes in flight fit the
+  // L2 cache together (512 samples of L = 8 to 24: 2631 us a step with one pass of
+  // half the cache in flight, 2694 with two of that size, 2362 with two of a quarter;
+  // L = 64 in FP16: 404, 388 and 347; three and four branches no faster).  The chunks
+  // per thread are tried anew: smaller passes want fewer.
   if (c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 && bestc.variant == HSG_VARIANT_TWO_PASS &&
       bestc.sweep == HSG_SWEEP_HALF) {
-    std::vector<int> near;
     for (int g : {bestc.gpt, (bestc.gpt + 1) / 2, 2 * bestc.gpt})
-      if (g <= c->G && std::find(near.begin(), near.end(), g) == near.end()) near.push_back(g);
+      if (g <= c->G && std::find(gpts.begin(), gpts.end(), g) == gpts.end()) gpts.push_back(g);
+    for (size_t k = 1; k < budgets.size(); ++k) budgets[k] /= 2;
     budgets[0] = (long long)(c->spin_bytes + 1) / 2 + (long long)c->rec_bytes;
     for (long long pb : budgets)
-      for (int g : near) HSG_TRY(time_candidate({HSG_VARIANT_TWO_PASS, g, pb, HSG_SWEEP_HALF, 0, 2}));
+      for (int g : gpts) HSG_TRY(time_candidate({HSG_VARIANT_TWO_PASS, g, pb, HSG_SWEEP_HALF, 0, 2}));
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
