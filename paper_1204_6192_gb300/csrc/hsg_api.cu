@@ -1141,7 +1141,7 @@ hsg_status autotune(hsg_ctx* c) {
   // L = 64 in FP16: 404, 388 and 347; three and four branches no faster).  The chunks
   // per thread are tried anew: smaller passes want fewer.
   if (c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 && bestc.variant == HSG_VARIANT_TWO_PASS &&
-      bestc.sweep == HSG_SWEEP_HALF) {
+      (bestc.sweep == HSG_SWEEP_HALF || (bestc.sweep == HSG_SWEEP_STAGED && sk == HSG_SWEEP_AUTO))) {
     for (int g : {bestc.gpt, (bestc.gpt + 1) / 2, 2 * bestc.gpt})
       if (g <= c->G && std::find(gpts.begin(), gpts.end(), g) == gpts.end()) gpts.push_back(g);
     for (size_t k = 1; k < budgets.size(); ++k) budgets[k] /= 2;

@@ -276,7 +276,7 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
       }
     }
 #pragma unroll
-    for (int k = 0; k < VEC / 2; ++k) or_move2(sv.x[k], sv.y[k], sv.z[k], hf.x[k], hf.y[k], hf.z[k]);
+    for (int k = 0; k < VEC / 2; ++k) or_move2_branch(sv.x[k], sv.y[k], sv.z[k], hf.x[k], hf.y[k], hf.z[k]);
     encode<F>(sv, c);
     if (store_ok) store_chunks<F>(own_base + (long long)(g0 + i) * gstride, ps, c);
     if constexpr (EN) {

@@ -160,3 +160,19 @@ def test_staged_half_sweeps(Ls, n_temps, precision, j16):
         out.append(state(ctx))
         ctx.close()
     same(out[0], out[1])
+
+
+@pytest.mark.parametrize("scale", [0.0, 1e-22, 1e-20, 4e-20, 1e-19, 1.0, 1e18, 3e18, 1e19, 1e20])
+def test_staged_move_at_extreme_fields(scale):
+    """Fields whose squares are zero, subnormal, at the edges of the normal numbers and
+    infinite: the staged move, which takes a shorter way for normal squares, gives the
+    spins of the plain half-sweep."""
+    base = inputs.small_sample(32, n_temps=2, disorder_seed=7)
+    smp = inputs.Sample(L=32, J=np.asarray(base.J) * scale, H=None, temps=base.temps)
+    out = []
+    for kernel in (hsg.SWEEP_HALF, hsg.SWEEP_STAGED):
+        ctx = hsg.Context([smp], 2, 5, variant=hsg.VARIANT_TWO_PASS, sweep_kernel=kernel)
+        ctx.sweep_or(2)
+        out.append(np.concatenate([s.ravel() for s in ctx.get_spins()]))
+        ctx.close()
+    np.testing.assert_array_equal(out[0], out[1])
