@@ -234,7 +234,9 @@ def timed_steps(ctx, stream, torch, steps, measure_every, flush=None):
     return total, n_meas
 
 
-SWEEP_NAMES = {1: "half", 2: "fused", 3: "wave", 4: "staged"}
+# (5, the resident sweeps, serve hsg_step only: an over-relaxation sweep of its own is
+# two half-sweep launches there)
+SWEEP_NAMES = {1: "half", 2: "fused", 3: "wave", 4: "staged", 5: "half"}
 
 
 def one_launch_per_sweep(info):
@@ -586,7 +588,7 @@ def main():
                    "l2": "state larger than L2 (no flush)", "parallelism": f"replicas x{world}",
                    "schedule": schedule_of(info)},
         "spin_updates_per_s": round(updates / (ms * 1e-3), 1),
-        "gpu_launches": args.steps * launches_per_step(info, wl) + n_meas * 2,
+        "gpu_launches": args.steps * launches_per_step(info, wl, tail=1) + n_meas * 2,
         "roofline": rl,
         "clocks": clocks.summary(),
         "observables_ms": observables_ms,
@@ -651,11 +653,14 @@ def schedule_of(info, short=False):
     kind = SWEEP_NAMES.get(info.sweep_kernel, "half")
     if short:
         return (("persistent" if persistent else "graph") + f"/gpt{info.chunks_per_thread}"
-                + f"/p{info.n_passes}" + ("" if kind == "half" else f"/{kind}"))
+                + f"/p{info.n_passes}"
+                + ("/resident" if info.sweep_kernel == 5 else "" if kind == "half" else f"/{kind}"))
     or_sweep = {"half": "one launch per half-sweep",
                 "staged": "one launch per half-sweep, neighbour rows staged in shared memory",
                 "fused": "fused (one launch per sweep, through shared memory)",
                 "wave": "wave (one launch per sweep, odd blocks trailing even blocks in L2)"}[kind]
+    if info.sweep_kernel == 5:
+        or_sweep = "resident (all sweeps of a step in one launch, lattices in shared memory)"
     out = {"variant": "persistent" if persistent else "two_pass (CUDA graph)",
            "chunks_per_thread": info.chunks_per_thread, "passes": info.n_passes,
            "or_sweep": or_sweep}
@@ -666,13 +671,17 @@ def schedule_of(info, short=False):
     return out
 
 
-def launches_per_step(info, wl):
+def launches_per_step(info, wl, tail=None):
     """Kernel launches of one step: the sweeps (two per sweep and pass, one per
-    fused sweep), the energy sums' first level and the PT pass with the sums'
-    last level (one launch for up to 4096 systems in all, else two)."""
+    fused sweep, one in all for resident lattices) and `tail` launches for the energy
+    sums and the PT pass.  This library takes one; without `tail` they are counted as
+    separate launches (two for up to 4096 systems in all, else three)."""
     if info.variant == 2:
         return 1
-    tail = 2 if info.n_samples * info.Wp <= 4096 else 3
+    if tail is None:
+        tail = 2 if info.n_samples * info.Wp <= 4096 else 3
+    if info.sweep_kernel == 5:
+        return 1 + tail
     if info.sweep_kernel == 2 and info.n_passes == 1:
         pairs = (wl.n_or - 1) // 2
         return 2 * wl.n_hb + 2 * pairs + 2 * (wl.n_or - 2 * pairs) + tail
