@@ -9,16 +9,24 @@
 // are computed once and reused for every chunk (the paper's reuse of J and H
 // across temperatures and replicas, Sec. 3.3).  Threads of a warp hold
 // consecutive sites, so every chunk load of a warp is contiguous.  The six
-// neighbours belong to the other parity, which this launch only reads, so
-// they go through the read-only data path.
+// neighbours belong to the other parity, which this launch only reads, but the
+// launch before it may still be writing when this one starts: plain loads after
+// chain_wait(), never the read-only path.
 #include "hsg_kernels.cuh"
 
 namespace hsg {
 
-// Both sweep kernels are latency-bound: the more warps resident per SM, the more
-// loads in flight.  Bounded to 64 registers, i.e. 4 blocks (32 warps) per SM,
-// every storage format but YX4 compiles with at most a few bytes of spill and
-// runs 2-15 % faster than at its natural 74-104 registers (2-3 blocks per SM).
+// What bounds them.  Heat bath: instruction issue (75 % of the slots at L = 128).
+// Over-relaxation with the spins in L2: the L1 data pipe (70 % of the active cycles
+// at L = 24, binary32; 21 loads and 3 stores of 512 bytes a warp and chunk, more
+// where rows are no whole lines) and the latency of L2 behind it; no share of L2's
+// own 20 TB/s (a tiled order of the sites that read a quarter less from L2 ran no
+// faster).  The more warps resident per SM, the more loads in flight, and every
+// spilled or staged word costs the pipe that is short: bounded to 64 registers, i.e.
+// 4 blocks (32 warps) per SM, every storage format but YX4 compiles with at most a
+// few bytes of spill and runs 2-15 % faster than at its natural 74-104 registers
+// (2-3 blocks per SM); 5 blocks at 48 registers (44-80 bytes of spills) are 20-40 %
+// slower, as is keeping the couplings in shared memory (10 %).
 // The YX4 decode of six neighbours needs ~120 registers and spills heavily under any
 // bound; with decoded neighbours its plain over-relaxation sweep takes 66.
 template <int F, bool HB, bool EN, bool DEC>
