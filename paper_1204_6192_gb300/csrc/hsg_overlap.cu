@@ -254,20 +254,24 @@ __host__ __device__ constexpr int staged_products() {
   return MODE == MEAS_QTENSOR ? 9 : (MODE == MEAS_CHIRAL ? 3 : 1) * (NR * (NR - 1) / 2);
 }
 // warp groups of a block.  The chiralities' components share no product and no
-// value, so three groups of 8 warps walk the same sites with a third of the sums
-// each: up to 42 accumulators a lane instead of 126, which left 8 warps on an SM.
-// (The tensor's rows all read replica 1: three groups decode it three times, 780 us
-// against 413 us at L = 128.)
-template <int MODE>
-__host__ __device__ constexpr int staged_groups() { return MODE == MEAS_CHIRAL ? 3 : 1; }
+// value, so for four replicas three groups of 8 warps walk the same sites with a
+// third of the sums each: 42 accumulators a lane instead of 126, which left 8 warps on
+// an SM.  Two and three replicas have 21 and 63 sums a lane, which fit beside enough
+// other warps, and there the groups only repeat each site's work (hsg_measure_overlaps,
+// L = 96: two replicas of 40 temperatures 1093 us in one group, 1570 in three; three of
+// 24 798 and 1056).  (The tensor's rows all read replica 1: three groups decode it three
+// times, 780 us against 413 us at L = 128.)
+template <int MODE, int NR>
+__host__ __device__ constexpr int staged_groups() { return MODE == MEAS_CHIRAL && NR >= 4 ? 3 : 1; }
 
 }  // namespace
 
 template <int F, int MODE, int NR>
-__global__ void __launch_bounds__(MEAS_BS * staged_groups<MODE>()) k_meas_staged(const OverlapParams p) {
+__global__ void __launch_bounds__(MEAS_BS * staged_groups<MODE, NR>()) k_meas_staged(const OverlapParams p) {
   using FI = FmtInfo<F>;
-  constexpr int NG = staged_groups<MODE>(), BS = MEAS_BS * NG;
+  constexpr int NG = staged_groups<MODE, NR>(), BS = MEAS_BS * NG;
   constexpr int NQ = staged_products<MODE, NR>(), NQG = NQ / NG;   // products of the block, of a group
+  constexpr int NC = 3 / NG;             // components of the chirality in a group
   constexpr int NV = NQ * NM;
   constexpr int NW = MEAS_BS / 32;       // warps of a group
   extern __shared__ __align__(128) unsigned char stage[];
@@ -405,16 +409,20 @@ __global__ void __launch_bounds__(MEAS_BS * staged_groups<MODE>()) k_meas_staged
           for (int nu = 0; nu < 3; ++nu) P[3 * mu + nu] = __fmul_rn(A[mu], B[nu]);
       } else if constexpr (MODE == MEAS_CHIRAL) {
         // the staged "spins" are the chiralities (kappa^x, kappa^y, kappa^z): per pair,
-        // in the pair order below, the product of component a = group
-        float K[NR];
+        // in the pair order below, the products of the group's components
+        float K[NR][NC];
 #pragma unroll
         for (int rr = 0; rr < NR; ++rr)
-          K[rr] = reinterpret_cast<const float*>(sj + off[rr] + group * PS)[jw[rr]];
+#pragma unroll
+          for (int a = 0; a < NC; ++a)
+            K[rr][a] = reinterpret_cast<const float*>(sj + off[rr] + (group * NC + a) * PS)[jw[rr]];
         int q = 0;
 #pragma unroll
         for (int bb = 1; bb < NR; ++bb)
 #pragma unroll
-          for (int aa = 0; aa < bb; ++aa) P[q++] = __fmul_rn(K[aa], K[bb]);
+          for (int aa = 0; aa < bb; ++aa)
+#pragma unroll
+            for (int a = 0; a < NC; ++a) P[q++] = __fmul_rn(K[aa][a], K[bb][a]);
       } else {
         // pairs in the order (0,1) (0,2) (1,2) (0,3) (1,3) (2,3)
         V3 S[NR];
@@ -485,7 +493,7 @@ __global__ void __launch_bounds__(MEAS_BS * staged_groups<MODE>()) k_meas_staged
 #pragma unroll
       for (int q = 0; q < NQG; ++q) {
         // product index in the output order (chiral: pair * 3 + component)
-        const int gq = MODE == MEAS_CHIRAL ? q * 3 + group : q;
+        const int gq = MODE == MEAS_CHIRAL ? q / NC * 3 + group * NC + q % NC : q;
         float* rv = red + (warp - w0) * per_warp + gq * NM * nt + tl;
         const float v[NM] = {a0[q], ak[q][0].x, ak[q][0].y, ak[q][1].x, ak[q][1].y, ak[q][2].x, ak[q][2].y};
 #pragma unroll
@@ -584,7 +592,7 @@ static cudaError_t staged_launch(OverlapParams p, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   const int rounds = (p.R_T + 31) / 32;
   e = launch_chained(k_meas_staged<F, MODE, NR>, dim3(p.n_tiles, rounds, p.n_samples),
-                     MEAS_BS * staged_groups<MODE>(), smem, st, p);
+                     MEAS_BS * staged_groups<MODE, NR>(), smem, st, p);
   if (e != cudaSuccess) return e;
   return launch_chained(k_meas_final_staged<MODE>, dim3((min(32, p.R_T) * NV + MF_COLS - 1) / MF_COLS, rounds, p.n_samples),
                         MF_COLS * MF_ROWS, 0, st, p, NV);
