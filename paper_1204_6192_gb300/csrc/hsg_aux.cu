@@ -119,8 +119,9 @@ __global__ void __launch_bounds__(RED_BS, F == FMT_YX4 ? 0 : 4) k_energy(const E
 // configuration that slot k+1 held before the pass with one carried up from some
 // slot j <= k: slot k's own when pair k-1 was rejected.  Whatever j will be, its
 // decision depends only on the energies and the pair's uniform, so all
-// (j <= k) decisions are taken at once, one warp per pair and 32 values of j, each
-// exactly as the sequential walk would take it.  What is left of the sequential
+// (j <= k) decisions are taken at once, one warp per pair and 32 values of j (with
+// fewer temperatures several pairs a warp: the FP64 instructions of a warp cost the
+// same for 8 lanes as for 32), each exactly as the sequential walk would take it.  What is left of the sequential
 // walk is one bit test per pair.  (R_T = 32: the walk with its FP64 arithmetic and
 // exponentials in the chain took 18 us and the sums before it 2.4; one launch now
 // takes 11.8; L32_fp32.)
@@ -131,14 +132,16 @@ constexpr int MAX_W = 1024, MAX_R_T = 256;   // limits of a context
 
 template <bool SUM, bool PT>
 __global__ void __launch_bounds__(TAIL_BS) k_energy_tail(const EnergyParams e, const PTParams p) {
-  __shared__ double red[8][32];
   __shared__ double sE[PT ? MAX_W : 1], sib[PT ? MAX_R_T : 1];   // energies by memory slot; inverse temperatures
   __shared__ int sperm[PT ? MAX_W : 1];         // the permutations before the pass
   __shared__ float su[PT ? MAX_W : 1];          // the pairs' uniforms
-  __shared__ uint32_t mask[PT ? TAIL_MASKS : 1];   // [chain of the batch][pair][j / 32]
+  __shared__ float2 sEf[PT ? MAX_W : 1];        // the same by slot: leading and trailing binary32 parts
+  __shared__ float sdb[PT ? MAX_R_T : 1];       // beta of slot k + 1 less that of slot k
+  __shared__ __align__(16) uint32_t mask[PT ? TAIL_MASKS : 512];   // [chain of the batch][pair][j / 32]
   __shared__ uint16_t walk[PT ? MAX_W : 1];     // [chain][slot]: carried j, bit 15: pair accepted
   __shared__ unsigned char sts[PT ? MAX_W : 1]; // tunnelling states
   __shared__ bool s_last;
+  double (*red)[32] = reinterpret_cast<double (*)[32]>(mask);   // [8][32], the sums' before the decisions
   chain_trigger();
   const int s = blockIdx.y, tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
   const unsigned char* active = SUM ? e.active : p.active;
@@ -184,7 +187,17 @@ __global__ void __launch_bounds__(TAIL_BS) k_energy_tail(const EnergyParams e, c
       if (!s_last) return;
       if (tid == 0) e.tickets[s] = 0u;
       __threadfence();
-      for (int g = 0; g < wgs; ++g) {
+      const bool few = e.splits <= 8;   // a warp adds a group's splits by itself, in the lanes' order
+      for (int g = ty; few && g < wgs; g += TAIL_BS / 32) {
+        const int v = g * 32 + tx;
+        if (v >= e.Wp) continue;
+        const double* src = e.splits == 1 ? e.E + (long long)s * e.Wp : e.partials2 + (long long)s * e.splits * e.Wp;
+        double t = 0.0;
+        for (int k = 0; k < e.splits; ++k) t += __ldcg(src + (long long)k * e.Wp + v);
+        if (e.splits > 1) e.E[(long long)s * e.Wp + v] = t;
+        if (PT) sE[v] = t;
+      }
+      for (int g = 0; !few && g < wgs; ++g) {
         const int v = g * 32 + tx;
         double acc = 0.0;
         if (v < e.Wp) {
@@ -215,20 +228,51 @@ __global__ void __launch_bounds__(TAIL_BS) k_energy_tail(const EnergyParams e, c
       }
     }
     __syncthreads();
+    for (int i = tid; i < W; i += TAIL_BS) {
+      const double E = sE[i / R * R + sperm[i]];
+      const float hi = (float)E;
+      sEf[i] = make_float2(hi, (float)(E - (double)hi));
+    }
+    for (int i = tid; i < R1; i += TAIL_BS) sdb[i] = (float)(sib[i + 1] - sib[i]);
+    __syncthreads();
+    int tw = 1;                  // lanes of a pair's word: its j <= k < R1
+    while (tw < min(R1, 32)) tw <<= 1;
     const int batch = R1 > 0 ? TAIL_MASKS / (R1 * nw) : p.R_O;
     for (int b0 = 0; b0 < p.R_O; b0 += batch) {
       const int nb = min(batch, p.R_O - b0);
-      for (int i = ty; i < nb * R1 * nw; i += TAIL_BS / 32) {
-        const int jw = i % nw, ck = i / nw, k = ck % R1, at = (b0 + ck / R1) * R;
-        const int j = jw * 32 + tx;
-        bool acc = false;
-        if (j <= k) {
-          const double dbeta = sib[k + 1] - sib[k];
-          const double dE = sE[at + sperm[at + k + 1]] - sE[at + sperm[at + j]];
-          acc = pt_accept(dbeta * dE, su[at + k]);
+      const int n = nb * R1;
+      for (int q0 = ty * (32 / tw); q0 < n; q0 += TAIL_BS / tw) {
+        const int q = min(q0 + tx / tw, n - 1), c = q / R1, k = q - c * R1, at = (b0 + c) * R;
+        const float2 b = sEf[at + k + 1];
+        const float db = sdb[k], u = su[at + k];
+        // (words above k are read by no walk; tw < 32: one word a pair)
+#pragma unroll 2
+        for (int jw = 0; jw < nw && (tw < 32 || jw * 32 <= k); ++jw) {
+          const int j = jw * 32 + tx % tw;
+          bool acc = false;
+          if (j <= k) {
+            // x = dbeta dE in binary32, within 3e-7 of its value (the difference of the
+            // leading parts, each a multiple of its last place, rounds once; the trailing
+            // parts reach 2^-48 of the energies): decided where that leaves no doubt,
+            // i.e. where dE is above the parts' resolution, no operand is subnormal or
+            // out of range, and u is not within 1e-5 of exp(x) <= 1; else by pt_accept
+            const float2 a = sEf[at + j];
+            const float dEf = __fadd_rn(__fsub_rn(b.x, a.x), __fsub_rn(b.y, a.y));
+            const float xf = __fmul_rn(db, dEf);
+            const float mag = fabsf(xf), lim = __fmul_rn(1e-6f, fabsf(a.x) + fabsf(b.x));
+            const float ex = expf(fmaxf(xf, -20.0f));
+            if (fabsf(dEf) > lim && mag > 1e-30f && mag < 1e30f && fabsf(db) > 1e-30f &&
+                (xf > 0.0f || xf < -17.1f || fabsf(u - ex) > 1e-5f * ex)) {
+              acc = xf > 0.0f || (xf >= -17.1f && u < ex);
+            } else {
+              const double dbeta = sib[k + 1] - sib[k];
+              const double dE = sE[at + sperm[at + k + 1]] - sE[at + sperm[at + j]];
+              acc = pt_accept(dbeta * dE, u);
+            }
+          }
+          const uint32_t m = __ballot_sync(0xffffffffu, acc) >> (tx & ~(tw - 1));
+          if (tx % tw == 0) mask[q * nw + jw] = tw == 32 ? m : m & ((1u << tw) - 1u);
         }
-        const uint32_t m = __ballot_sync(0xffffffffu, acc);
-        if (tx == 0) mask[i] = m;
       }
       __syncthreads();
       for (int c = tid; c < nb; c += TAIL_BS) {

@@ -64,7 +64,7 @@ def test_resident_limit():
         ctx.close()
 
 
-@pytest.mark.parametrize("R_T,R_O", [(1, 3), (2, 300), (32, 3), (33, 2), (64, 2), (97, 5), (256, 4)])
+@pytest.mark.parametrize("R_T,R_O", [(1, 3), (2, 300), (3, 100), (5, 7), (8, 64), (9, 33), (17, 20), (31, 3), (32, 3), (33, 2), (64, 2), (97, 5), (256, 4)])
 def test_pt_decisions_match_oracle(R_T, R_O):
     """Passes on given energies, where the decision words of the chains need one or
     several words a pair and one or several batches: permutations and diagnostics
