@@ -120,11 +120,10 @@ __global__ void __launch_bounds__(RED_BS, F == FMT_YX4 ? 0 : 4) k_energy(const E
 // slot j <= k: slot k's own when pair k-1 was rejected.  Whatever j will be, its
 // decision depends only on the energies and the pair's uniform, so all
 // (j <= k) decisions are taken at once, one warp per pair and 32 values of j (with
-// fewer temperatures several pairs a warp: the FP64 instructions of a warp cost the
+// fewer temperatures several pairs a warp: its instructions cost the
 // same for 8 lanes as for 32), each exactly as the sequential walk would take it.  What is
-// left of the
-// sequential walk is one bit test per pair.  (R_T = 32: the walk with its FP64 arithmetic
-// and exponentials in the chain took 18 us and the sums before it 2.4; one launch now
+// left of the sequential walk is one bit test per pair.  (R_T = 32: the walk with its
+// FP64 arithmetic and exponentials in the chain took 18 us and the sums before it 2.4; one launch now
 // takes 11 in all.)  R_T^2 / 2 decisions are many for long chains, and FP64 runs at two
 // lanes a clock and SM, so a decision is taken from the energies' two binary32 parts
 // where those leave no doubt (R_T = 256, R_O = 4, hsg_pt_exchange: 428 us with every
