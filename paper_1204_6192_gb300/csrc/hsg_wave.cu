@@ -54,6 +54,8 @@
 // time, mostly comes from L2.  The last block to finish resets the ticket and
 // completion counters and advances the epoch the completion flags carry, so
 // each launch (and each replay of a captured graph) starts clean.
+#include <algorithm>
+
 #include "hsg_async.cuh"
 #include "hsg_kernels.cuh"
 
@@ -478,7 +480,9 @@ size_t staged_smem(int fmt, int gpt, bool energy, int Lh_max, int* stage_off) {
   const size_t esum = energy ? sizeof(float) * NW * (size_t)gpt * 4 : 0;
   const size_t off = (STAGED_HEAD + esum + 127) / 128 * 128;
   *stage_off = (int)off;
-  return off + (size_t)STAGED_STAGES * staged_stage_bytes(fmt, Lh_max);
+  // (a block of one chunk group uses one stage; L = 256, 4 systems, FP16: with the room
+  // of both, 3 blocks an SM, a sweep took 728 us)
+  return off + (size_t)std::min(STAGED_STAGES, gpt) * staged_stage_bytes(fmt, Lh_max);
 }
 
 cudaError_t wave_occupancy(int fmt, bool j16, bool staged, size_t smem, int* blocks_per_sm) {
