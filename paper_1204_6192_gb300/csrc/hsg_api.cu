@@ -264,7 +264,7 @@ SweepParams sweep_params(hsg_ctx* c, int parity, int sweep_offset) {
   p.reverse = 0;
   p.dec = c->dec_both ? c->dec + (1 - parity) * c->dec_bytes : c->dec;
   p.dec_out = c->dec_both ? c->dec + parity * c->dec_bytes : nullptr;
-  p.stage_bytes = c->staged_possible ? staged_stage_bytes(c->fmt, c->Lh_max) : 0;
+  p.stage_bytes = c->staged_possible ? staged_stage_bytes(c->fmt, c->Lh_max, false) : 0;
   p.stage_off = 0;
   p.err = c->d_bar + 5;
   p.bounds_err = c->d_bar + 6;
@@ -347,7 +347,7 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
   if (!hb && c->use_staged) {
     const bool one_L = std::all_of(c->L.begin(), c->L.end(), [&](int L) { return L == c->L[0]; });
     int off = 0;
-    const size_t smem = staged_smem(c->fmt, c->GPT, energy, c->Lh_max, &off);
+    const size_t smem = staged_smem(c->fmt, c->GPT, energy, c->Lh_max, one_L, &off);
     for (int parity = 0; parity < 2; ++parity) {
       SweepParams p = sweep_params(c, parity, sweep_offset);
       p.blk_base = b0;
@@ -365,7 +365,7 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
     WaveParams w;
     w.sw = sweep_params(c, 0, sweep_offset);
     int off = 0;
-    size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, energy, c->Lh_max, &off)
+    size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, energy, c->Lh_max, false, &off)
                                      : (energy ? sizeof(float) * (SWEEP_BS / 32) * c->GPT * c->VEC : 0);
     w.sw.stage_off = off;
     w.order = c->d_wave_order;
@@ -753,7 +753,7 @@ hsg_status plan_wave(hsg_ctx* c, const std::vector<int4>& blocks, int lag) {
   }
   if (lag <= 0) {
     int per_sm = 0, n_sm = 0, off = 0;
-    const size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, false, c->Lh_max, &off) : 0;
+    const size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, false, c->Lh_max, false, &off) : 0;
     HSG_CUDA(c, wave_occupancy(c->fmt, c->j16, c->staged_possible, smem, &per_sm));
     HSG_CUDA(c, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device));
     lag = std::max(1, n_sm * per_sm / 2);
@@ -1064,7 +1064,7 @@ hsg_status autotune(hsg_ctx* c) {
       sweeps.push_back({HSG_SWEEP_WAVE, c->opt.wave_lag});
     } else {
       int per_sm = 0, n_sm = 0, off = 0;
-      const size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, false, c->Lh_max, &off) : 0;
+      const size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, false, c->Lh_max, false, &off) : 0;
       HSG_CUDA(c, wave_occupancy(c->fmt, c->j16, c->staged_possible, smem, &per_sm));
       HSG_CUDA(c, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device));
       const int resident = std::max(4, n_sm * per_sm);

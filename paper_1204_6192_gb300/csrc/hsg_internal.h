@@ -272,8 +272,9 @@ bool fmt_has_wave(int fmt);
 constexpr int STAGED_STAGES = 2;
 constexpr int STAGED_HEAD = 256;          // mbarriers
 bool lattice_has_staged(int L);
-int staged_stage_bytes(int fmt, int Lh_max);
-size_t staged_smem(int fmt, int gpt, bool energy, int Lh_max, int* stage_off);
+int staged_stage_bytes(int fmt, int Lh_max, bool own);
+// (one_L: every sample has this L / 2 and the kernel is the half-sweep's)
+size_t staged_smem(int fmt, int gpt, bool energy, int Lh_max, bool one_L, int* stage_off);
 // blocks per SM of the wave kernel (staged: with that dynamic shared memory)
 cudaError_t wave_occupancy(int fmt, bool j16, bool staged, size_t smem, int* blocks_per_sm);
 cudaError_t launch_wave(int fmt, bool j16, bool energy, bool staged, const WaveParams& p, size_t smem,

@@ -8,7 +8,7 @@
 // rows y0-1 .. y0+R of plane z (the +-x and +-y neighbours) and in rows
 // y0 .. y0+R-1 of planes z-1 and z+1.  Those rows, and the block's own, are
 // contiguous runs of the parity-split layout, so per component plane and chunk
-// group they reach shared memory as six cp.async.bulk copies (the rows y0-1 and
+// group they reach shared memory as six (five without the own rows) cp.async.bulk copies (the rows y0-1 and
 // y0+R apart, as they wrap in y).  The block walks its chunk groups through a
 // two-stage ring: while it computes chunk group g, the copies of g+1 are in
 // flight.  Each stage has a full mbarrier carrying the copies' bytes and an empty
@@ -79,9 +79,16 @@ __device__ __forceinline__ bool wait_flag(const unsigned int* f, unsigned int wa
 }
 
 // Chunks of one component plane of a stage: rows [y0-1 .. y0+R] of plane z, then rows
-// [y0 .. y0+R-1] of planes z-1 and z+1 of the opposite parity, then the block's own
-// sites (R Lh = 256).
-__host__ __device__ constexpr int stage_plane_chunks(int Lh) { return 4 * SWEEP_BS + 2 * Lh; }
+// [y0 .. y0+R-1] of planes z-1 and z+1 of the opposite parity, then (own) the block's
+// own sites (R Lh = 256).
+__host__ __device__ constexpr int stage_plane_chunks(int Lh, bool own) {
+  return (own ? 4 : 3) * SWEEP_BS + 2 * Lh;
+}
+// Own rows in the stage: with L / 2 in constants.  At L = 256 they would cost a resident
+// block (binary32: 2 -> 1, a sweep of 4 systems 1260 -> 1731 us), so the form for any L
+// loads them into registers ahead of its wait.
+__host__ __device__ constexpr bool stage_has_own(int LH) { return LH > 0; }
+constexpr int const_lh(int Lh) { return Lh == 32 || Lh == 64 ? Lh : 0; }
 
 // One block of an over-relaxation half-sweep (parity p.parity) with staged rows;
 // smem: dynamic shared memory laid out as in staged_smem().  LH: L / 2 of every sample
@@ -90,7 +97,8 @@ template <int F, bool J16, bool EN, int LH>
 __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, unsigned char* smem) {
   constexpr int VEC = FmtInfo<F>::VEC, PL = FmtInfo<F>::PLANES, CH = FmtInfo<F>::CHUNK;
   constexpr int S = STAGED_STAGES;
-  constexpr int KINDS = 6;              // copies per component plane
+  constexpr bool OWN = stage_has_own(LH);
+  constexpr int KINDS = OWN ? 6 : 5;    // copies per component plane
   using Chunk = typename FmtInfo<F>::Chunk;
   constexpr bool MIXED = (F == FMT_F16) && J16;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);          // a stage's copies have landed
@@ -111,8 +119,8 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
   const int r0 = blk.z / Lh;                  // first row (y + L z) of the block
   const int z = r0 / L, y0 = r0 - z * L;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int pc = stage_plane_chunks(Lh);
-  const int stage_bytes = LH ? PL * stage_plane_chunks(LH) * CH : p.stage_bytes;
+  const int pc = stage_plane_chunks(Lh, OWN);
+  const int stage_bytes = LH ? PL * stage_plane_chunks(LH, OWN) * CH : p.stage_bytes;
   const long long gstride = (long long)sd.N * CH;
   const uint32_t tx_bytes = (uint32_t)(PL * pc * CH);
 
@@ -208,16 +216,18 @@ __device__ __forceinline__ void staged_block(const SweepParams& p, int bidx, uns
   // chunk group g0 + i from stage s (constant in the unrolled loop below); false: a wait ran out
   auto step = [&](int s) {
     const uint32_t ph = (uint32_t)(i / S) & 1u;
+    Chunk c[PL];
+    if constexpr (!OWN) load_chunks<F, LD_PLAIN>(own_base + (long long)(g0 + i) * gstride, ps, c);
     if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, p.timeout_ns))) return false;
     const unsigned char* st = stages + s * stage_bytes;
-    Chunk nc[6][PL], c[PL];
+    Chunk nc[6][PL];
 #pragma unroll
     for (int n = 0; n < 6; ++n)
 #pragma unroll
       for (int pl = 0; pl < PL; ++pl)
         nc[n][pl] = *reinterpret_cast<const Chunk*>(st + (pl * pc + off[n]) * CH);
 #pragma unroll
-    for (int pl = 0; pl < PL; ++pl)
+    for (int pl = 0; OWN && pl < PL; ++pl)
       c[pl] = *reinterpret_cast<const Chunk*>(st + (pl * pc + (3 * R + 2) * Lh + tid) * CH);
 
     // local field h = sum_n J_n s_n + H, in the order +x, -x, +y, -y, +z, -z
@@ -436,7 +446,7 @@ cudaError_t launch_h(const SweepParams& p, int n_blocks, size_t smem, cudaStream
 
 template <int F, bool J16, bool EN>
 cudaError_t launch_hl(int Lh, const SweepParams& p, int n_blocks, size_t smem, cudaStream_t st) {
-  switch (Lh) {
+  switch (const_lh(Lh)) {
     case 32: return launch_h<F, J16, EN, 32>(p, n_blocks, smem, st);
     case 64: return launch_h<F, J16, EN, 64>(p, n_blocks, smem, st);
   }
@@ -469,20 +479,21 @@ bool fmt_has_wave(int fmt) { return fmt == FMT_F32 || fmt == FMT_F16 || fmt == F
 
 bool lattice_has_staged(int L) { return L >= 32 && (L & (L - 1)) == 0; }
 
-int staged_stage_bytes(int fmt, int Lh_max) {
+int staged_stage_bytes(int fmt, int Lh_max, bool own) {
   const int ch = fmt == FMT_F32 ? 16 : 8;   // component formats: 3 planes
-  return 3 * stage_plane_chunks(Lh_max) * ch;
+  return 3 * stage_plane_chunks(Lh_max, own) * ch;
 }
 
 // [0, STAGED_HEAD): mbarriers and stage counters; then the energy sums of the
 // warps (energy sweeps); then, 128-byte aligned, the ring of stages.
-size_t staged_smem(int fmt, int gpt, bool energy, int Lh_max, int* stage_off) {
+size_t staged_smem(int fmt, int gpt, bool energy, int Lh_max, bool one_L, int* stage_off) {
   const size_t esum = energy ? sizeof(float) * NW * (size_t)gpt * 4 : 0;
   const size_t off = (STAGED_HEAD + esum + 127) / 128 * 128;
   *stage_off = (int)off;
   // (a block of one chunk group uses one stage; L = 256, 4 systems, FP16: with the room
   // of both, 3 blocks an SM, a sweep took 728 us)
-  return off + (size_t)std::min(STAGED_STAGES, gpt) * staged_stage_bytes(fmt, Lh_max);
+  return off + (size_t)std::min(STAGED_STAGES, gpt) *
+                   staged_stage_bytes(fmt, Lh_max, one_L && stage_has_own(const_lh(Lh_max)));
 }
 
 cudaError_t wave_occupancy(int fmt, bool j16, bool staged, size_t smem, int* blocks_per_sm) {
