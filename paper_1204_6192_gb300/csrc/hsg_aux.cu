@@ -351,7 +351,10 @@ cudaError_t launch_pt(const PTParams& p, cudaStream_t st) {
 
 template <int F, bool J16>
 static cudaError_t energy_fmt(const EnergyParams& p, cudaStream_t st) {
+  // (up to 64 kB: a thread may walk all 256 chunk groups of 1024 systems)
   const size_t smem = sizeof(float) * 2 * (RED_BS / 32) * p.GPT * FmtInfo<F>::VEC;
+  const cudaError_t e = allow_smem(k_energy<F, J16>, smem);
+  if (e != cudaSuccess) return e;
   return launch_chained(k_energy<F, J16>, p.n_blocks, RED_BS, smem, st, p);
 }
 

@@ -413,12 +413,6 @@ __global__ void __launch_bounds__(SWEEP_BS, 4) k_wave_sweep(const WaveParams P) 
   }
 }
 
-template <typename K>
-cudaError_t allow_smem(K kernel, size_t smem) {
-  if (smem <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 template <int F, bool J16, bool EN, bool STG>
 cudaError_t launch_w(const WaveParams& p, size_t smem, cudaStream_t st) {
   cudaError_t e = allow_smem(k_wave_sweep<F, J16, EN, STG>, smem);
