@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(TAIL_BS) k_energy_tail(const EnergyParams e, c
       if (!s_last) return;
       if (tid == 0) e.tickets[s] = 0u;
       __threadfence();
-      const bool few = e.splits <= 8;   // a warp adds a group's splits by itself, in the lanes' order
+      const bool few = e.splits <= E_FEW_SPLITS;   // a warp adds a group's splits by itself, in order
       for (int g = ty; few && g < wgs; g += TAIL_BS / 32) {
         const int v = g * 32 + tx;
         if (v >= e.Wp) continue;

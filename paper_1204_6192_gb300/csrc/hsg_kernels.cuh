@@ -229,9 +229,10 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
 // ---------------------------------------------------------------------------
 // FP64 energy sums.  Level 1: split `split` of the block rows that hold a
 // system's chunk group, systems 32*wg .. 32*wg+31, on 256 threads = 32 systems x
-// 8 row lanes.  Level 2: the splits of one system.  Fixed order throughout.  A
-// block of the sweep block table leaves partials only for the systems of its own
-// chunk groups, so a system's rows are those of its group.
+// 8 row lanes.  Level 2: the splits of one system.  One order of additions, whatever
+// the schedule, the chunks per thread and the passes.  A block of the sweep block table
+// leaves partials only for the systems of its own chunk groups, so a system's rows are
+// those of its group.
 // ---------------------------------------------------------------------------
 template <bool CG>
 __device__ __forceinline__ double energy_rows(const EnergyParams& p, int s, int w, int split, int ty) {
@@ -272,19 +273,25 @@ __device__ __forceinline__ void energy_final1_unit(const EnergyParams& p, int s,
   if (ty == 0 && w < p.Wp) p.partials2[((long long)s * p.splits + split) * p.Wp + w] = t;
 }
 
-// Level 2 for system w of sample s, one warp: lane j adds splits j, j + 32, ...
-// in order, then the lanes are added by a fixed shuffle tree.
+// Level 2: up to E_FEW_SPLITS splits are added one after the other, more by eight lanes
+// (lane j adds splits j, j + 8, ... in order) that are then added in order.  Here for
+// systems w0 .. w0 + 3 of sample s, one warp, eight lanes a system.
+constexpr int E_FEW_SPLITS = 8;
 template <bool CG>
-__device__ __forceinline__ void energy_final2_warp(const EnergyParams& p, int s, int w, int lane) {
+__device__ __forceinline__ void energy_final2_warp(const EnergyParams& p, int s, int w0, int lane) {
   if (!p.active[s]) return;
+  const int w = w0 + (lane >> 3), j = lane & 7;
+  const int step = p.splits <= E_FEW_SPLITS ? 1 : 8;   // few: every lane adds them all
   double e = 0.0;
-  for (int k = lane; k < p.splits; k += 32) {
-    const double* a = p.partials2 + ((long long)s * p.splits + k) * p.Wp + w;
-    e += CG ? __ldcg(a) : *a;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) e += __shfl_down_sync(0xffffffffu, e, o);
-  if (lane == 0) p.E[(long long)s * p.Wp + w] = e;
+  if (w < p.Wp)
+    for (int k = step == 1 ? 0 : j; k < p.splits; k += step) {
+      const double* a = p.partials2 + ((long long)s * p.splits + k) * p.Wp + w;
+      e += CG ? __ldcg(a) : *a;
+    }
+  double t = step == 1 ? e : 0.0;
+  if (step == 8)
+    for (int k = 0; k < 8; ++k) t += __shfl_sync(0xffffffffu, e, (lane & 24) + k);
+  if (j == 0 && w < p.Wp) p.E[(long long)s * p.Wp + w] = t;
 }
 
 // Metropolis decision of a PT pair (Eq. 4): accept iff x >= 0 or u < exp(x),

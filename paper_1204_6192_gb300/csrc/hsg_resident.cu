@@ -10,8 +10,8 @@
 // each of its six uses).  A block barrier stands between half-sweeps in place of a
 // launch, and memory sees each spin once per step.  Every update goes through the
 // storage codec, in the operations and order of the per-half-sweep kernels, and the
-// energies are summed over the same 32 half-sites a warp, so the results are theirs
-// bit for bit.
+// energies are summed over the same 32 half-sites a warp, then as those kernels' blocks
+// of eight warps and their energy sums do, so the results are theirs bit for bit.
 //
 // What bounds it: on small contexts the latency of a half-sweep (about 0.7 us) where
 // a launch took 2.5 us; with many samples the issue rate.
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResidentParams p) {
   constexpr int PL = FmtInfo<F>::PLANES, CH = FmtInfo<F>::CHUNK;
   constexpr bool MIXED = (F == FMT_F16) && J16;
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[MAXT / 32][2];
+  __shared__ float red[2][MAXT / 32][2];        // [parity][warp][system]
   chain_trigger();
   const int s = blockIdx.x / p.n_pairs, pr = blockIdx.x % p.n_pairs;   // sample, pair of systems
   if (!p.active[s]) {            // a frozen sample
@@ -136,7 +136,6 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResidentParams p) {
   const float* bp = p.beta + (long long)s * p.Wp + pr * 2;
   const float2 bt = make_float2(bp[0], bp[1]);
   const uint32_t sweep0 = (uint32_t)p.counters[2 * s];
-  double e0 = 0.0, e1 = 0.0;     // lane 0: the pair's energies over the warp's sites
   __syncthreads();
 
   const int nsw = p.n_hb + p.n_or;
@@ -196,22 +195,25 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResidentParams p) {
         const float2 tx = elem_f2<F>(own[par][0]), ty = elem_f2<F>(own[par][1]), tz = elem_f2<F>(own[par][2]);
         const float2 d = par == 1 ? dot3_2(tx, ty, tz, fx, fy, fz)
                                   : dot3_2(tx, ty, tz, f2(h3[par][0]), f2(h3[par][1]), f2(h3[par][2]));
-        e0 += (double)warp_sum(live ? -d.x : 0.0f);
-        e1 += (double)warp_sum(live ? -d.y : 0.0f);
+        const float e0 = warp_sum(live ? -d.x : 0.0f), e1 = warp_sum(live ? -d.y : 0.0f);
+        if (lane == 0) {
+          red[par][warp][0] = e0;
+          red[par][warp][1] = e1;
+        }
       }
       __syncthreads();
     }
   }
   if (p.n_or == 0) return;       // (the energies come from the separate kernel)
-  if (lane == 0) {
-    red[warp][0] = e0;
-    red[warp][1] = e1;
-  }
-  __syncthreads();
-  if (tid < 2) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w][tid];
-    p.E[(long long)s * p.Wp + pr * 2 + tid] = t;
+  if (warp == 0) {
+    // rows of SWEEP_BS half-sites (at most 4: one split, and a row lane for each): their
+    // even sites' partial and their odd sites', lane = 4 row + 2 parity + system
+    const int w0 = (lane >> 2) * (SWEEP_BS / 32), w1 = min((int)(blockDim.x >> 5), w0 + SWEEP_BS / 32);
+    double part = 0.0, t = 0.0;
+    for (int w = w0; w < w1; ++w) part += (double)red[(lane >> 1) & 1][w][lane & 1];
+    part += __shfl_xor_sync(0xffffffffu, part, 2);
+    for (int row = 0; row < 4; ++row) t += __shfl_sync(0xffffffffu, part, 4 * row + (lane & 1));
+    if (lane < 2) p.E[(long long)s * p.Wp + pr * 2 + lane] = t;
   }
 }
 
