@@ -167,6 +167,7 @@ struct hsg_ctx {
 namespace {
 
 hsg_status fail(hsg_ctx* c, hsg_status st, const std::string& m) {
+  cudaGetLastError();   // reported here: the next launch's check must not find it again
   if (c) {
     if (c->err == HSG_OK) {
       c->err = st;
@@ -1232,6 +1233,7 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
   c->L.assign(L, L + n_samples);
 
   auto cleanup_fail = [&](hsg_status st) {
+    cudaGetLastError();
     g_create_error = c->msg;
     hsg_destroy(c);
     return st;
