@@ -139,7 +139,8 @@ typedef struct {
                                number of resident blocks and by the automatic schedule. */
   int inject_alloc_fault;   /* testing only: n > 0 makes the n-th device allocation of the
                                context fail as an out-of-memory would (HSG_ENOMEM; during
-                               hsg_create the partial context is released); 0: off */
+                               hsg_create the partial context is released; a packed format's
+                               second buffer of decoded spins gives way instead); 0: off */
 } hsg_options;
 
 enum {
@@ -351,6 +352,9 @@ typedef struct {
   int fused_items;         /* fused sweep: work items (columns of planes) per launch */
   int wave_lag;            /* wave sweep: the lag in use (even blocks) */
   int staged;              /* nonzero: the over-relaxation sweep stages its neighbour rows */
+  int decoded_parities;    /* packed formats: parities whose spins are kept decoded from one
+                              half-sweep to the next (2), or 1 where memory is short for
+                              that; 0 for the other formats */
 } hsg_info;
 hsg_status hsg_get_info(hsg_ctx* ctx, hsg_info* info);
 

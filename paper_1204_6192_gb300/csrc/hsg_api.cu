@@ -45,12 +45,13 @@ struct hsg_ctx {
   size_t spin_bytes = 0;
   // packed formats: the spins decoded to binary32 for their six neighbours.  One
   // buffer per parity: a half-sweep reads its neighbours from the other parity's and
-  // leaves its own spins decoded in its own (dec_both; where the second buffer does
-  // not fit, one buffer, filled before each half-sweep)
-  bool dec_once = false, dec_both = false;
-  bool dec_fresh = false;             // the next half-sweep's neighbours are in dec
-  unsigned char* dec = nullptr;       // [parity][dec_bytes], or [dec_bytes]
-  size_t dec_bytes = 0;
+  // leaves its own spins decoded in its own.  Without the odd one's (dec2; given up
+  // where memory is short) one buffer, filled before each half-sweep
+  bool dec_once = false;
+  bool dec_fresh = false;             // the next half-sweep's neighbours are decoded
+  unsigned char *dec = nullptr, *dec2 = nullptr;
+  bool dec2_captured = false;         // a graph of the caller's refers to dec2
+  size_t dec_bytes = 0;               // of one of them
   void* rec = nullptr;
   size_t rec_bytes = 0;
   SampleDev* d_sd = nullptr;
@@ -217,19 +218,65 @@ void fastdiv(uint32_t d, uint32_t* m, uint32_t* s) {
   *s = l;
 }
 
+// whether fault injection makes this allocation fail
+bool alloc_injected(hsg_ctx* c) { return c->alloc_fail_at > 0 && ++c->alloc_count == c->alloc_fail_at; }
+
+void drop_graph(hsg_ctx* c) {
+  if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
+  if (c->graph) cudaGraphDestroy(c->graph);
+  c->graph_exec = nullptr;
+  c->graph = nullptr;
+}
+
+// Give the odd parity's decoded spins back to the device (and with them a captured
+// step, which refers to them); false if there are none or a graph of the caller's
+// needs them.
+bool release_dec2(hsg_ctx* c) {
+  if (!c->dec2 || c->dec2_captured || cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
+  drop_graph(c);
+  cudaFree(c->dec2);
+  c->dec2 = nullptr;
+  c->dec_fresh = false;
+  return true;
+}
+
+// Device memory that the caller frees or registers; the decoded spins of the odd
+// parity, which only save time, give way to it.
+hsg_status dev_malloc(hsg_ctx* c, void** q, size_t bytes) {
+  const bool injected = alloc_injected(c);
+  cudaError_t e = injected ? cudaErrorMemoryAllocation : cudaMalloc(q, bytes > 0 ? bytes : 16);
+  if (e == cudaErrorMemoryAllocation && release_dec2(c)) {
+    cudaGetLastError();
+    e = cudaMalloc(q, bytes > 0 ? bytes : 16);
+  } else if (injected) {
+    return fail(c, HSG_ENOMEM, "cudaMalloc(" + std::to_string(bytes) + "): injected allocation failure");
+  }
+  if (e != cudaSuccess)
+    return fail(c, HSG_ENOMEM, "cudaMalloc(" + std::to_string(bytes) + "): " + cudaGetErrorString(e));
+  return HSG_OK;
+}
+
 template <typename T>
 hsg_status dev_alloc(hsg_ctx* c, T** p, size_t bytes) {
-  if (c->alloc_fail_at > 0 && ++c->alloc_count == c->alloc_fail_at)
-    return fail(c, HSG_ENOMEM, "cudaMalloc(" + std::to_string(bytes) + "): injected allocation failure");
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, bytes > 0 ? bytes : 16);
-  if (e != cudaSuccess) {
-    return fail(c, HSG_ENOMEM, std::string("cudaMalloc(") + std::to_string(bytes) + "): " +
-                                   cudaGetErrorString(e));
-  }
+  const hsg_status st = dev_malloc(c, &q, bytes);
+  if (st != HSG_OK) return st;
   c->allocations.push_back(q);
   *p = reinterpret_cast<T*>(q);
   return HSG_OK;
+}
+
+// The odd parity's decoded spins, last of a context's allocations and only where the
+// buffers of later calls (the tuner's copy and the fused sweep's second buffer of the
+// spins, the spins and the chiralities as binary32) still fit beside them.
+void try_dec2(hsg_ctx* c) {
+  const size_t xyz = 12 * (size_t)c->total_sites * c->Wp, later = 2 * c->spin_bytes + 2 * xyz;
+  size_t free_bytes = 0, total = 0;
+  if (alloc_injected(c) || cudaMemGetInfo(&free_bytes, &total) != cudaSuccess ||
+      free_bytes < later + c->dec_bytes || cudaMalloc(&c->dec2, c->dec_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    c->dec2 = nullptr;
+  }
 }
 
 #define HSG_TRY(expr)                  \
@@ -263,8 +310,8 @@ SweepParams sweep_params(hsg_ctx* c, int parity, int sweep_offset) {
   p.blk_base = 0;
   p.n_launch = c->n_sweep_blocks;
   p.reverse = 0;
-  p.dec = c->dec_both ? c->dec + (1 - parity) * c->dec_bytes : c->dec;
-  p.dec_out = c->dec_both ? c->dec + parity * c->dec_bytes : nullptr;
+  p.dec = c->dec2 && parity == 0 ? c->dec2 : c->dec;
+  p.dec_out = !c->dec2 ? nullptr : parity == 0 ? c->dec : c->dec2;
   p.stage_bytes = c->staged_possible ? staged_stage_bytes(c->fmt, c->Lh_max, false) : 0;
   p.stage_off = 0;
   p.err = c->d_bar + 5;
@@ -398,11 +445,11 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
     // of a launch are independent, so the order changes no result): each
     // launch starts on the planes whose spins the previous one left in L2.
     // Packed formats: the decode launch runs forward, the sweep backward.
-    p.reverse = c->dec_once && !c->dec_both ? 1 : parity;
+    p.reverse = c->dec_once && !c->dec2 ? 1 : parity;
     // packed formats: decode the other parity once for the six neighbour loads,
     // unless the half-sweep before this one left it decoded
     if (c->dec_once && !c->dec_fresh) HSG_CUDA(c, launch_decode_parity(c->fmt, p, 1 - parity, b1 - b0, c->stream));
-    c->dec_fresh = c->dec_both;
+    c->dec_fresh = c->dec2 != nullptr;
     HSG_CUDA(c, launch_half_sweep(c->fmt, hb, c->j16, c->opt.fast_math != 0, energy, c->dec_once, p,
                                   b1 - b0, c->stream));
   }
@@ -540,10 +587,21 @@ hsg_status fused_sweep_pairs(hsg_ctx* c, int pairs) {
   return HSG_OK;
 }
 
+// Before sweeps outside a step, which a caller may be capturing.
+hsg_status begin_sweeps(hsg_ctx* c) {
+  c->dec_fresh = false;
+  if (c->dec2 && !c->dec2_captured) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    HSG_CUDA(c, cudaStreamIsCapturing(c->stream, &capture));
+    c->dec2_captured = capture != cudaStreamCaptureStatusNone;
+  }
+  return HSG_OK;
+}
+
 // n OR sweeps outside a step: fused pairs where in use, the rest per half-sweep.
 hsg_status or_sweeps(hsg_ctx* c, int n, int sweep_offset) {
   int k = 0;
-  c->dec_fresh = false;
+  HSG_TRY(begin_sweeps(c));
   if (c->use_fused && n >= 2) {
     HSG_TRY(fused_sweep_pairs(c, n / 2));
     k = 2 * (n / 2);
@@ -894,14 +952,7 @@ hsg_status configure_schedule(hsg_ctx* c, int variant, int gpt, long long pass_b
   HSG_CUDA(c, cudaMemcpyAsync(c->d_sd, c->sd.data(), sizeof(SampleDev) * c->ns,
                               cudaMemcpyHostToDevice, c->stream));
   HSG_CUDA(c, cudaStreamSynchronize(c->stream));
-  if (c->graph_exec) {
-    cudaGraphExecDestroy(c->graph_exec);
-    c->graph_exec = nullptr;
-  }
-  if (c->graph) {
-    cudaGraphDestroy(c->graph);
-    c->graph = nullptr;
-  }
+  drop_graph(c);
   c->variant = variant;
   c->chains = chains;
   // the fused over-relaxation sweep serves the two-pass schedule in one pass,
@@ -1040,7 +1091,7 @@ hsg_status autotune(hsg_ctx* c) {
   }
   // save the state the trial steps will change
   void* spins_copy = nullptr;
-  HSG_CUDA(c, cudaMalloc(&spins_copy, c->spin_bytes));
+  HSG_TRY(dev_malloc(c, &spins_copy, c->spin_bytes));
   std::vector<unsigned char> saved(chain_state_bytes(c));
   cudaStream_t st = c->stream;
   const bool e_valid = c->e_valid;
@@ -1346,16 +1397,7 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
   HSG_ALLOC(c->spins, c->spin_bytes);
   c->dec_once = fmt_decodes_once(fmt);
   if (c->dec_once) {
-    // both parities if they fit (not counted as an allocation that has to succeed)
-    void* both = nullptr;
-    c->dec_both = opt.inject_alloc_fault == 0 && cudaMalloc(&both, 2 * c->dec_bytes) == cudaSuccess;
-    if (c->dec_both) {
-      c->allocations.push_back(both);
-      c->dec = (unsigned char*)both;
-    } else {
-      cudaGetLastError();
-      HSG_ALLOC(c->dec, c->dec_bytes);
-    }
+    HSG_ALLOC(c->dec, c->dec_bytes);
   }
   HSG_ALLOC(c->rec, c->rec_bytes);
   HSG_ALLOC(c->d_sd, sizeof(SampleDev) * n_samples);
@@ -1378,6 +1420,7 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
   HSG_ALLOC(c->d_tstate, sizeof(unsigned char) * n_samples * n_replicas * n_temps);
   HSG_ALLOC(c->d_tunnel, sizeof(unsigned int) * n_samples * n_replicas * n_temps);
 #undef HSG_ALLOC
+  if (c->dec_once) try_dec2(c);
 
   std::vector<double> inv(n_samples * (size_t)n_temps);
   std::vector<float> beta(n_samples * (size_t)Wp, 1.0f);
@@ -1528,7 +1571,7 @@ hsg_status hsg_sweep_hb(hsg_ctx* c, int n) {
   if (n == 0) return HSG_OK;
   HSG_CUDA(c, cudaSetDevice(c->device));
   c->e_valid = false;
-  c->dec_fresh = false;
+  HSG_TRY(begin_sweeps(c));
   for (int k = 0; k < n; ++k) HSG_TRY(half_sweeps(c, true, k));
   HSG_CUDA(c, launch_bump(c->d_counters, c->d_active, c->ns, n, 0, c->stream));
   return HSG_OK;
@@ -2046,6 +2089,7 @@ hsg_status hsg_get_info(hsg_ctx* c, hsg_info* info) {
   info->wave_lag = c->use_wave ? c->wave_lag : 0;
   info->fused_band_rows = c->fused_ny.empty() ? 0 : c->fused_ny[0];
   info->fused_items = c->n_fused_items;
+  info->decoded_parities = c->dec_once ? (c->dec2 ? 2 : 1) : 0;
   return HSG_OK;
 }
 
@@ -2109,12 +2153,12 @@ void hsg_destroy(hsg_ctx* c) {
   if (!c) return;
   cudaSetDevice(c->device);
   if (c->stream) cudaStreamSynchronize(c->stream);
-  if (c->graph_exec) cudaGraphExecDestroy(c->graph_exec);
-  if (c->graph) cudaGraphDestroy(c->graph);
+  drop_graph(c);
   if (c->side) cudaStreamDestroy(c->side);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_join) cudaEventDestroy(c->ev_join);
   for (void* p : c->allocations) cudaFree(p);
+  if (c->dec2) cudaFree(c->dec2);
   if (c->results) cudaFreeHost(c->results);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
   delete c;

@@ -57,7 +57,8 @@ class Info(ctypes.Structure):
                 ("n_passes", ctypes.c_int), ("pass_bytes", ctypes.c_longlong),
                 ("n_overlap_pairs", ctypes.c_int), ("sweep_kernel", ctypes.c_int),
                 ("fused_band_rows", ctypes.c_int), ("fused_items", ctypes.c_int),
-                ("wave_lag", ctypes.c_int), ("staged", ctypes.c_int)]
+                ("wave_lag", ctypes.c_int), ("staged", ctypes.c_int),
+                ("decoded_parities", ctypes.c_int)]
 
 
 _lib = None
