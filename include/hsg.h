@@ -101,6 +101,13 @@ typedef struct {
                                barrier of the next persistent launch, so the others time out,
                                or (wave sweep, outside hsg_step) makes one odd block of the next
                                hsg_sweep_or launch wait for a flag that no block sets */
+  int step_branches;        /* passes (pass_bytes) of a two-pass step in flight together: 1 = one
+                               after the other, 2 = the even and the odd passes on two branches
+                               of the step's graph, with the half-sweep and the staged kernel
+                               (the others, a single pass and the persistent schedule run one
+                               branch); pass_bytes 0 then means two halves of the systems.  0
+                               (default): chosen by the automatic schedule, one for an
+                               explicit variant.  Results do not depend on it. */
   long long pass_bytes;     /* system blocking of hsg_step: the systems are cut into passes
                                (ranges of 4-system chunks, samples kept whole where they fit)
                                of at most this many bytes of spins plus couplings, and each
@@ -151,8 +158,8 @@ enum {
   HSG_SWEEP_STAGED = 4,       /* one launch per half-sweep, neighbour rows staged in shared memory */
   HSG_SWEEP_RESIDENT = 5      /* hsg_info only (not an option): hsg_step runs all sweeps of a step in
                                  one launch, each pair of systems in the shared memory of one block;
-                                 where every L <= 12 and no sweep kernel, pass footprint or chunks
-                                 per thread is asked for.  hsg_sweep_or then uses HSG_SWEEP_HALF. */
+                                 where every L <= 12 and no sweep kernel, pass footprint, chunks per
+                                 thread or branches are asked for.  hsg_sweep_or then uses HSG_SWEEP_HALF. */
 };
 
 enum {
@@ -352,6 +359,7 @@ typedef struct {
   int fused_items;         /* fused sweep: work items (columns of planes) per launch */
   int wave_lag;            /* wave sweep: the lag in use (even blocks) */
   int staged;              /* nonzero: the over-relaxation sweep stages its neighbour rows */
+  int step_branches;       /* branches of a step's graph that its passes run on (1 or 2) */
   int decoded_parities;    /* packed formats: parities whose spins are kept decoded from one
                               half-sweep to the next (2), or 1 where memory is short for
                               that; 0 for the other formats */

@@ -954,7 +954,8 @@ hsg_status configure_schedule(hsg_ctx* c, int variant, int gpt, long long pass_b
   HSG_CUDA(c, cudaStreamSynchronize(c->stream));
   drop_graph(c);
   c->variant = variant;
-  c->chains = chains;
+  // (the fused sweep runs in one pass; the wave sweep's tickets serve one launch at a time)
+  c->chains = sweep == HSG_SWEEP_HALF || sweep == HSG_SWEEP_STAGED ? chains : 1;
   // the fused over-relaxation sweep serves the two-pass schedule in one pass,
   // the wave sweep the two-pass schedule with any passes
   c->use_fused = false;
@@ -1044,12 +1045,17 @@ hsg_status copy_chain_state(hsg_ctx* c, unsigned char* host, bool to_host) {
 }
 
 // Whether the resident sweeps can serve hsg_step: every lattice within a block's
-// threads, some sweeps, and no sweep kernel, pass footprint or chunks per thread
-// asked for.
+// threads, some sweeps, and no sweep kernel, pass footprint, chunks per thread or
+// number of branches asked for.
 bool resident_possible(const hsg_ctx* c) {
   return c->Lmax * c->Lmax * c->Lmax / 2 <= RES_MAX_HALF_SITES &&
          c->opt.n_hb_per_step + c->opt.n_or_per_step > 0 && c->opt.sweep_kernel == HSG_SWEEP_AUTO &&
-         c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0;
+         c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 && c->opt.step_branches == 0;
+}
+
+// Footprint of the passes that are halves of the systems.
+long long half_footprint(const hsg_ctx* c) {
+  return (long long)(c->spin_bytes + 1) / 2 + (long long)c->rec_bytes;
 }
 
 // Autotuner: the schedules, sweep kernels and chunks-per-thread settings
@@ -1074,7 +1080,8 @@ std::string tune_key(hsg_ctx* c) {
                   std::to_string(c->opt.n_hb_per_step) + "/" + std::to_string(c->opt.n_or_per_step) +
                   "/" + std::to_string(c->opt.pass_bytes) + "/" +
                   std::to_string(c->opt.chunks_per_thread) + "/" +
-                  std::to_string(c->opt.sweep_kernel) + "/" + std::to_string(c->opt.wave_lag) + "/L";
+                  std::to_string(c->opt.sweep_kernel) + "/" + std::to_string(c->opt.wave_lag) + "/" +
+                  std::to_string(c->opt.step_branches) + "/L";
   for (int L : c->L) k += std::to_string(L) + ",";
   return k;
 }
@@ -1172,7 +1179,9 @@ hsg_status autotune(hsg_ctx* c) {
     }
     return HSG_OK;
   };
+  const bool two_branches = c->opt.step_branches == 2 && sk != HSG_SWEEP_FUSED && sk != HSG_SWEEP_WAVE;
   for (long long pb : budgets) {
+    if (two_branches) break;   // asked for
     for (int v : {HSG_VARIANT_TWO_PASS, HSG_VARIANT_PERSISTENT}) {
       for (const auto& sw : sweeps) {
         // the fused sweep runs in the two-pass schedule with one pass only, the
@@ -1192,14 +1201,20 @@ hsg_status autotune(hsg_ctx* c) {
   // half the cache in flight, 2694 with two of that size, 2362 with two of a quarter;
   // L = 64 in FP16: 404, 388 and 347; three and four branches no faster).  The chunks
   // per thread are tried anew: smaller passes want fewer.
-  if (c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 && bestc.variant == HSG_VARIANT_TWO_PASS &&
-      (bestc.sweep == HSG_SWEEP_HALF || (bestc.sweep == HSG_SWEEP_STAGED && sk == HSG_SWEEP_AUTO))) {
-    for (int g : {bestc.gpt, (bestc.gpt + 1) / 2, 2 * bestc.gpt})
-      if (g <= c->G && std::find(gpts.begin(), gpts.end(), g) == gpts.end()) gpts.push_back(g);
-    for (size_t k = 1; k < budgets.size(); ++k) budgets[k] /= 2;
-    budgets[0] = (long long)(c->spin_bytes + 1) / 2 + (long long)c->rec_bytes;
+  if (two_branches ||
+      (c->opt.step_branches == 0 && c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 &&
+       bestc.variant == HSG_VARIANT_TWO_PASS &&
+       (bestc.sweep == HSG_SWEEP_HALF || (bestc.sweep == HSG_SWEEP_STAGED && sk == HSG_SWEEP_AUTO)))) {
+    if (c->opt.chunks_per_thread == 0)
+      for (int g : {bestc.gpt, (bestc.gpt + 1) / 2, 2 * bestc.gpt})
+        if (g <= c->G && std::find(gpts.begin(), gpts.end(), g) == gpts.end()) gpts.push_back(g);
+    if (c->opt.pass_bytes == 0) {
+      for (size_t k = 1; k < budgets.size(); ++k) budgets[k] /= 2;
+      budgets[0] = half_footprint(c);
+    }
+    const int kernel = sk == HSG_SWEEP_STAGED && c->staged_possible ? HSG_SWEEP_STAGED : HSG_SWEEP_HALF;
     for (long long pb : budgets)
-      for (int g : gpts) HSG_TRY(time_candidate({HSG_VARIANT_TWO_PASS, g, pb, HSG_SWEEP_HALF, 0, 2}));
+      for (int g : gpts) HSG_TRY(time_candidate({HSG_VARIANT_TWO_PASS, g, pb, kernel, 0, 2}));
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1240,6 +1255,8 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
   if (opt.sweep_kernel < HSG_SWEEP_AUTO || opt.sweep_kernel > HSG_SWEEP_STAGED)
     return bad_arg(nullptr, "unknown sweep_kernel");
   if (opt.wave_lag < 0) return bad_arg(nullptr, "wave_lag < 0");
+  if (opt.step_branches < 0 || opt.step_branches > 2)
+    return bad_arg(nullptr, "step_branches must be in [0, 2]");
   if (opt.inject_alloc_fault < 0) return bad_arg(nullptr, "inject_alloc_fault < 0");
   const int W = n_temps * n_replicas;
   if (W > 1024) return bad_arg(nullptr, "n_temps * n_replicas must be <= 1024");
@@ -1505,7 +1522,9 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
     // the two-pass schedule as an explicit choice: resident where possible (the
     // tuner, for an automatic one, times it against the others)
     if (opt.variant == HSG_VARIANT_TWO_PASS && resident_possible(c)) sweep = HSG_SWEEP_RESIDENT;
-    hsg_status st2 = configure_schedule(c, want, c->GPT, opt.pass_bytes, sweep, opt.wave_lag);
+    const int chains = opt.step_branches == 2 ? 2 : 1;
+    hsg_status st2 = configure_schedule(c, want, c->GPT, opt.pass_bytes == 0 && chains == 2 ? half_footprint(c) : opt.pass_bytes,
+                                        sweep, opt.wave_lag, chains);
     if (st2 != HSG_OK) return cleanup_fail(st2);
   }
   ConvParams cp = conv_params(c, nullptr, nullptr);
@@ -2089,6 +2108,7 @@ hsg_status hsg_get_info(hsg_ctx* c, hsg_info* info) {
   info->wave_lag = c->use_wave ? c->wave_lag : 0;
   info->fused_band_rows = c->fused_ny.empty() ? 0 : c->fused_ny[0];
   info->fused_items = c->n_fused_items;
+  info->step_branches = c->variant == HSG_VARIANT_TWO_PASS && c->chains == 2 && c->pass_bound.size() > 2 ? 2 : 1;
   info->decoded_parities = c->dec_once ? (c->dec2 ? 2 : 1) : 0;
   return HSG_OK;
 }

@@ -36,6 +36,7 @@ class Options(ctypes.Structure):
                 ("n_hb_per_step", ctypes.c_int), ("n_or_per_step", ctypes.c_int),
                 ("device", ctypes.c_int), ("stream", ctypes.c_void_p), ("variant", ctypes.c_int),
                 ("barrier_timeout_ms", ctypes.c_int), ("inject_barrier_fault", ctypes.c_int),
+                ("step_branches", ctypes.c_int),
                 ("pass_bytes", ctypes.c_longlong), ("chunks_per_thread", ctypes.c_int),
                 ("sweep_kernel", ctypes.c_int), ("wave_lag", ctypes.c_int),
                 ("inject_alloc_fault", ctypes.c_int)]
@@ -58,7 +59,7 @@ class Info(ctypes.Structure):
                 ("n_overlap_pairs", ctypes.c_int), ("sweep_kernel", ctypes.c_int),
                 ("fused_band_rows", ctypes.c_int), ("fused_items", ctypes.c_int),
                 ("wave_lag", ctypes.c_int), ("staged", ctypes.c_int),
-                ("decoded_parities", ctypes.c_int)]
+                ("step_branches", ctypes.c_int), ("decoded_parities", ctypes.c_int)]
 
 
 _lib = None
@@ -151,7 +152,7 @@ class Context:
                  device: int = 0, stream: Optional[int] = None, variant: int = VARIANT_AUTO,
                  barrier_timeout_ms: int = 2000, inject_barrier_fault: bool = False,
                  pass_bytes: int = 0, chunks_per_thread: int = 0, sweep_kernel: int = SWEEP_AUTO,
-                 wave_lag: int = 0, inject_alloc_fault: int = 0):
+                 wave_lag: int = 0, inject_alloc_fault: int = 0, step_branches: int = 0):
         L = lib()
         self._ctx = ctypes.c_void_p()
         opt = default_options()
@@ -170,6 +171,7 @@ class Context:
         opt.sweep_kernel = int(sweep_kernel)
         opt.wave_lag = int(wave_lag)
         opt.inject_alloc_fault = int(inject_alloc_fault)
+        opt.step_branches = int(step_branches)
         self.samples = list(samples)
         self.n_samples = len(self.samples)
         self.n_temps = len(self.samples[0].temps)
