@@ -628,6 +628,7 @@ hsg_status resident_sweeps(hsg_ctx* c) {
   p.n_or = c->opt.n_or_per_step;
   p.max_half_sites = c->Lmax * c->Lmax * c->Lmax / 2;
   for (int r = 0; r < 20; ++r) p.rk[r] = sp.rk[r];
+  p.bounds_err = sp.bounds_err;
   HSG_CUDA(c, launch_resident(c->fmt, c->j16, c->opt.fast_math != 0, p, c->stream));
   return HSG_OK;
 }

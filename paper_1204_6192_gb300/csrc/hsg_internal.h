@@ -306,6 +306,7 @@ struct ResidentParams {
   int Wp, n_hb, n_or;
   int max_half_sites;       // of the context's largest lattice
   uint32_t rk[20];          // Philox round keys of the seed
+  unsigned int* bounds_err; // HSG_CHECK builds: set when a device bounds check fails
 };
 cudaError_t launch_resident(int fmt, bool j16, bool fast, const ResidentParams& p, cudaStream_t st);
 

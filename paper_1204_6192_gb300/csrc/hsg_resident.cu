@@ -95,8 +95,14 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResidentParams p) {
   const SampleDev& sd = p.samples[s];
   const int L = sd.L, Lh = sd.Lh, P = L * Lh;    // half-sites of a row, of a plane
   const int HN = sd.N >> 1;
+  // HSG_CHECK builds: a thread and shared memory for every half-site, the pair within
+  // the sample (else the block leaves the pair as it is)
+  if (HSG_OUT_OF_BOUNDS(HN <= (int)blockDim.x && HN <= p.max_half_sites && 2 * pr + 2 <= p.Wp, p.bounds_err)) {
+    chain_wait();
+    return;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool live = tid < HN;
+  bool live = tid < HN;
   const int h = live ? tid : HN - 1;             // (idle threads repeat the last site, unstored)
   E* sp = reinterpret_cast<E*>(smem);            // [parity][component][HN]
   unsigned char* mine = p.spins + sd.spin_off + ((long long)(pr >> 1) * sd.N + h) * CH + (pr & 1) * (CH / 2);
@@ -108,7 +114,7 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResidentParams p) {
   const int z = (int)((__umulhi(r, sd.fdL_m) + r) >> sd.fdL_s), y = (int)r - z * L;
   const int nyp = y + 1 == L ? h + Lh - P : h + Lh, nym = y == 0 ? h - Lh + P : h - Lh;
   const int nzp = z + 1 == L ? h + P - HN : h + P, nzm = z == 0 ? h - P + HN : h - P;
-  int nxp[2], nxm[2];
+  int nxp[2], nxm[2], nyz[4] = {nyp, nym, nzp, nzm};
   float j6[2][6], h3[2][3];
   uint32_t jh[2][6];
 #pragma unroll
@@ -116,6 +122,12 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResidentParams p) {
     const bool f = (par + y + z) & 1;            // x = 2 hx + f
     nxp[par] = f ? (hx + 1 == Lh ? h + 1 - Lh : h + 1) : h;
     nxm[par] = f ? h : (hx == 0 ? h + Lh - 1 : h - 1);
+    // HSG_CHECK builds: every neighbour a half-site of the lattice (else the thread
+    // reads half-site 0 and stores nothing)
+    bool bad = false;
+    for (int* n : {&nxp[par], &nxm[par], &nyz[0], &nyz[1], &nyz[2], &nyz[3]})
+      if (HSG_OUT_OF_BOUNDS(*n >= 0 && *n < HN, p.bounds_err)) bad = true, *n = 0;
+    if (bad) live = false;
     load_record<J16>(p.rec, sd.rec_off + par * HN + h, j6[par], h3[par]);
     if (MIXED) load_record_j16(p.rec, sd.rec_off + par * HN + h, jh[par]);
   }
@@ -144,7 +156,7 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResidentParams p) {
 #pragma unroll
     for (int par = 0; par < 2; ++par) {
       const E* O = sp + (1 - par) * 3 * HN;
-      const int nb[6] = {nxp[par], nxm[par], nyp, nym, nzp, nzm};
+      const int nb[6] = {nxp[par], nxm[par], nyz[0], nyz[1], nyz[2], nyz[3]};
       E nv[6][3];
 #pragma unroll
       for (int n = 0; n < 6; ++n)
