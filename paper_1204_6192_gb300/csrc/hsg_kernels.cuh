@@ -64,7 +64,10 @@ __device__ __forceinline__ void sweep_block(const SweepParams& p, int bidx, floa
       bad = bad || HSG_OUT_OF_BOUNDS(gm.nb[n] >= nb0 && gm.nb[n] < nb0 + half_n, p.bounds_err);
     if (bad) {
       active = false;
-      if (!EN) return;
+      if (!EN) {
+        if (CHAINED) chain_wait();   // (every block waits, also one that fails all over)
+        return;
+      }
       gm.own = own0;
 #pragma unroll
       for (int n = 0; n < 6; ++n) gm.nb[n] = nb0;
