@@ -1072,6 +1072,10 @@ struct TuneChoice {
   int sweep, lag, chains;
 };
 constexpr int TUNE_REPS = 5;
+// (the first step of a new shape: L = 64, FP16, 64 systems 414 ms without the cut and the
+// two-branch candidates, 456 with these, 264 with both; 512 samples of L = 8 to 24 1301,
+// 1651, 896; the same choices)
+constexpr float TUNE_CUT = 1.2f;
 std::mutex g_tune_mu;
 std::map<std::string, TuneChoice> g_tune_cache;
 
@@ -1158,7 +1162,8 @@ hsg_status autotune(hsg_ctx* c) {
   // one warm-up step, then the median of TUNE_REPS timings of two steps; a
   // candidate replaces the current choice only when it is at least 1% faster, so that
   // timing noise between near-equal candidates does not decide (candidates are tried
-  // simplest first)
+  // simplest first).  One whose first timing is TUNE_CUT times the best median is
+  // not timed again.
   auto time_candidate = [&](const TuneChoice& t) -> hsg_status {
     HSG_TRY(configure_schedule(c, t.variant, t.gpt, t.pass_bytes, t.sweep, t.lag, t.chains));
     if (t.sweep == HSG_SWEEP_FUSED && !c->use_fused) return HSG_OK;
@@ -1166,6 +1171,7 @@ hsg_status autotune(hsg_ctx* c) {
     HSG_TRY(run_steps(c, 1));
     float ms[TUNE_REPS];
     for (int r = 0; r < TUNE_REPS; ++r) {
+      if (r == 1 && ms[0] > TUNE_CUT * best) return poll_device_error(c);
       HSG_CUDA(c, cudaEventRecord(e0, st));
       HSG_TRY(run_steps(c, 2));
       HSG_CUDA(c, cudaEventRecord(e1, st));
