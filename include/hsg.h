@@ -159,7 +159,8 @@ enum {
   HSG_SWEEP_RESIDENT = 5      /* hsg_info only (not an option): hsg_step runs all sweeps of a step in
                                  one launch, each pair of systems in the shared memory of one block;
                                  where every L <= 12 and no sweep kernel, pass footprint, chunks per
-                                 thread or branches are asked for.  hsg_sweep_or then uses HSG_SWEEP_HALF. */
+                                 thread or branches are asked for (an explicit two-pass schedule:
+                                 where L <= 8 or the systems are few).  hsg_sweep_or then uses HSG_SWEEP_HALF. */
 };
 
 enum {

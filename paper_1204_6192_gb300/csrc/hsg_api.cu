@@ -1054,6 +1054,20 @@ bool resident_possible(const hsg_ctx* c) {
          c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 && c->opt.step_branches == 0;
 }
 
+// The two-pass schedule as an explicit choice, which no timing stands behind: resident
+// where that wins or ties for every storage format.  Up to L = 8 at any number of systems;
+// above, with one block an SM (L = 10 and 12), up to three rounds of blocks, i.e. while
+// launches and latency count (L = 10, FP16, us a step, half-sweeps and resident: 38 and 22
+// with 64 blocks, 51 and 35 with 256, 87 and 99 with 1024, 487 and 700 with 8192; L = 12,
+// FP16 57 and 49, 141 and 145, 826 and 1051; FP32 64 and 55, 172 and 168, 1161 and 1230;
+// L = 8, FP16 40 and 20, 57 and 41, 228 and 229).
+hsg_status resident_untimed(hsg_ctx* c, bool* use) {
+  int n_sm = 0;
+  HSG_CUDA(c, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device));
+  *use = resident_possible(c) && (c->Lmax <= 8 || (long long)c->ns * (c->Wp / 2) <= 3ll * n_sm);
+  return HSG_OK;
+}
+
 // Footprint of the passes that are halves of the systems.
 long long half_footprint(const hsg_ctx* c) {
   return (long long)(c->spin_bytes + 1) / 2 + (long long)c->rec_bytes;
@@ -1526,12 +1540,13 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
       c->Lh_max = std::max(c->Lh_max, L[s] / 2);
     }
     int sweep = opt.sweep_kernel == HSG_SWEEP_AUTO ? HSG_SWEEP_HALF : opt.sweep_kernel;
-    // the two-pass schedule as an explicit choice: resident where possible (the
-    // tuner, for an automatic one, times it against the others)
-    if (opt.variant == HSG_VARIANT_TWO_PASS && resident_possible(c)) sweep = HSG_SWEEP_RESIDENT;
     const int chains = opt.step_branches == 2 ? 2 : 1;
-    hsg_status st2 = configure_schedule(c, want, c->GPT, opt.pass_bytes == 0 && chains == 2 ? half_footprint(c) : opt.pass_bytes,
-                                        sweep, opt.wave_lag, chains);
+    bool resident = false;
+    hsg_status st2 = opt.variant == HSG_VARIANT_TWO_PASS ? resident_untimed(c, &resident) : HSG_OK;
+    if (resident) sweep = HSG_SWEEP_RESIDENT;
+    if (st2 == HSG_OK)
+      st2 = configure_schedule(c, want, c->GPT, opt.pass_bytes == 0 && chains == 2 ? half_footprint(c) : opt.pass_bytes,
+                               sweep, opt.wave_lag, chains);
     if (st2 != HSG_OK) return cleanup_fail(st2);
   }
   ConvParams cp = conv_params(c, nullptr, nullptr);

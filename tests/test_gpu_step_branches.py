@@ -93,3 +93,13 @@ def test_schedules_without_branches():
     for bad in (-1, 3):
         with pytest.raises(hsg.HsgError, match="step_branches"):
             hsg.Context([smp], 2, 1, step_branches=bad)
+
+
+@pytest.mark.parametrize("L,n_samples,kernel", [(8, 64, 5), (10, 8, 5), (12, 28, 5), (12, 32, 1), (10, 64, 1)])
+def test_explicit_two_pass_takes_the_resident_sweeps_where_they_win(L, n_samples, kernel):
+    """No timing stands behind an explicit schedule: resident up to L = 8, above only with
+    few systems (32 a sample here), where launches and latency count."""
+    samples = [inputs.small_sample(L, n_temps=16, disorder_seed=k) for k in range(2)] * (n_samples // 2)
+    ctx = hsg.Context(samples, 2, 3, precision="fp16", variant=hsg.VARIANT_TWO_PASS)
+    assert ctx.info().sweep_kernel == kernel
+    ctx.close()
