@@ -1220,12 +1220,14 @@ hsg_status autotune(hsg_ctx* c) {
   // systems, and half the footprints above, so that the two passes in flight fit the
   // L2 cache together (512 samples of L = 8 to 24: 2631 us a step with one pass of
   // half the cache in flight, 2694 with two of that size, 2362 with two of a quarter;
-  // L = 64 in FP16: 404, 388 and 347; three and four branches no faster).  The chunks
+  // L = 64 in FP16: 404, 388 and 347; three and four branches no faster; also where the
+  // resident sweeps lead so far: 256 samples of L = 12, 32 systems, FP32 580, 467).  The chunks
   // per thread are tried anew: smaller passes want fewer.
   if (two_branches ||
       (c->opt.step_branches == 0 && c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 &&
        bestc.variant == HSG_VARIANT_TWO_PASS &&
-       (bestc.sweep == HSG_SWEEP_HALF || (bestc.sweep == HSG_SWEEP_STAGED && sk == HSG_SWEEP_AUTO)))) {
+       (bestc.sweep == HSG_SWEEP_HALF || bestc.sweep == HSG_SWEEP_RESIDENT ||
+        (bestc.sweep == HSG_SWEEP_STAGED && sk == HSG_SWEEP_AUTO)))) {
     if (c->opt.chunks_per_thread == 0)
       for (int g : {bestc.gpt, (bestc.gpt + 1) / 2, 2 * bestc.gpt})
         if (g <= c->G && std::find(gpts.begin(), gpts.end(), g) == gpts.end()) gpts.push_back(g);
