@@ -441,14 +441,15 @@ __device__ __forceinline__ void or_move2(float2& sx, float2& sy, float2& sz, flo
   if (hh.y > 0.0f) { sx.y = nx.y; sy.y = ny.y; sz.y = nz.y; }
 }
 
-// The same where it may branch: with h.h of both systems a normal number below 2^125
-// the quotient needs no scaling of subnormal operands and h = 0 no selection, and
-// -s' = s - 2 (s.h)/(h.h) h spares the negations.  The values are or_move2's bit for
-// bit (a subnormal quotient and the sign of a component that cancels to zero apart).
-// A sixth fewer instructions, but two basic blocks more: the staged sweep, whose
-// neighbours are in shared memory by then, gains (L = 128, FP16: 2198 -> 2151 us a
-// step); the one that loads into registers loses (512 samples of L = 8 to 24 in
-// binary32: 2357 -> 2392), since its loads are not moved over the branches.
+// The same, bit for bit, where it may branch: with h.h of both systems a normal number
+// below 2^125 there is no h = 0 to select for and the quotient is 2 (s.h) times the
+// hardware's reciprocal (as PTX defines div.approx, without the scaling it needs for a
+// subnormal divisor; equal to __fdividef for 3 x 2^32 random pairs, subnormal s.h and
+// quotients among them).  Fewer instructions, but two basic blocks more: the staged sweep,
+// whose neighbours are in shared memory by then, gains in 16-bit formats (L = 128, 48
+// systems, a sweep: FP16 307 -> 299 us, BF16 320 -> 311; FP32 576 either way); the one that
+// loads into registers loses (512 samples of L = 8 to 24 in binary32: 2357 -> 2392 us a
+// step), since its loads are not moved over the branches.
 __device__ __forceinline__ void or_move2_branch(float2& sx, float2& sy, float2& sz, float2 hx,
                                                 float2 hy, float2 hz) {
   const float2 hh = dot3_2(hx, hy, hz, hx, hy, hz);
@@ -457,18 +458,15 @@ __device__ __forceinline__ void or_move2_branch(float2& sx, float2& sy, float2& 
     or_move2(sx, sy, sz, hx, hy, hz);
     return;
   }
-  const float2 t = mul2(dot3_2(sx, sy, sz, hx, hy, hz), f2(-2.0f));
-  float2 f;
-  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(f.x) : "f"(t.x), "f"(hh.x));
-  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(f.y) : "f"(t.y), "f"(hh.y));
-  sx = fma2(f, hx, sx);
-  sy = fma2(f, hy, sy);
-  sz = fma2(f, hz, sz);
-  const float2 n2 = dot3_2(sx, sy, sz, sx, sy, sz);
-  const float2 inv = make_float2(-rsqrtf(n2.x), -rsqrtf(n2.y));
-  sx = mul2(sx, inv);
-  sy = mul2(sy, inv);
-  sz = mul2(sz, inv);
+  const float2 sh = dot3_2(sx, sy, sz, hx, hy, hz);
+  float2 r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(hh.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(hh.y));
+  const float2 f = mul2(add2(sh, sh), r);
+  sx = fma2(f, hx, neg2(sx));
+  sy = fma2(f, hy, neg2(sy));
+  sz = fma2(f, hz, neg2(sz));
+  normalize2(sx, sy, sz);
 }
 
 // (sin, cos) of 2 pi u for a uniform u in (0, 1), for one system or a pair.

@@ -1,5 +1,6 @@
 """Every step schedule and over-relaxation kernel gives the same bits: the energies'
-FP64 sums are taken in one order."""
+FP64 sums are taken in one order, and a move leaves the same spins down to the sign of
+a zero component."""
 import numpy as np
 import pytest
 
@@ -61,3 +62,48 @@ def test_resident_energies_are_summed_in_the_same_order(Ls, precision):
     E = [energies(samples, 3, kw, 3, precision=precision) for kw in (HALF, resident, PERSISTENT)]
     np.testing.assert_array_equal(E[1], E[0])
     np.testing.assert_array_equal(E[2], E[0])
+
+
+# unit vectors with zero components of both signs
+UNITS = np.array([[1, 0, 0], [0, 1, 0], [0, 0, 1], [0.6, 0.8, 0], [0, -0.6, 0.8], [-0.8, 0, 0.6]])
+UNITS = np.concatenate([UNITS, -UNITS, UNITS * np.where(UNITS == 0, -1, 1)])
+
+
+def structured(L, kind, seed):
+    """Couplings and fields among a few values, so that local fields vanish, lie along the
+    axes, or stand at right angles to the spins up to tiny components."""
+    rng = np.random.default_rng(seed)
+    values = {"axes": [1.0, -1.0, 0.0, 0.5], "tiny": [1.0, -1.0, 0.0, 1e-20, -1e-30, 1e-38, -3e-39],
+              "wide": [1.0, 1e-18, -1e17, 3e-25, 0.0, -2e-12]}[kind]
+    J = rng.choice(values, (L ** 3, 3))
+    H = UNITS[rng.integers(len(UNITS), size=L ** 3)] * rng.choice(values, (L ** 3, 1))
+    spins = UNITS[rng.integers(len(UNITS), size=(6, L ** 3))]
+    if kind == "axes":          # half of the systems ordered
+        spins[::2] = UNITS[rng.integers(len(UNITS), size=3)][:, None]
+    return inputs.Sample(L=L, J=J, H=H if seed % 2 else None, temps=np.array([0.5, 1.0, 2.0])), spins.astype(np.float32)
+
+
+@pytest.mark.parametrize("seed", [0, 1])
+@pytest.mark.parametrize("kind", ["axes", "tiny", "wide"])
+@pytest.mark.parametrize("L,precision", [(8, "fp32"), (8, "fp16"), (32, "fp32"), (32, "fp16"),
+                                         (32, "fp16j"), (32, "bf16"), (64, "fp32"), (64, "fp16")])
+def test_moves_leave_the_same_bits(L, precision, kind, seed):
+    """Spins and fields with zero components, zero, subnormal and far apart fields:
+    over-relaxation by every kernel, and steps by every schedule, the sign of zeros
+    included."""
+    smp, spins = structured(L, kind, seed)
+    ways = [HALF, PERSISTENT, {"variant": hsg.VARIANT_TWO_PASS, "sweep_kernel": hsg.SWEEP_FUSED},
+            {"variant": hsg.VARIANT_TWO_PASS, "sweep_kernel": hsg.SWEEP_WAVE}]
+    ways.append({"variant": hsg.VARIANT_TWO_PASS, "sweep_kernel": hsg.SWEEP_STAGED if L >= 32 else hsg.SWEEP_AUTO})
+    out = []
+    for kw in ways:
+        ctx = hsg.Context([smp], 2, 5, precision=precision[:4], j_fp16=precision == "fp16j", n_hb=0, n_or=3, **kw)
+        ctx.set_spins([spins])
+        ctx.sweep_or(2)
+        a = ctx.get_spins()[0].copy()
+        ctx.step(1)
+        out.append((a, ctx.get_spins()[0].copy()))
+        ctx.close()
+    for kw, o in zip(ways[1:], out[1:]):
+        for x, ref in zip(o, out[0]):
+            np.testing.assert_array_equal(x.view(np.uint32), ref.view(np.uint32), err_msg=str(kw))
