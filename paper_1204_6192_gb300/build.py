@@ -20,8 +20,8 @@ LIB = os.path.join(HERE, "libhsg.so")
 BUILD_CHECK = os.path.join(HERE, "_build_check")
 LIB_CHECK = os.path.join(HERE, "libhsg_check.so")
 SOURCES = ["hsg_api.cu", "hsg_sweep.cu", "hsg_aux.cu", "hsg_persist.cu", "hsg_noalloc.cu",
-           "hsg_overlap.cu", "hsg_multihit.cu", "hsg_fused.cu", "hsg_wave.cu",
-           "hsg_resident.cu"]
+           "hsg_overlap.cu", "hsg_multihit.cu", "hsg_fused.cu", "hsg_staged.cu",
+           "hsg_staged_mixed.cu", "hsg_wave.cu", "hsg_resident.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -130,7 +130,8 @@ struct hsg_ctx {
   // of the wave sweep where possible, or of two half-sweep launches)
   bool staged_possible = false;         // format and every L allow it
   bool use_staged = false;              // HSG_SWEEP_STAGED in use
-  int Lh_max = 0;
+  int stage_bytes = 0;                  // shared memory of a stage: the most of the lattices
+  int one_Lh = 0;                       // L / 2 of every sample; 0: not all alike
   int wave_lag = 0;                     // lag in use (even blocks)
   int* d_wave_order = nullptr;          // [2 max_sweep_blocks] ticket order of every pass
   int4* d_wave_deps = nullptr;          // [max_sweep_blocks] even-block ranges of each odd block
@@ -312,7 +313,7 @@ SweepParams sweep_params(hsg_ctx* c, int parity, int sweep_offset) {
   p.reverse = 0;
   p.dec = c->dec2 && parity == 0 ? c->dec2 : c->dec;
   p.dec_out = !c->dec2 ? nullptr : parity == 0 ? c->dec : c->dec2;
-  p.stage_bytes = c->staged_possible ? staged_stage_bytes(c->fmt, c->Lh_max, false) : 0;
+  p.one_Lh = c->one_Lh;
   p.stage_off = 0;
   p.err = c->d_bar + 5;
   p.bounds_err = c->d_bar + 6;
@@ -393,17 +394,15 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
                        int b1 = -1) {
   if (b1 < 0) b1 = c->n_sweep_blocks;
   if (!hb && c->use_staged) {
-    const bool one_L = std::all_of(c->L.begin(), c->L.end(), [&](int L) { return L == c->L[0]; });
     int off = 0;
-    const size_t smem = staged_smem(c->fmt, c->GPT, energy, c->Lh_max, one_L, &off);
+    const size_t smem = staged_smem(c->GPT, energy, c->stage_bytes, &off);
     for (int parity = 0; parity < 2; ++parity) {
       SweepParams p = sweep_params(c, parity, sweep_offset);
       p.blk_base = b0;
       p.n_launch = b1 - b0;
       p.reverse = parity;
       p.stage_off = off;
-      HSG_CUDA(c, launch_staged_half(c->fmt, c->j16, energy, one_L ? c->Lh_max : 0, p, b1 - b0, smem,
-                                     c->stream));
+      HSG_CUDA(c, launch_staged_half(c->fmt, c->j16, energy, p, b1 - b0, smem, c->stream));
     }
     return HSG_OK;
   }
@@ -413,7 +412,7 @@ hsg_status half_sweeps(hsg_ctx* c, bool hb, int sweep_offset, bool energy = fals
     WaveParams w;
     w.sw = sweep_params(c, 0, sweep_offset);
     int off = 0;
-    size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, energy, c->Lh_max, false, &off)
+    size_t smem = c->staged_possible ? staged_smem(c->GPT, energy, c->stage_bytes, &off)
                                      : (energy ? sizeof(float) * (SWEEP_BS / 32) * c->GPT * c->VEC : 0);
     w.sw.stage_off = off;
     w.order = c->d_wave_order;
@@ -813,7 +812,7 @@ hsg_status plan_wave(hsg_ctx* c, const std::vector<int4>& blocks, int lag) {
   }
   if (lag <= 0) {
     int per_sm = 0, n_sm = 0, off = 0;
-    const size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, false, c->Lh_max, false, &off) : 0;
+    const size_t smem = c->staged_possible ? staged_smem(c->GPT, false, c->stage_bytes, &off) : 0;
     HSG_CUDA(c, wave_occupancy(c->fmt, c->j16, c->staged_possible, smem, &per_sm));
     HSG_CUDA(c, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device));
     lag = std::max(1, n_sm * per_sm / 2);
@@ -1142,7 +1141,7 @@ hsg_status autotune(hsg_ctx* c) {
       sweeps.push_back({HSG_SWEEP_WAVE, c->opt.wave_lag});
     } else {
       int per_sm = 0, n_sm = 0, off = 0;
-      const size_t smem = c->staged_possible ? staged_smem(c->fmt, c->GPT, false, c->Lh_max, false, &off) : 0;
+      const size_t smem = c->staged_possible ? staged_smem(c->GPT, false, c->stage_bytes, &off) : 0;
       HSG_CUDA(c, wave_occupancy(c->fmt, c->j16, c->staged_possible, smem, &per_sm));
       HSG_CUDA(c, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device));
       const int resident = std::max(4, n_sm * per_sm);
@@ -1537,9 +1536,10 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
       if (L[s] % 4 != 0 || L[s] < 8) c->fused_possible = false;
     c->wave_possible = fmt_has_wave(fmt);
     c->staged_possible = c->wave_possible;
+    c->one_Lh = std::all_of(L, L + n_samples, [&](int l) { return l == L[0]; }) ? L[0] / 2 : 0;
     for (int s = 0; s < n_samples; ++s) {
       c->staged_possible = c->staged_possible && lattice_has_staged(L[s]);
-      c->Lh_max = std::max(c->Lh_max, L[s] / 2);
+      if (c->staged_possible) c->stage_bytes = std::max(c->stage_bytes, staged_stage_bytes(fmt, L[s]));
     }
     int sweep = opt.sweep_kernel == HSG_SWEEP_AUTO ? HSG_SWEEP_HALF : opt.sweep_kernel;
     const int chains = opt.step_branches == 2 ? 2 : 1;

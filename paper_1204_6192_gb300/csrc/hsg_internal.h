@@ -94,9 +94,9 @@ struct SweepParams {
   uint32_t rk[20];          // Philox round keys of the seed
   const unsigned char* dec; // packed formats: the opposite parity as binary32 (see SampleDev)
   unsigned char* dec_out;   // packed formats: where the updated spins go as binary32 (null: nowhere)
-  // staged sweeps (hsg_wave.cu): bytes of one stage of rows, offset of
+  // staged sweeps (hsg_staged.cuh): L / 2 of every sample (0: not all alike), offset of
   // stage 0 in dynamic shared memory, the error word of their bounded waits
-  int stage_bytes, stage_off;
+  int one_Lh, stage_off;
   unsigned int* err;
   unsigned long long timeout_ns;
   unsigned int* bounds_err;  // HSG_CHECK builds: set when a device bounds check fails
@@ -274,22 +274,24 @@ struct WaveParams {
 bool fmt_has_wave(int fmt);
 // Staged sweeps: every block copies the opposite-parity rows its sites read
 // (plane z: rows y0-1 .. y0+R, planes z-1 and z+1: rows y0 .. y0+R-1; R = 256 /
-// (L/2)) and its own rows into a two-stage shared-memory ring with cp.async.bulk, one chunk group
-// per stage.  Possible for every sample with L a power of 2, L >= 32.
+// (L/2)) and, up to L = 128, its own rows into a two-stage shared-memory ring with
+// cp.async.bulk, one chunk group per stage.  Possible where every L is a power of 2, L >= 32.
 constexpr int STAGED_STAGES = 2;
 constexpr int STAGED_HEAD = 256;          // mbarriers
 bool lattice_has_staged(int L);
-int staged_stage_bytes(int fmt, int Lh_max, bool own);
-// (one_L: every sample has this L / 2 and the kernel is the half-sweep's)
-size_t staged_smem(int fmt, int gpt, bool energy, int Lh_max, bool one_L, int* stage_off);
+int staged_stage_bytes(int fmt, int L);
+// (stage_bytes: the most of the context's lattices)
+size_t staged_smem(int gpt, bool energy, int stage_bytes, int* stage_off);
 // blocks per SM of the wave kernel (staged: with that dynamic shared memory)
 cudaError_t wave_occupancy(int fmt, bool j16, bool staged, size_t smem, int* blocks_per_sm);
 cudaError_t launch_wave(int fmt, bool j16, bool energy, bool staged, const WaveParams& p, size_t smem,
                         cudaStream_t st);
-// one half-sweep (p.parity) of over-relaxation with the staged block body; Lh: L / 2 if
-// every sample has the same, else 0
-cudaError_t launch_staged_half(int fmt, bool j16, bool energy, int Lh, const SweepParams& p, int n_blocks,
+// one half-sweep (p.parity) of over-relaxation with the staged block body
+cudaError_t launch_staged_half(int fmt, bool j16, bool energy, const SweepParams& p, int n_blocks,
                                size_t smem, cudaStream_t st);
+// (contexts with lattices of several sizes)
+cudaError_t launch_staged_mixed(int fmt, bool j16, bool energy, const SweepParams& p, int n_blocks,
+                                size_t smem, cudaStream_t st);
 
 // The sweeps of a step with a pair of systems' lattice resident in a block's shared
 // memory (hsg_resident.cu), for lattices of at most RES_MAX_HALF_SITES sites of a parity.
