@@ -7,8 +7,11 @@
 
 #include <algorithm>
 #include <cmath>
+#include <initializer_list>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -157,7 +160,7 @@ struct hsg_ctx {
   // grows to the largest result asked for, at most RESULT_MAX
   unsigned char* results = nullptr;
   size_t results_bytes = 0;
-  std::vector<unsigned char> results_large;   // of one call beyond RESULT_MAX, or without pinned memory
+  std::unique_ptr<unsigned char[]> results_large;   // of one call beyond RESULT_MAX, or without pinned memory
 
   hsg_status err = HSG_OK;
   std::string msg;
@@ -714,13 +717,13 @@ hsg_status poll_device_error(hsg_ctx* c) {
 // copies go to the context's pinned buffer behind the kernels, so one
 // synchronisation serves them all (copies to pageable memory each waited for the
 // stream, and the error words for another round trip).  host[k] points to the
-// bytes of the k-th source until the next call.
+// bytes of the k-th source (of no bytes: not copied) until the next call.
 constexpr size_t RESULT_MAX = 64u << 20;
 struct ResultCopy {
   const void* src;
   size_t bytes;
 };
-hsg_status fetch_results(hsg_ctx* c, const std::vector<ResultCopy>& src, const unsigned char** host) {
+hsg_status fetch_results(hsg_ctx* c, std::initializer_list<ResultCopy> src, const unsigned char** host) {
   size_t need = 64;
   for (const auto& r : src) need += (r.bytes + 63) / 64 * 64;
   if (need > c->results_bytes && need <= RESULT_MAX) {
@@ -731,13 +734,14 @@ hsg_status fetch_results(hsg_ctx* c, const std::vector<ResultCopy>& src, const u
     else cudaGetLastError();
   }
   unsigned char* buf = c->results;
-  c->results_large = std::vector<unsigned char>(need > c->results_bytes ? need : 0);
-  if (need > c->results_bytes) buf = c->results_large.data();
+  c->results_large.reset(need > c->results_bytes ? new (std::nothrow) unsigned char[need] : nullptr);
+  if (need > c->results_bytes) buf = c->results_large.get();
+  if (!buf) return fail(c, HSG_ENOMEM, "host memory for " + std::to_string(need) + " bytes of results");
   size_t off = 64;
-  for (size_t k = 0; k < src.size(); ++k) {
-    HSG_CUDA(c, cudaMemcpyAsync(buf + off, src[k].src, src[k].bytes, cudaMemcpyDeviceToHost, c->stream));
-    host[k] = buf + off;
-    off += (src[k].bytes + 63) / 64 * 64;
+  for (const auto& r : src) {
+    if (r.bytes) HSG_CUDA(c, cudaMemcpyAsync(buf + off, r.src, r.bytes, cudaMemcpyDeviceToHost, c->stream));
+    *host++ = buf + off;
+    off += (r.bytes + 63) / 64 * 64;
   }
   HSG_CUDA(c, cudaMemcpyAsync(buf, c->d_bar + 2, sizeof(unsigned int) * ERR_WORDS, cudaMemcpyDeviceToHost, c->stream));
   HSG_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -1789,15 +1793,13 @@ hsg_status hsg_measure(hsg_ctx* c, hsg_obs* o) {
   const size_t q_bytes = pairs && o->q ? sizeof(double) * c->ns * c->R_T * 9 : 0;
   const size_t qk_bytes = pairs && o->qk ? sizeof(double) * c->ns * c->R_T * 54 : 0;
   const unsigned char* host[4];
-  std::vector<ResultCopy> src{{c->d_E, sizeof(double) * c->ns * (size_t)c->Wp},
-                              {c->d_perm, sizeof(int) * c->ns * (size_t)c->R_O * c->R_T}};
-  if (q_bytes) src.push_back({c->d_q, q_bytes});
-  if (qk_bytes) src.push_back({c->d_qk, qk_bytes});
-  HSG_TRY(fetch_results(c, src, host));
+  HSG_TRY(fetch_results(c, {{c->d_E, sizeof(double) * c->ns * (size_t)c->Wp},
+                            {c->d_perm, sizeof(int) * c->ns * (size_t)c->R_O * c->R_T},
+                            {c->d_q, q_bytes}, {c->d_qk, qk_bytes}}, host));
   const double* E = reinterpret_cast<const double*>(host[0]);
   const int* perm = reinterpret_cast<const int*>(host[1]);
   if (q_bytes) std::memcpy(o->q, host[2], q_bytes);
-  if (qk_bytes) std::memcpy(o->qk, host[q_bytes ? 3 : 2], qk_bytes);
+  if (qk_bytes) std::memcpy(o->qk, host[3], qk_bytes);
   for (int s = 0; s < c->ns; ++s)
     for (int r = 0; r < c->R_O; ++r)
       for (int t = 0; t < c->R_T; ++t) {
@@ -1912,12 +1914,9 @@ hsg_status hsg_measure_overlaps(hsg_ctx* c, double* D, double* C) {
   }
   const size_t n = sizeof(double) * c->ns * (size_t)c->R_T * n_pairs;
   const unsigned char* host[2];
-  std::vector<ResultCopy> src;
-  if (D) src.push_back({c->d_D, 8 * n});
-  if (C) src.push_back({c->d_C, 24 * n});
-  HSG_TRY(fetch_results(c, src, host));
+  HSG_TRY(fetch_results(c, {{c->d_D, D ? 8 * n : 0}, {c->d_C, C ? 24 * n : 0}}, host));
   if (D) std::memcpy(D, host[0], 8 * n);
-  if (C) std::memcpy(C, host[D ? 1 : 0], 24 * n);
+  if (C) std::memcpy(C, host[1], 24 * n);
   return HSG_OK;
 }
 
