@@ -354,8 +354,8 @@ typedef struct {
   int n_passes;            /* system-blocked passes per step (1: no blocking) */
   long long pass_bytes;    /* footprint bound of a pass in use (0: one pass) */
   int n_overlap_pairs;     /* replica pairs hsg_measure_overlaps reports (0 if n_replicas < 2) */
-  int sweep_kernel;        /* HSG_SWEEP_HALF, HSG_SWEEP_FUSED, HSG_SWEEP_WAVE or
-                              HSG_SWEEP_STAGED: the over-relaxation sweep in use */
+  int sweep_kernel;        /* HSG_SWEEP_HALF, HSG_SWEEP_FUSED, HSG_SWEEP_WAVE, HSG_SWEEP_STAGED
+                              or HSG_SWEEP_RESIDENT: the over-relaxation sweep in use */
   int fused_band_rows;     /* fused sweep: rows of y per block of sample 0 (L: whole planes) */
   int fused_items;         /* fused sweep: work items (columns of planes) per launch */
   int wave_lag;            /* wave sweep: the lag in use (even blocks) */

@@ -447,8 +447,9 @@ __device__ __forceinline__ void or_move2(float2& sx, float2& sy, float2& sz, flo
 // subnormal divisor; equal to __fdividef for 3 x 2^32 random pairs, subnormal s.h and
 // quotients among them).  Fewer instructions, but two basic blocks more: the staged sweep,
 // whose neighbours are in shared memory by then, gains in 16-bit formats (L = 128, 48
-// systems, a sweep: FP16 307 -> 299 us, BF16 320 -> 311; FP32 576 either way); the one that
-// loads into registers loses (512 samples of L = 8 to 24 in binary32: 2357 -> 2392 us a
+// systems, a sweep: FP16 307 -> 299 us, BF16 320 -> 311) and not in FP32 (577 and 578; L = 256,
+// 4 systems: 1044 -> 1115), which keeps the plain move; the sweep that loads into registers
+// loses (512 samples of L = 8 to 24 in binary32: 2357 -> 2392 us a
 // step), since its loads are not moved over the branches.
 __device__ __forceinline__ void or_move2_branch(float2& sx, float2& sy, float2& sz, float2 hx,
                                                 float2 hy, float2 hz) {

@@ -1,24 +1,22 @@
 // Staged over-relaxation half-sweeps (Sec. 3.1, Eq. 3): the block body that stages its
 // data through shared memory instead of loading it into registers.
 //
-// A block of the sweep block table updates 256 consecutive
-// storage sites of one parity: R = 256 / (L/2) whole rows y0 .. y0+R-1 of one
-// plane z (L a power of 2, L >= 32).  Its sites read the opposite parity in
-// rows y0-1 .. y0+R of plane z (the +-x and +-y neighbours) and in rows
-// y0 .. y0+R-1 of planes z-1 and z+1.  Those rows, and the block's own, are
-// contiguous runs of the parity-split layout, so per component plane and chunk
-// group they reach shared memory as six (five without the own rows) cp.async.bulk
-// copies (the rows y0-1 and y0+R apart, as they wrap in y).  The block walks its chunk groups through a
-// two-stage ring: while it computes chunk group g, the copies of g+1 are in
-// flight.  Each stage has a full mbarrier carrying the copies' bytes and an empty
-// one that its warps arrive at once they have read it.  The copies of the stage's
-// next chunk group are issued by one warp, another in each iteration, at the end of
-// its own update, when the others have mostly read the stage: no warp waits there
-// for long, and none issues all of them.  The update is the per-half-sweep
-// kernel's, in the same operations and order, so the results are bit for bit
-// the same.  Every wait is bounded: one that runs out sets the error word, and
-// the block stops computing but keeps waiting (bounded) for the copies it
-// issued before it exits.
+// A block of the sweep block table updates 256 consecutive storage sites of one parity:
+// R = 256 / (L/2) whole rows y0 .. y0+R-1 of one plane z (L a power of 2, L >= 32).  Its
+// sites read the opposite parity in rows y0-1 .. y0+R of plane z (the +-x and +-y
+// neighbours) and in rows y0 .. y0+R-1 of planes z-1 and z+1.  Those rows, and the block's
+// own, are contiguous runs of the parity-split layout, so per component plane and chunk
+// group they reach shared memory as six (five without the own rows) cp.async.bulk copies
+// (the rows y0-1 and y0+R apart, as they wrap in y).  The block walks its chunk groups
+// through a two-stage ring: while it computes chunk group g, the copies of g+1 are in
+// flight.  Each stage has a full mbarrier carrying the copies' bytes and an empty one that
+// its warps arrive at once they have read it.  The copies of the stage's next chunk group
+// are issued by one warp, another in each iteration, at the end of its own update, when the
+// others have mostly read the stage: no warp waits there for long, and none issues all of
+// them.  The update is the per-half-sweep kernel's, in the same operations and order, so the
+// results are bit for bit the same.  Every wait is bounded: one that runs out sets the error
+// word, and the block stops computing but keeps waiting (bounded) for the copies it issued
+// before it exits.
 //
 // What bounds it: at L = 128 the half-sweep's one pass over each parity in DRAM; with the
 // spins in L2 the wait for a stage's copies.  Against the kernel that loads into registers,

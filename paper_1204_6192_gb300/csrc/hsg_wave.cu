@@ -1,25 +1,25 @@
 // The wave launch: both half-sweeps of an over-relaxation sweep (Sec. 3.1, Eq. 3) at once.
 //
-// One launch has one block per (block table entry, parity): the
-// blocks of the two per-half-sweep launches.  A block takes a ticket on entry
-// (an atomic counter) and does the work the host-built order assigns to it.
-// The order walks the even blocks in table order (z-major within a chunk
-// group) and inserts each odd block `lag` even blocks after the last even block
-// it depends on.  An odd block of planes [z0, z1] reads the even sites of
-// planes z0-1 .. z1+1 (new values) and overwrites odd sites that the even
-// blocks of those planes read (old values), so before its update it waits until
-// every even block of those planes has signalled completion.  Those blocks hold
-// earlier tickets, so they are already running and never wait themselves: no
-// wait can deadlock, whatever the number of resident blocks.  Every even site
-// sees only old odd spins and every odd site only new even spins, so the
-// result is that of the even half-sweep followed by the odd one, bit for bit.
-// Staged odd blocks read the even spins through bulk copies (L2, after a proxy
-// fence); unstaged odd blocks read them bypassing L1.  Between the even update
-// of a plane and the odd updates that read it lie about `lag` blocks of work,
-// so the opposite parity, which two separate launches read from DRAM a second
-// time, mostly comes from L2.  The last block to finish resets the ticket and
-// completion counters and advances the epoch the completion flags carry, so
-// each launch (and each replay of a captured graph) starts clean.
+// One launch has one block per (block table entry, parity): the blocks of the two
+// per-half-sweep launches.  A block takes a ticket on entry (an atomic counter) and does the
+// work the host-built order assigns to it.  The order walks the even blocks in table order
+// (z-major within a chunk group) and inserts each odd block `lag` even blocks after the last
+// even block it depends on.  An odd block of planes [z0, z1] reads the even sites of planes
+// z0-1 .. z1+1 (new values) and overwrites odd sites that the even blocks of those planes
+// read (old values), so before its update it waits until every even block of those planes
+// has signalled completion.  Those blocks hold earlier tickets, so they are already running
+// and never wait themselves: no wait can deadlock, whatever the number of resident blocks.
+// Every even site sees only old odd spins and every odd site only new even spins, so the
+// result is that of the even half-sweep followed by the odd one, bit for bit.  Staged odd
+// blocks (hsg_staged.cuh) read the even spins through bulk copies (L2, after a proxy fence);
+// unstaged odd blocks read them bypassing L1.  Between the even update of a plane and the
+// odd updates that read it lie about `lag` blocks of work, so the opposite parity, which two
+// separate launches read from DRAM a second time, mostly comes from L2.  The last block to
+// finish resets the ticket and completion counters and advances the epoch the completion
+// flags carry, so each launch (and each replay of a captured graph) starts clean.
+//
+// A sweep of 48 systems at L = 128, FP16: 337 us (two staged launches 299); FP32, 24 systems
+// 342; L = 256, 4 systems 826 and 1511 (two launches 599 and 1044).
 #include "hsg_staged.cuh"
 
 namespace hsg {
