@@ -32,6 +32,7 @@ def test_error_of_a_refused_call_does_not_reach_the_next_context(call):
         getattr(ctx, call)()
     graph = ctypes.c_void_p()
     rt.cudaStreamEndCapture(stream.cuda_stream, ctypes.byref(graph))
+    rt.cudaGetLastError()       # the capture's failure, in this runtime (torch's)
     assert err.value.status in (2, 3)      # (the allocation or the wait that is refused)
     ctx.close()
     out = []
