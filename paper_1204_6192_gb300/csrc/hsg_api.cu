@@ -1057,17 +1057,16 @@ bool resident_possible(const hsg_ctx* c) {
          c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 && c->opt.step_branches == 0;
 }
 
-// The two-pass schedule as an explicit choice, which no timing stands behind: resident
-// where that wins or ties for every storage format.  Up to L = 8 at any number of systems;
-// above, with one block an SM (L = 10 and 12), up to three rounds of blocks, i.e. while
-// launches and latency count (L = 10, FP16, us a step, half-sweeps and resident: 38 and 22
-// with 64 blocks, 51 and 35 with 256, 87 and 99 with 1024, 487 and 700 with 8192; L = 12,
-// FP16 57 and 49, 141 and 145, 826 and 1051; FP32 64 and 55, 172 and 168, 1161 and 1230;
-// L = 8, FP16 40 and 20, 57 and 41, 228 and 229).
-hsg_status resident_untimed(hsg_ctx* c, bool* use) {
+// Few systems for the resident sweeps' blocks (a pair of systems each): up to three rounds
+// at one block an SM (L = 10 and 12), i.e. while launches and latency count and the resident
+// sweeps win for every storage format (L = 10, FP16, us a step, half-sweeps and resident:
+// 38 and 22 with 64 blocks, 51 and 35 with 256, 87 and 99 with 1024, 487 and 700 with 8192;
+// L = 12, FP16 57 and 49, 141 and 145, 826 and 1051; FP32 64 and 55, 172 and 168, 1161 and
+// 1230).  Up to L = 8 they win or tie at any number (FP16 40 and 20, 57 and 41, 228 and 229).
+hsg_status resident_few(hsg_ctx* c, bool* few) {
   int n_sm = 0;
   HSG_CUDA(c, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, c->device));
-  *use = resident_possible(c) && (c->Lmax <= 8 || (long long)c->ns * (c->Wp / 2) <= 3ll * n_sm);
+  *few = (long long)c->ns * (c->Wp / 2) <= 3ll * n_sm;
   return HSG_OK;
 }
 
@@ -1203,6 +1202,8 @@ hsg_status autotune(hsg_ctx* c) {
     }
     return HSG_OK;
   };
+  bool few = false;
+  HSG_TRY(resident_few(c, &few));
   const bool two_branches = c->opt.step_branches == 2 && sk != HSG_SWEEP_FUSED && sk != HSG_SWEEP_WAVE;
   for (long long pb : budgets) {
     if (two_branches) break;   // asked for
@@ -1224,12 +1225,14 @@ hsg_status autotune(hsg_ctx* c) {
   // L2 cache together (512 samples of L = 8 to 24: 2631 us a step with one pass of
   // half the cache in flight, 2694 with two of that size, 2362 with two of a quarter;
   // L = 64 in FP16: 404, 388 and 347; three and four branches no faster; also where the
-  // resident sweeps lead so far: 256 samples of L = 12, 32 systems, FP32 580, 467).  The chunks
+  // resident sweeps lead so far: 256 samples of L = 12, 32 systems, FP32 580, 467; not with
+  // few systems, where they cannot win, and a graph launch takes 0.7 us longer in a process
+  // that has run one of two branches: L = 8, 16 systems 17.8, 18.4).  The chunks
   // per thread are tried anew: smaller passes want fewer.
   if (two_branches ||
       (c->opt.step_branches == 0 && c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 &&
        bestc.variant == HSG_VARIANT_TWO_PASS &&
-       (bestc.sweep == HSG_SWEEP_HALF || bestc.sweep == HSG_SWEEP_RESIDENT ||
+       (bestc.sweep == HSG_SWEEP_HALF || (bestc.sweep == HSG_SWEEP_RESIDENT && !few) ||
         (bestc.sweep == HSG_SWEEP_STAGED && sk == HSG_SWEEP_AUTO)))) {
     if (c->opt.chunks_per_thread == 0)
       for (int g : {bestc.gpt, (bestc.gpt + 1) / 2, 2 * bestc.gpt})
@@ -1547,9 +1550,11 @@ hsg_status create_impl(hsg_ctx** out, int n_samples, const int* L, const double*
     }
     int sweep = opt.sweep_kernel == HSG_SWEEP_AUTO ? HSG_SWEEP_HALF : opt.sweep_kernel;
     const int chains = opt.step_branches == 2 ? 2 : 1;
-    bool resident = false;
-    hsg_status st2 = opt.variant == HSG_VARIANT_TWO_PASS ? resident_untimed(c, &resident) : HSG_OK;
-    if (resident) sweep = HSG_SWEEP_RESIDENT;
+    bool few = false;
+    hsg_status st2 = resident_few(c, &few);
+    // the two-pass schedule as an explicit choice, which no timing stands behind
+    if (opt.variant == HSG_VARIANT_TWO_PASS && resident_possible(c) && (c->Lmax <= 8 || few))
+      sweep = HSG_SWEEP_RESIDENT;
     if (st2 == HSG_OK)
       st2 = configure_schedule(c, want, c->GPT, opt.pass_bytes == 0 && chains == 2 ? half_footprint(c) : opt.pass_bytes,
                                sweep, opt.wave_lag, chains);
