@@ -1226,9 +1226,9 @@ hsg_status autotune(hsg_ctx* c) {
   // half the cache in flight, 2694 with two of that size, 2362 with two of a quarter;
   // L = 64 in FP16: 404, 388 and 347; three and four branches no faster; also where the
   // resident sweeps lead so far: 256 samples of L = 12, 32 systems, FP32 580, 467; not with
-  // few systems, where they cannot win, and a graph launch takes 0.7 us longer in a process
-  // that has run one of two branches: L = 8, 16 systems 17.8, 18.4).  The chunks
-  // per thread are tried anew: smaller passes want fewer.
+  // few systems, where they cannot win, and where a step and a copy of the spins take 0.6 us
+  // longer in a process that has run a graph of two branches: L = 8, 16 systems 16.8, 17.4).
+  // The chunks per thread are tried anew: smaller passes want fewer.
   if (two_branches ||
       (c->opt.step_branches == 0 && c->opt.pass_bytes == 0 && c->opt.chunks_per_thread == 0 &&
        bestc.variant == HSG_VARIANT_TWO_PASS &&

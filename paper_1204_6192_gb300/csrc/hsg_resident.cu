@@ -220,11 +220,11 @@ __global__ void __launch_bounds__(MAXT) k_resident(const ResidentParams p) {
   if (warp == 0) {
     // rows of SWEEP_BS half-sites (at most 4: one split, and a row lane for each): their
     // even sites' partial and their odd sites', lane = 4 row + 2 parity + system
-    const int w0 = (lane >> 2) * (SWEEP_BS / 32), w1 = min((int)(blockDim.x >> 5), w0 + SWEEP_BS / 32);
+    const int nw = blockDim.x >> 5, w0 = (lane >> 2) * (SWEEP_BS / 32), w1 = min(nw, w0 + SWEEP_BS / 32);
     double part = 0.0, t = 0.0;
     for (int w = w0; w < w1; ++w) part += (double)red[(lane >> 1) & 1][w][lane & 1];
     part += __shfl_xor_sync(0xffffffffu, part, 2);
-    for (int row = 0; row < 4; ++row) t += __shfl_sync(0xffffffffu, part, 4 * row + (lane & 1));
+    for (int row = 0; row * (SWEEP_BS / 32) < nw; ++row) t += __shfl_sync(0xffffffffu, part, 4 * row + (lane & 1));
     if (lane < 2) p.E[(long long)s * p.Wp + pr * 2 + lane] = t;
   }
 }
